@@ -1,5 +1,6 @@
 // C-ABI of libfourphonon: context, validation, device memory, launches (see include/fourphonon.h).
 #include <algorithm>
+#include <array>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -100,6 +101,52 @@ int neg_index(const fp_ctx* c, int q) {
   return grid_index(c, m);
 }
 
+// Whether the quartet list obeys the transposition symmetry of Sec. 2.3 (Eq. TS) in the legs that the pair kernel
+// exchanges: (i, a) <-> (j, b), re-based to the new home cell, and (k, c) <-> (l, d).  Quartets listed more than once
+// add up.  The tolerance, 1e-13 of the largest entry, covers the rounding of symmetrised input and keeps the rates
+// within a few 1e-13 of those of the list as given.
+bool leg_symmetric(int n, const fp_fc4* fc4) {
+  using Key = std::array<int, 13>;
+  std::map<Key, std::array<double, 81>> sum;
+  double big = 0.0;
+  for (int b = 0; b < n; ++b) {
+    const fp_fc4& f = fc4[b];
+    const Key key = {f.i, f.j, f.k, f.l, f.Rj[0], f.Rj[1], f.Rj[2], f.Rk[0], f.Rk[1], f.Rk[2], f.Rl[0], f.Rl[1], f.Rl[2]};
+    auto it = sum.find(key);
+    if (it == sum.end()) {
+      it = sum.emplace(key, std::array<double, 81>()).first;
+      it->second.fill(0.0);
+    }
+    for (int x = 0; x < 81; ++x) {
+      it->second[x] += f.fc[x];
+      big = std::max(big, std::fabs(f.fc[x]));
+    }
+  }
+  const double tol = 1e-13 * big;
+  for (const auto& kv : sum) {
+    const Key& q = kv.first;
+    Key ij = {q[1], q[0], q[2], q[3], 0, 0, 0, 0, 0, 0, 0, 0, 0}, kl = {q[0], q[1], q[3], q[2], q[4], q[5], q[6], 0, 0, 0, 0, 0, 0};
+    for (int d = 0; d < 3; ++d) {
+      ij[4 + d] = -q[4 + d];
+      ij[7 + d] = q[7 + d] - q[4 + d];
+      ij[10 + d] = q[10 + d] - q[4 + d];
+      kl[7 + d] = q[10 + d];
+      kl[10 + d] = q[7 + d];
+    }
+    const auto pij = sum.find(ij), pkl = sum.find(kl);
+    for (int al = 0; al < 3; ++al)
+      for (int be = 0; be < 3; ++be)
+        for (int ga = 0; ga < 3; ++ga)
+          for (int th = 0; th < 3; ++th) {
+            const double v = kv.second[((al * 3 + be) * 3 + ga) * 3 + th];
+            const double vij = pij == sum.end() ? 0.0 : pij->second[((be * 3 + al) * 3 + ga) * 3 + th];
+            const double vkl = pkl == sum.end() ? 0.0 : pkl->second[((al * 3 + be) * 3 + th) * 3 + ga];
+            if (!(std::fabs(v - vij) <= tol) || !(std::fabs(v - vkl) <= tol)) return false;
+          }
+  }
+  return true;
+}
+
 }  // namespace
 
 namespace fp {
@@ -138,6 +185,9 @@ void fp_free(fp_ctx* c) {
   dfree(c->d_grp_q);
   dfree(c->d_kl_start);
   dfree(c->d_kl_grp);
+  dfree(c->d_pk_start);
+  dfree(c->d_pk_grp);
+  dfree(c->d_pk_zero);
   dfree(c->d_tw);
   dfree(c->d_omega);
   dfree(c->d_evec);
@@ -304,6 +354,20 @@ int fp_init(fp_ctx** out, const double lattice[9], int natoms, const double* fra
     std::vector<int> fill(kl_start.begin(), kl_start.end() - 1);
     for (int gi = 0; gi < c->G; ++gi) kl_grp[fill[gmeta[5 * gi] * natoms + gmeta[5 * gi + 1]]++] = gi;
   }
+  // the same groups for the pair kernel: by atom k and then l, without those of D = 0 (at most one per (k, l))
+  std::vector<int> pk_start(natoms + 1, 0), pk_grp, pk_zero(na2, -1);
+  for (int k = 0; k < natoms; ++k) {
+    for (int l = 0; l < natoms; ++l)
+      for (int i = kl_start[k * natoms + l]; i < kl_start[k * natoms + l + 1]; ++i) {
+        const int* gm = &gmeta[5 * (size_t)kl_grp[i]];
+        if (gm[2] == 0 && gm[3] == 0 && gm[4] == 0)
+          pk_zero[k * natoms + l] = kl_grp[i];
+        else
+          pk_grp.push_back(kl_grp[i] | l << 24);
+      }
+    pk_start[k + 1] = (int)pk_grp.size();
+  }
+  c->leg_symmetric = c->G < (1 << 24) && leg_symmetric(n_fc4, fc4);
   INIT_CUDA(dalloc(&c->d_qmeta, qmeta.size()));
   INIT_CUDA(dalloc(&c->d_qfc, qfc.size()));
   INIT_CUDA(dalloc(&c->d_gmeta, gmeta.size()));
@@ -312,6 +376,12 @@ int fp_init(fp_ctx** out, const double lattice[9], int natoms, const double* fra
   INIT_CUDA(dalloc(&c->d_kl_start, kl_start.size()));
   INIT_CUDA(dalloc(&c->d_kl_grp, kl_grp.size()));
   INIT_CUDA(dalloc(&d_atoms4, atoms4.size()));
+  INIT_CUDA(dalloc(&c->d_pk_start, pk_start.size()));
+  INIT_CUDA(dalloc(&c->d_pk_grp, pk_grp.size()));
+  INIT_CUDA(dalloc(&c->d_pk_zero, pk_zero.size()));
+  INIT_CUDA(cudaMemcpyAsync(c->d_pk_start, pk_start.data(), pk_start.size() * sizeof(int), cudaMemcpyHostToDevice, s));
+  INIT_CUDA(cudaMemcpyAsync(c->d_pk_grp, pk_grp.data(), pk_grp.size() * sizeof(int), cudaMemcpyHostToDevice, s));
+  INIT_CUDA(cudaMemcpyAsync(c->d_pk_zero, pk_zero.data(), pk_zero.size() * sizeof(int), cudaMemcpyHostToDevice, s));
   INIT_CUDA(cudaMemcpyAsync(c->d_qmeta, qmeta.data(), qmeta.size() * sizeof(int), cudaMemcpyHostToDevice, s));
   INIT_CUDA(cudaMemcpyAsync(c->d_qfc, qfc.data(), qfc.size() * sizeof(double), cudaMemcpyHostToDevice, s));
   INIT_CUDA(cudaMemcpyAsync(c->d_gmeta, gmeta.data(), gmeta.size() * sizeof(int), cudaMemcpyHostToDevice, s));
@@ -648,18 +718,19 @@ int phase_pass(fp_ctx* c, const fp_rates_opts& o, int nT, const double* T, doubl
   int rc = fp::make_selection(c, o, stride == 1, &sel, err);  // a q' stride is not symmetric under q -> -q
   if (rc) return rc;
   fp::Plan p;
-  rc = fp::plan_rates(c, o, nT, sel, 0, &p, err);
+  rc = fp::plan_rates(c, o, nT, sel, 0, &p, err, stride == 1);
   if (rc) return rc;
   if (stride > 1) {  // a q' tile of one stride: every item owns exactly one sampled q'
     p.t1 = stride;
     p.ntile = (c->N + stride - 1) / stride;
     p.n_items = (long long)p.ntile * p.nq_sel * p.nchunk;
+    p.values = p.n_items * p.J;
     if (p.ctas > p.n_items) p.ctas = (int)std::max<long long>(1, p.n_items);
   }
   size_t sz[fp::kScratchParts], total = 0;
   fp::scratch_sizes(c, p, nT, sz);
   for (size_t x : sz) total += x;
-  const size_t cnt_bytes = (size_t)std::max<long long>(1, p.n_items) * p.J * sizeof(unsigned long long);
+  const size_t cnt_bytes = (size_t)std::max<long long>(1, p.values) * sizeof(unsigned long long);
   unsigned char* b = nullptr;
   cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&b), total + cnt_bytes);
   if (e != cudaSuccess) {

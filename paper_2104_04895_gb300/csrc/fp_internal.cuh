@@ -65,8 +65,9 @@ struct RatesArgs {
   double rec[9];
   double* partial;           // [n_items][J][nT]
   unsigned long long* counter;
-  unsigned long long* counts; // [6]: accepted ++, +-, -- (weighted by mult), vertex entries W formed, accepted
-                              // terms evaluated, tensor-core completion waits that ran out of polls
+  unsigned long long* counts; // [8]: accepted ++, +-, -- (weighted by mult), vertex entries W formed, accepted
+                              // terms evaluated, tensor-core completion waits that ran out of polls, (pair kernel)
+                              // (q, q', q'') iterations and (q, q') pairs evaluated
   int unit_vertex;           // 1: |W|^2 = 1 (weighted phase space), q' on a stride, ordered (q', q'') pairs
   int k1_stride;             // q' stride of the unit-vertex mode
   unsigned cand_mask;        // candidates summed (bit c = ordering * 3 + process), from process_mask
@@ -75,6 +76,12 @@ struct RatesArgs {
   unsigned long long* item_counts;  // [n_items][J] accepted terms per (item, j0), or null (not counted)
   double* mode_counts;       // [N*nb] reduction output: accepted terms per selected mode x count_scale, or null
   double count_scale;
+  // pair kernel (fp_pair_kernel.cuh)
+  int mirror;                // 1: `partial` has a slot per (evaluated point, q') and a pair fills the slots of both its
+                             // members; 0: a slot per work item, every q' evaluated
+  const int* pk_start;       // [natoms + 1] groups with D != 0 by atom k, in l order
+  const int* pk_grp;         // their group index | l << 24
+  const int* pk_zero;        // [natoms^2] the group of (k, l) with D = 0 (phase 1), or -1
 };
 
 // Which q-points a rates call evaluates, and for which modes.  Time reversal (e^{-lambda} = conj e^{lambda},
@@ -98,12 +105,15 @@ struct Plan {
   int J, threads, t1, nchunk, ntile, nq_sel, ctas;
   long long n_items;
   size_t smem;
+  bool pair = false, mirror = false;  // the pair kernel; with a slot per (evaluated point, q')
+  long long values = 0;               // partial sums per temperature
 };
 
 // Device working memory of one rates call (owned by the caller of run_rates), in the order of scratch_sizes.
 constexpr int kScratchParts = 16;
 constexpr int kScratchPartial = 7;  // index of the per-item partial sums
-constexpr int kCounters = 8;        // queue, accepted ++, +-, --, vertex entries, terms evaluated, wait timeouts, spare
+constexpr int kCounters = 10;       // queue, accepted ++, +-, --, vertex entries, terms evaluated, wait timeouts,
+                                    // iterations, pairs, spare
 struct Scratch {
   unsigned long long* counters;  // [kCounters]
   double* T;                     // [kMaxT]
@@ -112,7 +122,7 @@ struct Scratch {
   int* qlist;                    // [N]
   int* qpos;                     // [N]
   double* wt;                    // [nT][N*nb][3]
-  double* partial;               // [n_items][J][nT]
+  double* partial;               // [Plan::values][nT]
   float* omh;                    // [N*nb]
   float* oml;
   float* velh;                   // [N*nb*3]
@@ -149,6 +159,10 @@ struct fp_ctx {
   int* d_kl_start = nullptr;
   int* d_kl_grp = nullptr;
   double2* d_tw = nullptr;
+  int* d_pk_start = nullptr;  // groups as the pair kernel walks them (RatesArgs)
+  int* d_pk_grp = nullptr;
+  int* d_pk_zero = nullptr;
+  bool leg_symmetric = false;  // the quartet list obeys the transposition symmetry (Eq. TS)
   int* d_bzm = nullptr;  // [N][3] Brillouin-zone shifts (bz_shifts)
   // third-order force constants (fp_set_fc3), grouped by atom triple
   bool have_fc3 = false;
@@ -194,9 +208,10 @@ cudaError_t launch_weights(fp_ctx* c, int nT, const double* d_T, double* d_wt, c
 // unless o.no_time_reversal or o.nu_select is set or fold_allowed is false.  FP_EINVAL on a bad q range.
 int make_selection(const fp_ctx* c, const fp_rates_opts& o, bool fold_allowed, Selection* s, std::string* err);
 // Validate options and choose tiles; `partial_budget` (bytes, 0 = unlimited) enlarges the q'-tile until the
-// per-item partial sums fit.  Returns FP_OK or an FP_E* code with a message in *err.
+// per-item partial sums fit; `mirror` allows the pair kernel's slot per (evaluated point, q') where it fits.
+// Returns FP_OK or an FP_E* code with a message in *err.
 int plan_rates(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, size_t partial_budget, Plan* p,
-               std::string* err);
+               std::string* err, bool mirror = true);
 // Byte sizes of the Scratch buffers of a plan, in the order of the Scratch fields (each rounded up to 256).
 void scratch_sizes(const fp_ctx* c, const Plan& p, int nT, size_t sizes[kScratchParts]);
 // Scratch pointers laid out from `base` with the sizes of scratch_sizes.

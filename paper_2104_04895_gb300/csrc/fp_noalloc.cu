@@ -104,7 +104,7 @@ extern "C" int fp_rates4_noalloc(fp_ctx* c, int nT, const double* T, double sb, 
   fp::Plan p0;
   fp_rates_opts o_probe = o;
   if (o_probe.k1_tile <= 0) o_probe.k1_tile = c->N;  // smallest partials, for the fixed-size part
-  rc = fp::plan_rates(c, o_probe, nT, sel, 0, &p0, &err);
+  rc = fp::plan_rates(c, o_probe, nT, sel, 0, &p0, &err, false);
   if (rc) return nfail(c, rc, "fp_rates4_noalloc: " + err);
   size_t sz[fp::kScratchParts], fixed = 0;
   fp::scratch_sizes(c, p0, nT, sz);

@@ -1,0 +1,16 @@
+// Double-float instantiations of the pair kernel (FP_PREC_DOUBLE_FLOAT) for 1, 2 and 4 atoms per cell.
+#include "fp_pair_kernel.cuh"
+
+namespace fp {
+const void* pair_kernel_df(int nb, int maxt) {
+  switch (nb * 100 + maxt) {
+    case 301: return reinterpret_cast<const void*>(pair_kernel<3, 1, true>);
+    case 308: return reinterpret_cast<const void*>(pair_kernel<3, kMaxT, true>);
+    case 601: return reinterpret_cast<const void*>(pair_kernel<6, 1, true>);
+    case 608: return reinterpret_cast<const void*>(pair_kernel<6, kMaxT, true>);
+    case 1201: return reinterpret_cast<const void*>(pair_kernel<12, 1, true>);
+    case 1208: return reinterpret_cast<const void*>(pair_kernel<12, kMaxT, true>);
+    default: return nullptr;
+  }
+}
+}  // namespace fp

@@ -1,0 +1,16 @@
+// FP64 instantiations of the pair kernel for 1, 2 and 4 atoms per cell.
+#include "fp_pair_kernel.cuh"
+
+namespace fp {
+const void* pair_kernel_f64(int nb, int maxt) {
+  switch (nb * 100 + maxt) {
+    case 301: return reinterpret_cast<const void*>(pair_kernel<3, 1, false>);
+    case 308: return reinterpret_cast<const void*>(pair_kernel<3, kMaxT, false>);
+    case 601: return reinterpret_cast<const void*>(pair_kernel<6, 1, false>);
+    case 608: return reinterpret_cast<const void*>(pair_kernel<6, kMaxT, false>);
+    case 1201: return reinterpret_cast<const void*>(pair_kernel<12, 1, false>);
+    case 1208: return reinterpret_cast<const void*>(pair_kernel<12, kMaxT, false>);
+    default: return nullptr;
+  }
+}
+}  // namespace fp

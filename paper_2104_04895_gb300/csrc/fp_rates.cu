@@ -1,10 +1,12 @@
 // Host side of the rate path: FP32 prep kernel, fixed-order reduction, tile plan and the launch routine
 // shared by fp_rates4, fp_rates4_device and fp_rates4_noalloc.  The rate kernel itself is in
 // fp_rates_kernel.cuh.
-#include "fp_rates_kernel.cuh"
+#include "fp_pair_kernel.cuh"
 
 namespace fp {
-// kernel pointers of the two precision instantiations (fp_rates_f64.cu, fp_rates_f32.cu)
+// kernel pointers of the instantiations (fp_pair_*.cu, fp_rates_*.cu)
+const void* pair_kernel_f64(int nb, int maxt);
+const void* pair_kernel_df(int nb, int maxt);
 const void* rates_kernel_f64(int nb, int maxt);
 const void* rates_kernel_f32(int nb, int maxt);
 const void* rates_kernel_f32_tc(int nb, int maxt);
@@ -86,6 +88,45 @@ __global__ void reduce_kernel(RatesArgs a, double pref, double* rates) {
   }
 }
 
+// The same for the pair kernel's slots: one warp per output, the slots of q (its pair with every q') summed by lane
+// and then across lanes, in a fixed order.  A slot that a chunked mirrored pair wrote holds one value per chunk.
+__global__ void pair_reduce_kernel(RatesArgs a, double pref, double* rates) {
+  const long long n = (long long)a.nT * a.q_out_n * a.nb;
+  const long long o = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (o >= n) return;
+  const int j = (int)(o % a.nb);
+  const int q = a.q_out_begin + (int)((o / a.nb) % a.q_out_n);
+  const int t = (int)(o / ((long long)a.nb * a.q_out_n));
+  if (!a.sel[(size_t)q * a.nb + j]) return;
+  const int qi = a.qpos[q];
+  const int qe = a.qlist[qi];
+  const int chunk = j / a.J, jj = j % a.J;
+  double s = 0.0;
+  unsigned long long cnt = 0;
+  for (int b = lane; b < a.N; b += 32) {
+    const size_t base = ((size_t)qi * a.N + b) * a.nchunk;
+    if (a.nchunk == 1 || pair_role(a, qi, qe, b).run) {
+      const size_t v = (base + chunk) * a.nb + jj;
+      s += a.partial[v * a.nT + t];
+      if (a.mode_counts && t == 0) cnt += a.item_counts[v];
+    } else {
+      for (int c = 0; c < a.nchunk; ++c) {
+        const size_t v = (base + c) * a.nb + j;
+        s += a.partial[v * a.nT + t];
+        if (a.mode_counts && t == 0) cnt += a.item_counts[v];
+      }
+    }
+  }
+  for (int off = 16; off > 0; off >>= 1) {
+    s += __shfl_down_sync(0xffffffffu, s, off);
+    cnt += __shfl_down_sync(0xffffffffu, cnt, off);
+  }
+  if (lane) return;
+  rates[((size_t)t * a.N + q) * a.nb + j] = s * pref;
+  if (a.mode_counts && t == 0) a.mode_counts[(size_t)q * a.nb + j] = (double)cnt * a.count_scale;
+}
+
 // p[i] = v (the unit weight table of the unweighted phase space)
 __global__ void fill_kernel(double* p, long long n, double v) {
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
@@ -93,22 +134,24 @@ __global__ void fill_kernel(double* p, long long n, double v) {
 }
 
 // kernel for (precision, nb, number of temperatures, tensor cores): one accumulator per temperature, 1 or up to 8
-const void* rates_kernel_ptr(int precision, int nb, int nT, bool tc) {
+const void* rates_kernel_ptr(int precision, int nb, int nT, bool tc, bool pair) {
   const int maxt = nT == 1 ? 1 : kMaxT;
+  if (pair) return precision == FP_PREC_DOUBLE_FLOAT ? pair_kernel_df(nb, maxt) : pair_kernel_f64(nb, maxt);
   if (tc) return precision == FP_PREC_MIXED ? rates_kernel_f32_tc(nb, maxt) : nullptr;
   if (precision == FP_PREC_DOUBLE_FLOAT) return rates_kernel_df(nb, maxt);
   return precision == FP_PREC_FP64 ? rates_kernel_f64(nb, maxt) : rates_kernel_f32(nb, maxt);
 }
 
-size_t smem_bytes(int precision, int nb, int J, int G, int nquart, int nT, int threads, bool tc) {
+size_t smem_bytes(int precision, int nb, int J, int G, int nquart, int nT, int threads, bool tc, bool pair) {
+  if (pair) return make_pair_carve(nb, J, G, nquart, nT, threads).bytes();
   const bool f32 = precision == FP_PREC_MIXED;  // the double-float path has the FP64 path's shared memory
   Carve c = make_carve(nb, J, G, nquart, nT, threads, f32);
   const size_t b = c.bytes(f32 ? sizeof(Cx<float>) : sizeof(Cx<double>));
   return tc ? align128(b) + kTcBytes : b;
 }
 
-int max_ctas_per_sm(int precision, int nb, int nT, int threads, size_t smem, bool tc) {
-  const void* k = rates_kernel_ptr(precision, nb, nT, tc);
+int max_ctas_per_sm(int precision, int nb, int nT, int threads, size_t smem, bool tc, bool pair) {
+  const void* k = rates_kernel_ptr(precision, nb, nT, tc, pair);
   if (!k) return 0;
   if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
   int n = 0;
@@ -187,14 +230,17 @@ int make_selection(const fp_ctx* c, const fp_rates_opts& o, bool fold_allowed, S
 }
 
 int plan_rates(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, size_t partial_budget, Plan* p,
-               std::string* err) {
+               std::string* err, bool mirror) {
   const int N = c->N, nb = c->nb;
   const bool tc = o.tensor_cores != 0;
   if (tc && (o.precision != FP_PREC_MIXED || nb != 6)) {
     *err = "tensor_cores needs the mixed precision and 6 branches";
     return FP_EINVAL;
   }
-  if (!rates_kernel_ptr(o.precision, nb, nT, tc)) {
+  // The pair kernel identifies vertices whose legs are permuted, so it needs Phi4 to have that symmetry.  It is not
+  // built for the mixed path.
+  const bool pair = c->leg_symmetric && o.precision != FP_PREC_MIXED;
+  if (!rates_kernel_ptr(o.precision, nb, nT, tc, pair)) {
     *err = "unsupported number of branches";
     return FP_EINVAL;
   }
@@ -209,10 +255,13 @@ int plan_rates(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, size_t
     }
   }
   if (J <= 0) {
-    // largest divisor of nb whose rows fit a block and whose tile leaves room for two blocks per SM
+    // largest divisor of nb whose rows fit a block and whose tile leaves room for two blocks per SM (the pair kernel
+    // with twelve branches: one)
+    const int most = pair ? pair_threads_for(nb) : max_threads_for(nb);
+    const size_t room = pair ? (pair_blocks_for(nb) == 1 ? 227 : 112) * 1024 : 110 * 1024;
     J = nb;
-    while (J > 1 && (J * nb * nb > max_threads_for(nb) ||
-                     smem_bytes(o.precision, nb, J, c->G, c->nquart, nT, max_threads_for(nb), tc) > 110 * 1024)) {
+    while (J > 1 && (J * nb * nb > most ||
+                     smem_bytes(o.precision, nb, J, c->G, c->nquart, nT, pair ? (J * nb * nb + 31) / 32 * 32 : most, tc, pair) > room)) {
       int nj = J - 1;
       while (nj > 1 && nb % nj) --nj;
       J = nj;
@@ -225,7 +274,8 @@ int plan_rates(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, size_t
   const int rows = J * nb * nb;
   int threads = o.threads > 0 ? o.threads : th_tuned > 0 ? th_tuned : ((rows + 31) / 32) * 32;
   if (threads < 32) threads = 32;
-  if (threads % 32 || threads < rows || threads > max_threads_for(nb)) {
+  const int max_threads = o.block_j0 > 0 || o.threads > 0 || !pair ? max_threads_for(nb) : pair_threads_for(nb);
+  if (threads % 32 || threads < rows || threads > max_threads) {
     *err = "threads must be a multiple of 32, >= block_j0*nb^2 and <= " + std::to_string(max_threads_for(nb));
     return FP_EINVAL;
   }
@@ -235,7 +285,18 @@ int plan_rates(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, size_t
   auto part_bytes = [&](int tile) {
     return (size_t)((N + tile - 1) / tile) * nq_sel * nchunk * J * nT * sizeof(double);
   };
-  if (o.k1_tile <= 0 && partial_budget)
+  // a slot per (evaluated point, q') halves the pairs to evaluate; without the memory for it, every q' is evaluated
+  // and a work item has one slot
+  mirror = mirror && pair;
+  const long long mirror_values = (long long)nq_sel * N * nchunk * nb;
+  const size_t mirror_bytes = (size_t)mirror_values * nT * sizeof(double);
+  if (mirror && partial_budget && mirror_bytes > partial_budget) mirror = false;
+  if (mirror && mirror_bytes > (size_t(256) << 20) && mirror_bytes > c->scratch_cap) {
+    size_t mem_free = 0, mem_total = 0;
+    mirror = cudaMemGetInfo(&mem_free, &mem_total) == cudaSuccess && mirror_bytes < mem_free / 2;
+  }
+  if (mirror && o.k1_tile <= 0 && t1_tuned <= 0) t1 = 1;
+  if (o.k1_tile <= 0 && partial_budget && !mirror)
     while (t1 < N && part_bytes(t1) > partial_budget) t1 = t1 < 8 ? t1 + 1 : t1 + t1 / 4;
   if (t1 > N) t1 = N;
   // the kernel counts an item's accepted terms in 32 bits: at most 6 per (q', q'', j''') of a row, times the
@@ -252,16 +313,16 @@ int plan_rates(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, size_t
     }
     t1 = (int)max_t1;
   }
-  if (partial_budget && part_bytes(t1) > partial_budget) {
+  if (partial_budget && !mirror && part_bytes(t1) > partial_budget) {
     *err = "per-item partial sums do not fit the scratch";
     return FP_EINVAL;
   }
-  const size_t smem = smem_bytes(o.precision, nb, J, c->G, c->nquart, nT, threads, tc);
+  const size_t smem = smem_bytes(o.precision, nb, J, c->G, c->nquart, nT, threads, tc, pair);
   if (smem > 227 * 1024) {
     *err = "tile does not fit in shared memory";
     return FP_EINVAL;
   }
-  const int per_sm = max_ctas_per_sm(o.precision, nb, nT, threads, smem, tc);
+  const int per_sm = max_ctas_per_sm(o.precision, nb, nT, threads, smem, tc, pair);
   if (per_sm < 1) {
     *err = "kernel tile cannot be resident on an SM";
     return FP_EINVAL;
@@ -279,6 +340,9 @@ int plan_rates(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, size_t
   p->nq_sel = nq_sel;
   p->n_items = (long long)p->ntile * nq_sel * nchunk;
   p->smem = smem;
+  p->pair = pair;
+  p->mirror = mirror;
+  p->values = mirror ? mirror_values : p->n_items * J;
   long long ctas = (long long)nsm * per_sm;
   if (ctas > p->n_items) ctas = p->n_items > 0 ? p->n_items : 1;
   p->ctas = (int)ctas;
@@ -301,7 +365,7 @@ void scratch_sizes(const fp_ctx* c, const Plan& p, int nT, size_t s[kScratchPart
   s[4] = up256((size_t)c->N * sizeof(int));               // qlist
   s[5] = up256((size_t)c->N * sizeof(int));               // qpos
   s[6] = up256(3 * nm * nT * sizeof(double));             // wt
-  s[kScratchPartial] = up256((size_t)p.n_items * p.J * nT * sizeof(double));
+  s[kScratchPartial] = up256((size_t)p.values * nT * sizeof(double));
   s[8] = up256(nm * sizeof(float));
   s[9] = up256(nm * sizeof(float));
   s[10] = up256(3 * nm * sizeof(float));
@@ -417,6 +481,10 @@ int run_rates(fp_ctx* c, const fp_rates_opts& o, const Selection& sel, const Pla
   a.partial = sc.partial;
   a.counter = sc.counters;
   a.counts = sc.counters + 1;
+  a.mirror = p.mirror ? 1 : 0;
+  a.pk_start = c->d_pk_start;
+  a.pk_grp = c->d_pk_grp;
+  a.pk_zero = c->d_pk_zero;
   a.unit_vertex = unit_stride > 0 ? 1 : 0;
   a.k1_stride = unit_stride > 0 ? unit_stride : 1;
   {
@@ -435,7 +503,7 @@ int run_rates(fp_ctx* c, const fp_rates_opts& o, const Selection& sel, const Pla
   const double pref = unit_stride > 0
                           ? (double)unit_stride / ((double)N * (double)N)
                           : kPi * kHbar * kHbar * conv * conv * conv * conv / (8.0 * (double)N * (double)N);
-  const void* k = rates_kernel_ptr(o.precision, nb, nT, o.tensor_cores != 0);
+  const void* k = rates_kernel_ptr(o.precision, nb, nT, o.tensor_cores != 0, p.pair);
   // the device part of a rate set: Bose weights, FP32 tables, cleared counters and output, the persistent
   // rate kernel and the reduction
   auto enqueue = [&]() -> cudaError_t {
@@ -460,7 +528,10 @@ int run_rates(fp_ctx* c, const fp_rates_opts& o, const Selection& sel, const Pla
       void* args[] = {&aa};
       if ((e = cudaLaunchKernel(k, dim3(p.ctas), dim3(p.threads), args, p.smem, s)) != cudaSuccess) return e;
       const long long n = (long long)nT * (sel.q_out_end - sel.q_out_begin) * nb;
-      reduce_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(a, pref, d_out);
+      if (p.mirror)
+        pair_reduce_kernel<<<(unsigned)((n + 7) / 8), 256, 0, s>>>(a, pref, d_out);
+      else
+        reduce_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(a, pref, d_out);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -544,7 +615,9 @@ void fill_stats(const fp_ctx* c, const fp_rates_opts& o, const Selection& sel, c
   const double pairs = 0.5 * (double)N * (double)(N + 1);
   const double per_pair = 8.0 * (9.0 * J * nb * c->G + J * (double)nb * nb * nb * nb);
   const double prolog = 8.0 * 9.0 * J * nb * 9.0 * c->nquart;
-  st->flops = (double)sel.active_chunks * (pairs * per_pair + (double)N * prolog) + 8.0 * nb * st->vertex_entries;
+  st->flops = p.pair ? (double)counts[7] * per_pair + (double)counts[8] * prolog
+                     : (double)sel.active_chunks * (pairs * per_pair + (double)N * prolog);
+  st->flops += 8.0 * nb * st->vertex_entries;
   float ms = 0.f;
   cudaEventElapsedTime(&ms, c->ev0, c->ev1);
   st->ms = ms;
@@ -566,12 +639,13 @@ int phase4_sampled(fp_ctx* c, int nT, const double* T, double sb, int stride, do
   int rc = make_selection(c, o, false, &sel, err);  // q' on a stride is not symmetric under q -> -q
   if (rc) return rc;
   Plan p;
-  rc = plan_rates(c, o, nT, sel, 0, &p, err);
+  rc = plan_rates(c, o, nT, sel, 0, &p, err, false);
   if (rc) return rc;
   // a q' tile of one stride: every item owns exactly one sampled q'
   p.t1 = stride;
   p.ntile = (c->N + stride - 1) / stride;
   p.n_items = (long long)p.ntile * p.nq_sel * p.nchunk;
+  p.values = p.n_items * p.J;
   if (p.ctas > p.n_items) p.ctas = (int)p.n_items;
   size_t sz[kScratchParts], total = 0;
   scratch_sizes(c, p, nT, sz);

@@ -434,6 +434,7 @@ int fp_modes(fp_ctx* c, double* omega, double* evec, double* vel) {
     return fail(c, FP_EUNSTABLE, "fp_modes: imaginary frequencies (omega^2 < -1e-8 max omega^2)");
   }
   c->have_modes = true;
+  c->unit_modes = true;
   return FP_OK;
 }
 
@@ -441,9 +442,16 @@ int fp_set_modes(fp_ctx* c, const double* omega, const double* evec, const doubl
   if (!c) return fail(nullptr, FP_EINVAL, "fp_set_modes: NULL context");
   if (!omega || !evec || !vel) return fail(c, FP_EINVAL, "fp_set_modes: NULL table");
   const int nb = c->nb;
+  bool unit = true;  // eigenvectors of norm 1 (a table may scale them; the sliced contraction is built for unit ones)
   for (int q = 0; q < c->N; ++q) {
     const int p = neg_index(c, q);
     for (int j = 0; j < nb; ++j) {
+      double norm2 = 0.0;
+      for (int k = 0; k < 2 * nb; ++k) {
+        const double x = evec[2 * ((size_t)q * nb + j) * nb + k];
+        norm2 += x * x;
+      }
+      unit = unit && std::fabs(norm2 - 1.0) <= 2e-5;
       double w = omega[q * nb + j];
       if (!(w >= 0.0) || !std::isfinite(w)) return fail(c, FP_EINVAL, "fp_set_modes: omega must be finite and >= 0");
       if (omega[p * nb + j] != w) return fail(c, FP_EINVAL, "fp_set_modes: omega(-q) != omega(q)");
@@ -467,6 +475,7 @@ int fp_set_modes(fp_ctx* c, const double* omega, const double* evec, const doubl
   FP_CUDA(c, cudaMemcpyAsync(c->d_vel, vel, nm * 3 * sizeof(double), cudaMemcpyHostToDevice, s));
   FP_CUDA(c, cudaStreamSynchronize(s));
   c->have_modes = true;
+  c->unit_modes = unit;
   return FP_OK;
 }
 
@@ -718,7 +727,7 @@ int phase_pass(fp_ctx* c, const fp_rates_opts& o, int nT, const double* T, doubl
   int rc = fp::make_selection(c, o, stride == 1, &sel, err);  // a q' stride is not symmetric under q -> -q
   if (rc) return rc;
   fp::Plan p;
-  rc = fp::plan_rates(c, o, nT, sel, 0, &p, err, stride == 1);
+  rc = fp::plan_rates(c, o, nT, sel, 0, &p, err, stride == 1 ? fp::kPairMirror : fp::kPairSliced);
   if (rc) return rc;
   if (stride > 1) {  // a q' tile of one stride: every item owns exactly one sampled q'
     p.t1 = stride;
@@ -727,6 +736,7 @@ int phase_pass(fp_ctx* c, const fp_rates_opts& o, int nT, const double* T, doubl
     p.values = p.n_items * p.J;
     if (p.ctas > p.n_items) p.ctas = (int)std::max<long long>(1, p.n_items);
   }
+  p.psi_u = p.operands = false;  // no vertex
   size_t sz[fp::kScratchParts], total = 0;
   fp::scratch_sizes(c, p, nT, sz);
   for (size_t x : sz) total += x;

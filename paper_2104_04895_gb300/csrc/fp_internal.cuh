@@ -82,6 +82,8 @@ struct RatesArgs {
   const int* pk_start;       // [natoms + 1] groups with D != 0 by atom k, in l order
   const int* pk_grp;         // their group index | l << 24
   const int* pk_zero;        // [natoms^2] the group of (k, l) with D = 0 (phase 1), or -1
+  const double2* psi_u;      // [nq_sel][nb][nquart][3][9] sum_alpha phi e0 of the evaluated points, or null
+  const unsigned* operands;  // [N][2][Shape::kOperand] sliced eigenvectors in fragment order (fp_slices.cuh)
 };
 
 // Which q-points a rates call evaluates, and for which modes.  Time reversal (e^{-lambda} = conj e^{lambda},
@@ -106,11 +108,14 @@ struct Plan {
   long long n_items;
   size_t smem;
   bool pair = false, mirror = false;  // the pair kernel; with a slot per (evaluated point, q')
+  bool sliced = false;                // its contractions on the tensor cores
+  bool operands = false;              // with the sliced eigenvectors in the scratch
+  bool psi_u = false;                 // its Psi prologue from the table U
   long long values = 0;               // partial sums per temperature
 };
 
 // Device working memory of one rates call (owned by the caller of run_rates), in the order of scratch_sizes.
-constexpr int kScratchParts = 16;
+constexpr int kScratchParts = 18;
 constexpr int kScratchPartial = 7;  // index of the per-item partial sums
 constexpr int kCounters = 10;       // queue, accepted ++, +-, --, vertex entries, terms evaluated, wait timeouts,
                                     // iterations, pairs, spare
@@ -131,6 +136,8 @@ struct Scratch {
   float* qfcf;                   // [nquart*81]
   float2* twf;                   // [L]
   float* wtf;                    // [nT][N*nb][3]
+  double2* psi_u;                // [nq_sel][nb][nquart][3][9] (pair kernel, where it fits)
+  unsigned* operands;            // [N][2][Shape::kOperand] (sliced pair kernel)
 };
 
 }  // namespace fp
@@ -172,6 +179,7 @@ struct fp_ctx {
   double* d_t3_fc = nullptr;   // [n3][27] Phi3 / sqrt(Mi Mj Mk)
   // modes
   bool have_modes = false;
+  bool unit_modes = false;  // eigenvectors of norm 1 within 1e-5
   double* d_omega = nullptr;
   double2* d_evec = nullptr;
   double* d_vel = nullptr;
@@ -208,10 +216,11 @@ cudaError_t launch_weights(fp_ctx* c, int nT, const double* d_T, double* d_wt, c
 // unless o.no_time_reversal or o.nu_select is set or fold_allowed is false.  FP_EINVAL on a bad q range.
 int make_selection(const fp_ctx* c, const fp_rates_opts& o, bool fold_allowed, Selection* s, std::string* err);
 // Validate options and choose tiles; `partial_budget` (bytes, 0 = unlimited) enlarges the q'-tile until the
-// per-item partial sums fit; `mirror` allows the pair kernel's slot per (evaluated point, q') where it fits.
-// Returns FP_OK or an FP_E* code with a message in *err.
+// per-item partial sums fit; `form` is the richest form of the rate kernel that the caller allows.  Returns FP_OK or an
+// FP_E* code with a message in *err.
+enum RateForm { kOrdered = 0, kPair = 1, kPairSliced = 2, kPairMirror = 3 };
 int plan_rates(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, size_t partial_budget, Plan* p,
-               std::string* err, bool mirror = true);
+               std::string* err, RateForm form = kPairMirror);
 // Byte sizes of the Scratch buffers of a plan, in the order of the Scratch fields (each rounded up to 256).
 void scratch_sizes(const fp_ctx* c, const Plan& p, int nT, size_t sizes[kScratchParts]);
 // Scratch pointers laid out from `base` with the sizes of scratch_sizes.

@@ -104,19 +104,25 @@ extern "C" int fp_rates4_noalloc(fp_ctx* c, int nT, const double* T, double sb, 
   fp::Plan p0;
   fp_rates_opts o_probe = o;
   if (o_probe.k1_tile <= 0) o_probe.k1_tile = c->N;  // smallest partials, for the fixed-size part
-  rc = fp::plan_rates(c, o_probe, nT, sel, 0, &p0, &err, false);
-  if (rc) return nfail(c, rc, "fp_rates4_noalloc: " + err);
   size_t sz[fp::kScratchParts], fixed = 0;
-  fp::scratch_sizes(c, p0, nT, sz);
-  for (int i = 0; i < fp::kScratchParts; ++i)
-    if (i != fp::kScratchPartial) fixed += sz[i];
+  fp::RateForm form = fp::kPairMirror;
+  for (;;) {  // simpler forms of the rate kernel need less scratch
+    rc = fp::plan_rates(c, o_probe, nT, sel, 0, &p0, &err, form == fp::kPairMirror ? fp::kPairSliced : form);
+    if (rc) return nfail(c, rc, "fp_rates4_noalloc: " + err);
+    fp::scratch_sizes(c, p0, nT, sz);
+    fixed = 0;
+    for (int i = 0; i < fp::kScratchParts; ++i)
+      if (i != fp::kScratchPartial) fixed += sz[i];
+    if (fixed + sz[fp::kScratchPartial] <= kScratchBytes || form == fp::kOrdered) break;
+    form = form == fp::kPairMirror ? fp::kPair : fp::kOrdered;
+  }
   if (fixed + sz[fp::kScratchPartial] > kScratchBytes)
     return nfail(c, FP_EINVAL, "fp_rates4_noalloc: this problem needs at least " +
                                    std::to_string(fixed + sz[fp::kScratchPartial]) +
                                    " bytes of scratch; the static scratch holds " + std::to_string(kScratchBytes) +
                                    " bytes (use fp_rates4_device)");
   fp::Plan p;
-  rc = fp::plan_rates(c, o, nT, sel, kScratchBytes - fixed - 256, &p, &err);
+  rc = fp::plan_rates(c, o, nT, sel, kScratchBytes - fixed - 256, &p, &err, form);
   if (rc) return nfail(c, rc, "fp_rates4_noalloc: " + err);
   fp::scratch_sizes(c, p, nT, sz);
   size_t total = 0;

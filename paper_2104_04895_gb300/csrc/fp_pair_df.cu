@@ -4,12 +4,12 @@
 namespace fp {
 const void* pair_kernel_df(int nb, int maxt) {
   switch (nb * 100 + maxt) {
-    case 301: return reinterpret_cast<const void*>(pair_kernel<3, 1, true>);
-    case 308: return reinterpret_cast<const void*>(pair_kernel<3, kMaxT, true>);
-    case 601: return reinterpret_cast<const void*>(pair_kernel<6, 1, true>);
-    case 608: return reinterpret_cast<const void*>(pair_kernel<6, kMaxT, true>);
-    case 1201: return reinterpret_cast<const void*>(pair_kernel<12, 1, true>);
-    case 1208: return reinterpret_cast<const void*>(pair_kernel<12, kMaxT, true>);
+    case 301: return reinterpret_cast<const void*>(pair_kernel<3, 1, true, false>);
+    case 308: return reinterpret_cast<const void*>(pair_kernel<3, kMaxT, true, false>);
+    case 601: return reinterpret_cast<const void*>(pair_kernel<6, 1, true, false>);
+    case 608: return reinterpret_cast<const void*>(pair_kernel<6, kMaxT, true, false>);
+    case 1201: return reinterpret_cast<const void*>(pair_kernel<12, 1, true, false>);
+    case 1208: return reinterpret_cast<const void*>(pair_kernel<12, kMaxT, true, false>);
     default: return nullptr;
   }
 }

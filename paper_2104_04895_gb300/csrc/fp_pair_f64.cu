@@ -2,14 +2,19 @@
 #include "fp_pair_kernel.cuh"
 
 namespace fp {
-const void* pair_kernel_f64(int nb, int maxt) {
-  switch (nb * 100 + maxt) {
-    case 301: return reinterpret_cast<const void*>(pair_kernel<3, 1, false>);
-    case 308: return reinterpret_cast<const void*>(pair_kernel<3, kMaxT, false>);
-    case 601: return reinterpret_cast<const void*>(pair_kernel<6, 1, false>);
-    case 608: return reinterpret_cast<const void*>(pair_kernel<6, kMaxT, false>);
-    case 1201: return reinterpret_cast<const void*>(pair_kernel<12, 1, false>);
-    case 1208: return reinterpret_cast<const void*>(pair_kernel<12, kMaxT, false>);
+// sliced: the contractions on the tensor cores (6 and 12 branches)
+const void* pair_kernel_f64(int nb, int maxt, bool sliced) {
+  switch (nb * 1000 + maxt * 10 + (sliced ? 1 : 0)) {
+    case 3010: return reinterpret_cast<const void*>(pair_kernel<3, 1, false, false>);
+    case 3080: return reinterpret_cast<const void*>(pair_kernel<3, kMaxT, false, false>);
+    case 6010: return reinterpret_cast<const void*>(pair_kernel<6, 1, false, false>);
+    case 6080: return reinterpret_cast<const void*>(pair_kernel<6, kMaxT, false, false>);
+    case 12010: return reinterpret_cast<const void*>(pair_kernel<12, 1, false, false>);
+    case 12080: return reinterpret_cast<const void*>(pair_kernel<12, kMaxT, false, false>);
+    case 6011: return reinterpret_cast<const void*>(pair_kernel<6, 1, false, true>);
+    case 6081: return reinterpret_cast<const void*>(pair_kernel<6, kMaxT, false, true>);
+    case 12011: return reinterpret_cast<const void*>(pair_kernel<12, 1, false, true>);
+    case 12081: return reinterpret_cast<const void*>(pair_kernel<12, kMaxT, false, true>);
     default: return nullptr;
   }
 }

@@ -27,19 +27,27 @@
 // compacted into a list that the warp evaluates 32 at a time (W, Gaussian), and each value returns to the row that
 // owns it: the FP64 pipe, the bound of the FP64 path, runs on full warps however unevenly the terms fall on rows.
 //
-// Measured (GB300) against the ordered kernel: diamond 6^3 FP64 578 -> 223 ms, diamond 7x6x5 double-float 262 -> 87 ms,
-// LiCoO2 5x4x3 FP64 with 3 T 387 -> 154 ms, BAs 5^3 normal/Umklapp 294 -> 131 ms, BAs 6x5x5 phase space 140 -> 41 ms,
-// simple cubic 4^3 2.15 -> 1.49 ms.  The FP64 path stays bound by the FP64 pipe (about 1.7 lane operations per clock
-// and SM in a DFMA chain): per k2 of six branches 31k lane DFMAs for T, 20k for W (64 % of the entries accepted), 8k
-// for A and 12k for the terms.
+// On the FP64 path with 6 or 12 branches and unit eigenvectors both vertex contractions run on the tensor cores in exact integer slices
+// (SL, fp_slices.cuh): A is built in FP64, its digits contract with those of e3 to T, T's digits with those of e2 to
+// every W of the block, which costs the FP64 pipe only the A sums and |W|^2.  A scale per (j0, x), the power of two
+// above the Frobenius norm of its A block, keeps all three in range.
+//
+// Measured (GB300): ordered kernel -> pair kernel -> with slices and the U table of the prologue:
+//   diamond 6^3 FP64            578 -> 223 -> 125 ms      LiCoO2 5x4x3 FP64, 3 T   386 -> 154 -> 82 ms
+//   diamond 7x6x5 double-float  262 -> 88 ms (no slices: 107 ms with them, the FP64 A sums and conversions cost more
+//                               than the FP32 contraction; LiCoO2 4x3x3 24.3 ms either way)
+//   simple cubic 4^3 FP64       2.15 -> 1.49 -> 1.13 ms (nb = 3: no slices)
+// Without slices the FP64 pipe (about 1.7 lane FMAs per clock and SM) is 91 % busy: per k2 of six branches 31k lane
+// FMAs for T, 20k for W, 8k for A, 12k for the terms.  With them it is the terms, A and the barriers between phases.
 #pragma once
 #include "fp_rates_kernel.cuh"
+#include "fp_slices.cuh"
 
 namespace fp {
 namespace {
 
 constexpr int kPairGroup = 6;   // j3 values compacted at once (five tests each: 30 bits of a lane's mask)
-constexpr int kPairCap = 192;   // list entries per warp and round
+constexpr int kPairCap = 128;   // list entries per warp and round
 
 // Role of the slot (qi, b) of `partial`: the value R(q; b) of the evaluated point q = qlist[qi].
 struct PairRole {
@@ -108,9 +116,10 @@ __host__ __device__ constexpr int pair_blocks_for(int nb) { return nb == 12 ? 1 
 
 struct PairCarve {
   size_t E0, E1, E2, E3, Psi, T, Tw2, TwQ, ncx;                                           // 16-byte complex elements
-  size_t Om0, Om1, Om2, Om3, X, V2, V3, Iv8, F, WB, Wc, Wd, Y, Val, ExpT, ndbl;            // doubles
+  size_t Op;                                                                              // 16-byte words (sliced)
+  size_t Om0, Om1, Om2, Om3, X, V2, V3, Iv8, F, WB, Wc, Wd, Val, ExpT, ndbl;            // doubles
   size_t H0, H1, H2, H3, VH2, VL2, VH3, VL3, PM, nflt;                                     // floats
-  size_t KLs, KLg, KLz, nint;                                                             // ints
+  size_t KLs, KLg, KLz, Sc, nint;                                                             // ints
   size_t Ent;                                                                             // uint16
   size_t Mult;                                                                            // bytes
   __host__ __device__ size_t bytes() const {
@@ -118,18 +127,21 @@ struct PairCarve {
   }
 };
 
-__host__ __device__ inline PairCarve make_pair_carve(int nb, int J, int G, int nquart, int nT, int threads) {
+__host__ __device__ inline PairCarve make_pair_carve(int nb, int J, int G, int nquart, int nT, int threads,
+                                                   bool sliced) {
   PairCarve c;
   const size_t nb2 = (size_t)nb * nb, na = nb / 3, nwarps = ((size_t)threads + 31) / 32;
   size_t o = 0;
   c.E0 = o; o += (size_t)J * nb;
   c.E1 = o; o += nb2;
-  c.E2 = o; o += nb2;
-  c.E3 = o; o += nb2;
+  c.E2 = o; o += sliced ? 0 : nb2;
+  c.E3 = o; o += sliced ? 0 : nb2;
   c.Psi = o; o += (size_t)J * nb * G * 9;
-  c.T = o; o += (size_t)J * nb * (nb2 + 1);
+  // T blocks (j0, x), padded by one entry; sliced: rows of digits of A and then of T, later |W|^2 and the lists
+  c.T = o; o += sliced ? nwarps * 32 * (nb == 6 ? 36 : 76) / 4 : (size_t)J * nb * (nb2 + 1);
   c.Tw2 = o; o += G;
   c.TwQ = o; o += nquart;
+  c.Op = o; o += sliced ? 2 * 6 * (nb == 6 ? 2 * 32 * 2 : 3 * 32 * 3) / 4 : 0;
   c.ncx = o;
   size_t d = 0;
   c.Om0 = d; d += J;
@@ -144,8 +156,7 @@ __host__ __device__ inline PairCarve make_pair_carve(int nb, int J, int G, int n
   c.WB = d; d += nT > 1 ? 3 * (size_t)nT * nb2 : 0;  // c and d weights of P1, P2, P3 per temperature
   c.Wc = d; d += 2 * (size_t)nT * nb;  // (1+n)/w and n/w of k2
   c.Wd = d; d += 2 * (size_t)nT * nb;  // and of k3
-  c.Y = d; d += 2 * nb2;               // wc + wd, wc - wd
-  c.Val = d; d += nwarps * kPairCap;
+  c.Val = d; d += sliced ? 0 : nwarps * kPairCap;
   c.ExpT = d; d += kExpTab;
   c.ndbl = d;
   size_t f = 0;
@@ -164,8 +175,9 @@ __host__ __device__ inline PairCarve make_pair_carve(int nb, int J, int G, int n
   c.KLs = k; k += na + 1;
   c.KLg = k; k += G;
   c.KLz = k; k += na * na;
+  c.Sc = k; k += sliced ? (size_t)J * nb : 0;
   c.nint = k;
-  c.Ent = nwarps * kPairCap;
+  c.Ent = sliced ? 0 : nwarps * kPairCap;
   c.Mult = (size_t)J + nb;
   return c;
 }
@@ -177,9 +189,42 @@ __device__ __forceinline__ double pair_val<double>(double v) { return v; }
 template <>
 __device__ __forceinline__ float2 pair_val<float2>(double v) { return df_make(v); }
 
-// NB branches, up to MAXT temperatures; DF: vertex contraction and P1 terms in double-float on the FP32 pipes
-template <int NB, int MAXT, bool DF>
+// x + y or x - y (the sign flipped in the integer pipe)
+__device__ __forceinline__ double add_signed(double x, double y, bool plus) {
+  return __dadd_rn(x, __hiloint2double(__double2hiint(y) ^ (plus ? 0 : 0x80000000), __double2loint(y)));
+}
+
+// exp_neg64 (fp_rates_kernel.cuh) with the range test and the rounding of v to k kept off the FP64 compare and convert
+// instructions: v + 1.5 2^52 holds k = rint(v) in its low bits
+__device__ __forceinline__ double pair_exp_neg64(double v, const double* tab) {
+  if (__double2hiint(v) > 0x40700000) return exp(-v * kExpH);  // v >= 256 (1 + 2^-20) (also NaN)
+  const double vm = __dadd_rn(v, slices::kMagic);
+  const int k = __double2loint(vm);
+  const double t = __dsub_rn(__dsub_rn(vm, slices::kMagic), v);
+  double p = (1.0 / 120.0) / 1073741824.0;
+  p = fma(p, t, (1.0 / 24.0) / 16777216.0);
+  p = fma(p, t, (1.0 / 6.0) / 262144.0);
+  p = fma(p, t, 0.5 / 4096.0);
+  p = fma(p, t, kExpH);
+  p = fma(p, t, 1.0);
+  return tab[k] * p;
+}
+
+// exp of the second order of {c, d} averaged in (rare: out of line)
+__device__ __noinline__ double pair_two_orders(double ex, double z8, const double* tab) {
+  return 0.5 * (ex + pair_exp_neg64(z8 * z8, tab));
+}
+__device__ __noinline__ float2 pair_two_orders(float2 ex, float2 z8, const float2* tab) {
+  const float2 m = df_add(ex, df_exp_neg64(df_mul(z8, z8), tab));
+  return make_float2(0.5f * m.x, 0.5f * m.y);
+}
+
+// NB branches, up to MAXT temperatures.  DF: vertex contraction and terms in double-float on the FP32 pipes.  SL: both
+// vertex contractions on the tensor cores in exact slices (fp_slices.cuh; unit eigenvectors, nb = 6 or 12): A in FP64,
+// T as digits, |W|^2 of every entry in FP64.
+template <int NB, int MAXT, bool DF, bool SL>
 __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pair_kernel(RatesArgs a) {
+  static_assert(!(DF && SL), "the double-float contraction has no sliced form");
   constexpr int NB2 = NB * NB, NA = NB / 3;
   using C = Cx<double>;
   using VT = typename std::conditional<DF, float2, double>::type;  // value of an evaluated entry
@@ -189,7 +234,7 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
   const int J = a.J, G = a.G, nT = a.nT, N = a.N;
   const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, warp = tid >> 5;
   const int rows = J * NB2;
-  const PairCarve cv = make_pair_carve(NB, J, G, a.nquart, nT, nthr);
+  const PairCarve cv = make_pair_carve(NB, J, G, a.nquart, nT, nthr, SL);
   C* cx = reinterpret_cast<C*>(smem);
   C *sE0 = cx + cv.E0, *sE1 = cx + cv.E1, *sE2 = cx + cv.E2, *sE3 = cx + cv.E3;
   C *sPsi = cx + cv.Psi, *sT = cx + cv.T, *sTw2 = cx + cv.Tw2, *sTwQ = cx + cv.TwQ;
@@ -197,10 +242,14 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
   double *sOm0 = db + cv.Om0, *sOm1 = db + cv.Om1, *sOm2 = db + cv.Om2, *sOm3 = db + cv.Om3;
   double *sV2 = db + cv.V2, *sV3 = db + cv.V3, *sWc = db + cv.Wc, *sWd = db + cv.Wd;
   // values of the path's type: doubles, or double-floats in the same slots
-  VT *sX = reinterpret_cast<VT*>(db + cv.X), *sY = reinterpret_cast<VT*>(db + cv.Y);
+  double* sX = db + cv.X;
   VT *sIv8 = reinterpret_cast<VT*>(db + cv.Iv8), *sF = reinterpret_cast<VT*>(db + cv.F);
   VT *sWB = reinterpret_cast<VT*>(db + cv.WB), *sExpT = reinterpret_cast<VT*>(db + cv.ExpT);
-  VT* sVal = reinterpret_cast<VT*>(db + cv.Val) + (size_t)warp * kPairCap;
+  // sliced: W [j0 x][y][j3] (combine_magic) and the lists take the place of the digits once these are in registers
+  double2* sW = reinterpret_cast<double2*>(sT);
+  unsigned* sDig = reinterpret_cast<unsigned*>(sT);
+  const unsigned* sOp = reinterpret_cast<const unsigned*>(cx + cv.Op);
+  VT* sVal = reinterpret_cast<VT*>(SL ? reinterpret_cast<double*>(sW + (size_t)J * NB * NB2) : db + cv.Val) + (size_t)warp * kPairCap;
   double* sRed = reinterpret_cast<double*>(sT);  // the T block, free outside the k2 loop
   float* fb = reinterpret_cast<float*>(db + cv.ndbl);
   float *sH0 = fb + cv.H0, *sH1 = fb + cv.H1, *sH2 = fb + cv.H2, *sH3 = fb + cv.H3;
@@ -208,7 +257,10 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
   float2* sPM = reinterpret_cast<float2*>(fb + cv.PM);
   int* ib = reinterpret_cast<int*>(fb + cv.nflt);
   int *sKLs = ib + cv.KLs, *sKLg = ib + cv.KLg, *sKLz = ib + cv.KLz;
-  unsigned short* sEnt = reinterpret_cast<unsigned short*>(ib + cv.nint) + (size_t)warp * kPairCap;
+  int* sSc = ib + cv.Sc;
+  unsigned short* sEnt = (SL ? reinterpret_cast<unsigned short*>(reinterpret_cast<double*>(sW + (size_t)J * NB * NB2) +
+                                                                (size_t)((nthr + 31) / 32) * kPairCap)
+                             : reinterpret_cast<unsigned short*>(ib + cv.nint)) + (size_t)warp * kPairCap;
   unsigned char* sMa = reinterpret_cast<unsigned char*>(reinterpret_cast<unsigned short*>(ib + cv.nint) + cv.Ent);
   unsigned char* sMb = sMa + J;
 
@@ -282,12 +334,47 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
       for (int x = 0; x < NB; ++x) any |= sMb[x];
       for (int o = tid; o < J * NB; o += nthr) {
         const int jj = o / NB, x = o % NB;
-        sX[o] = pair_val<VT>(sOm0[jj] + sOm1[x]);
-        sX[J * NB + o] = pair_val<VT>(sOm0[jj] - sOm1[x]);
+        sX[o] = __dadd_rn(sOm0[jj], sOm1[x]);
+        sX[J * NB + o] = __dsub_rn(sOm0[jj], sOm1[x]);
       }
       // Psi[jj][j1][grp][gt] (see fp_rates_kernel.cuh): one thread per (jj, j1, grp) and block of three (gamma, theta)
       constexpr int kGtb = 3;
-      const int npsi = unit || !any ? 0 : J * NB * G * (9 / kGtb);
+      if (a.psi_u && !unit && any) {
+        // with U = sum_alpha phi e0 of this q at hand: Psi = sum_Q sum_beta (tw1_Q e1_beta) U, 36 FMAs per quartet and
+        // three (gamma, theta) instead of 90
+        const double2* U = a.psi_u + ((size_t)qi * NB + j0b) * a.nquart * 27;
+        for (int o = tid; o < J * NB * G * (9 / kGtb); o += nthr) {
+          const int gb = o % (9 / kGtb), jr = (o / (9 / kGtb)) % (J * NB), grp = o / ((9 / kGtb) * J * NB);
+          const int j1 = jr % NB, jj = jr / NB;
+          C sum[kGtb];
+#pragma unroll
+          for (int u = 0; u < kGtb; ++u) sum[u] = cmk<double>(0, 0);
+          for (int qq = a.grp_qstart[grp]; qq < a.grp_qstart[grp + 1]; ++qq) {
+            const int Q = a.grp_q[qq];
+            const C tq = sTwQ[Q];
+            const double2* uq = U + ((size_t)jj * a.nquart + Q) * 27 + gb * kGtb;
+            const C* e1 = sE1 + j1 * NB + 3 * a.qmeta[9 * Q + 1];
+#pragma unroll
+            for (int be = 0; be < 3; ++be) {
+              const C et = cmul(tq, e1[be]);
+#pragma unroll
+              for (int u = 0; u < kGtb; ++u) {
+                const double2 v = uq[be * 9 + u];
+                cfma(sum[u], et, cmk<double>(v.x, v.y));
+              }
+            }
+          }
+#pragma unroll
+          for (int u = 0; u < kGtb; ++u) {
+            const size_t at = (size_t)(jr * G + grp) * 9 + gb * kGtb + u;
+            if constexpr (DF)
+              reinterpret_cast<float4*>(sPsi)[at] = cdf_from(sum[u].re, sum[u].im);
+            else
+              sPsi[at] = sum[u];
+          }
+        }
+      }
+      const int npsi = a.psi_u || unit || !any ? 0 : J * NB * G * (9 / kGtb);
       for (int o = tid; o < npsi; o += nthr) {
         const int gb = o % (9 / kGtb);
         const int jr = (o / (9 / kGtb)) % (J * NB);
@@ -327,6 +414,35 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
             reinterpret_cast<float4*>(sPsi)[(size_t)t9 * 9 + gb * kGtb + u] = cdf_from(sum[u].re, sum[u].im);
           else
             sPsi[(size_t)t9 * 9 + gb * kGtb + u] = sum[u];
+        }
+      }
+
+      if constexpr (SL) {
+        // scale of every (j0, x): 2^s above the Frobenius norm of its A block for any phases, so above every element of
+        // A, T and W (unit eigenvectors)
+        double* sB = reinterpret_cast<double*>(sT);
+        __syncthreads();
+        if (!unit && any) {
+          for (int o = tid; o < J * NB * NB2; o += nthr) {
+            const int ab = o / NB2, k = (o / NB) % NB, l = o % NB;
+            const C* ps = sPsi + (size_t)ab * G * 9 + (k % 3) * 3 + l % 3;
+            double sum = 0.0;
+            auto take = [&](int grp) {  // |z| <= max + (sqrt 2 - 1) min
+              const C z = ps[grp * 9];
+              const double u = fabs(z.re), v = fabs(z.im);
+              sum += fmax(u, v) + 0.41421357 * fmin(u, v);
+            };
+            if (sKLz[(k / 3) * NA + l / 3] >= 0) take(sKLz[(k / 3) * NA + l / 3]);
+            for (int gi = sKLs[k / 3]; gi < sKLs[k / 3 + 1]; ++gi)
+              if (sKLg[gi] >> 24 == l / 3) take(sKLg[gi] & 0xffffff);
+            sB[o] = sum * sum;
+          }
+          __syncthreads();
+          for (int ab = tid; ab < J * NB; ab += nthr) {
+            double f = 0.0;
+            for (int o = 0; o < NB2; ++o) f += sB[ab * NB2 + o];
+            sSc[ab] = f > 0.0 ? (f < 1e300 ? ilogb(sqrt(f) * 1.0001) + 1 : 1000) : 0;
+          }
         }
       }
 
@@ -445,6 +561,14 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
         const bool twice = kd != k2;  // both orders of {c, d} come from this visit
         // ---- tables of k2 and k3
         if (a.nu_select != 0 && tid == 0) s_umask = pair_umklapp_bits(a, g, g1, g2, g3);
+        if constexpr (SL) {
+          constexpr int kOp4 = slices::Shape<SL ? NB : 6>::kOperand / 4;
+          const uint4* src = reinterpret_cast<const uint4*>(a.operands);
+          uint4* dst = reinterpret_cast<uint4*>(cx + cv.Op);
+          if (!unit)
+            for (int o = tid; o < 2 * kOp4; o += nthr)
+              dst[o] = src[(size_t)(o < kOp4 ? k3 : k2) * 2 * kOp4 + o];
+        } else
         for (int o = tid; o < NB2; o += nthr) {
           const double2 e2v = a.evec[(size_t)k2 * NB2 + o], e3v = a.evec[(size_t)k3 * NB2 + o];
           if constexpr (DF) {
@@ -517,11 +641,9 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
           const double f = iv >= 0.0 ? iv * kInvSqrtPi : 1.0;
           if (tab) {
             sF[e] = pair_val<VT>((twice ? 1.0 : 0.5) * f * (MAXT == 1 ? sWc[2 * y + 1] * sWd[2 * j3 + 1] : 1.0));
-            sY[e] = pair_val<VT>(sOm2[y] + sOm3[j3]);
           } else {
             sF[NB2 + e] = pair_val<VT>(0.5 * f * (MAXT == 1 ? sWc[2 * y] * sWd[2 * j3 + 1] : 1.0));
             sF[2 * NB2 + e] = pair_val<VT>(0.5 * f * (MAXT == 1 ? sWc[2 * y + 1] * sWd[2 * j3] : 1.0));
-            sY[NB2 + e] = pair_val<VT>(sOm2[y] - sOm3[j3]);
           }
         }
         if constexpr (MAXT > 1)
@@ -615,14 +737,109 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
               for (int th = 0; th < 3; ++th) cfma(cur[th], tw, ps[th]);
             }
             put();
-            C* trow = sT + (size_t)(rjj * NB + rj1) * (NB2 + 1) + rc * NB;
+            if constexpr (SL) {
+              const int sc = sSc[rjj * NB + rj1];
+              unsigned* drow = sDig + tid * slices::Shape<SL ? NB : 6>::kRow;
 #pragma unroll
-            for (int j3 = 0; j3 < NB; ++j3) {
-              C s = cmk<double>(0, 0);
+              for (int d = 0; d < NB; ++d) {
+                const unsigned long long vr = slices::fixed_from(Arow[d].re, sc), vi = slices::fixed_from(Arow[d].im, sc);
 #pragma unroll
-              for (int d = 0; d < NB; ++d) cfma_conj(s, Arow[d], sE3[j3 * NB + d]);
-              trow[j3] = s;
+                for (int i = 0; i < slices::kDigits; ++i) drow[i * NB + d] = slices::pack_digit(i, vr, vi);
+              }
+            } else {
+              C* trow = sT + (size_t)(rjj * NB + rj1) * (NB2 + 1) + rc * NB;
+#pragma unroll
+              for (int j3 = 0; j3 < NB; ++j3) {
+                C s = cmk<double>(0, 0);
+#pragma unroll
+                for (int d = 0; d < NB; ++d) cfma_conj(s, Arow[d], sE3[j3 * NB + d]);
+                trow[j3] = s;
+              }
             }
+          }
+        }
+        if constexpr (SL) {
+          if (!unit) {
+            // T = A conj(e3) and W = T e2 in slices; a warp's 32 rows are two row tiles.  Rows of A are (j0, x, k gamma);
+            // the digits of T go to rows (j0, x, j3), which other warps may hold, so its fragments and stores are
+            // separated by barriers
+            using Sh = slices::Shape<SL ? NB : 6>;
+            const int g = lane >> 2, t = lane & 3;
+            unsigned af[2][slices::kDigits][Sh::kA];
+            __syncwarp();
+            slices::load_a<SL ? NB : 6>(sDig, warp * 32, lane, af[0]);
+            slices::load_a<SL ? NB : 6>(sDig, warp * 32 + 16, lane, af[1]);
+            __syncthreads();
+#pragma unroll
+            for (int nt = 0; nt < Sh::kTiles; ++nt) {
+              unsigned bf[slices::kDigits][Sh::kB];
+              slices::load_b<SL ? NB : 6>(sOp, nt, lane, bf);
+#pragma unroll
+              for (int mt = 0; mt < 2; ++mt) {
+                float acc[slices::kLevels][4];
+                slices::contract<SL ? NB : 6>(acc, af[mt], bf);
+                float D[4][slices::kLevels];
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+#pragma unroll
+                  for (int s = 0; s < slices::kLevels; ++s) D[c][s] = acc[s][c];
+                const int r0 = warp * 32 + mt * 16 + g;
+                if (NB == 6 && nt == 1) {  // one real of branches 4, 5 per lane, of two rows
+                  const unsigned long long v0 = slices::combine_fixed<NB>(D[0]), v1 = slices::combine_fixed<NB>(D[2]);
+                  const int j = 4 + (t >> 1), ri = t & 1;
+                  unsigned short* d0 = reinterpret_cast<unsigned short*>(sDig + ((r0 / NB) * NB + j) * Sh::kRow + r0 % NB) + ri;
+                  unsigned short* d1 = reinterpret_cast<unsigned short*>(sDig + (((r0 + 8) / NB) * NB + j) * Sh::kRow + (r0 + 8) % NB) + ri;
+#pragma unroll
+                  for (int i = 0; i < slices::kDigits; ++i) {
+                    const unsigned w = slices::pack_digit(i, v0, v1);
+                    if (r0 < rows) d0[2 * i * NB] = (unsigned short)w;
+                    if (r0 + 8 < rows) d1[2 * i * NB] = (unsigned short)(w >> 16);
+                  }
+                } else {
+#pragma unroll
+                  for (int h = 0; h < 2; ++h) {
+                    const int r = r0 + 8 * h;
+                    const unsigned long long vr = slices::combine_fixed<NB>(D[2 * h]), vi = slices::combine_fixed<NB>(D[2 * h + 1]);
+                    unsigned* drow = sDig + ((r / NB) * NB + nt * 4 + t) * Sh::kRow + r % NB;
+                    if (r < rows)
+#pragma unroll
+                      for (int i = 0; i < slices::kDigits; ++i) drow[i * NB] = slices::pack_digit(i, vr, vi);
+                  }
+                }
+              }
+            }
+            __syncthreads();
+            slices::load_a<SL ? NB : 6>(sDig, warp * 32, lane, af[0]);
+            slices::load_a<SL ? NB : 6>(sDig, warp * 32 + 16, lane, af[1]);
+            __syncthreads();
+#pragma unroll
+            for (int nt = 0; nt < Sh::kTiles; ++nt) {
+              unsigned bf[slices::kDigits][Sh::kB];
+              slices::load_b<SL ? NB : 6>(sOp + Sh::kOperand, nt, lane, bf);
+#pragma unroll
+              for (int mt = 0; mt < 2; ++mt) {
+                float acc[slices::kLevels][4];
+                slices::contract<SL ? NB : 6>(acc, af[mt], bf);
+                float D[4][slices::kLevels];
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+#pragma unroll
+                  for (int s = 0; s < slices::kLevels; ++s) D[c][s] = acc[s][c];
+                const int r0 = warp * 32 + mt * 16 + g;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                  const int r = r0 + 8 * h, at = (r / NB) * NB2 + r % NB;  // row (j0, x, j3): entry [j0 x][y][j3]
+                  const double x = slices::combine_magic<NB>(D[2 * h]);
+                  if (NB == 6 && nt == 1) {
+                    if (r < rows) reinterpret_cast<double*>(sW + at + (4 + (t >> 1)) * NB)[t & 1] = x;
+                  } else {
+                    const double y = slices::combine_magic<NB>(D[2 * h + 1]);
+                    if (r < rows) sW[at + (nt * 4 + t) * NB] = make_double2(x, y);
+                  }
+                }
+              }
+            }
+            if (has_row) nwf += NB;
           }
         }
         __syncthreads();
@@ -704,7 +921,7 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
             // compacted in lane order, test by test within a lane
             const int nmy = __popc(m);
             nte += nmy;
-            if (!unit) nwf += nmy;
+            if (!SL && !unit) nwf += nmy;
             int incl = nmy;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
@@ -732,9 +949,15 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
                 const bool tab0 = kind == 1 || kind == 2;
                 const VT iv8 = sIv8[(tab0 ? 0 : NB2) + e];
                 VT gv = sF[(tab0 ? kind : 0) * NB2 + e];
-                const VT vx = sX[(kind >= 3 ? J * NB : 0) + ab];
-                VT vy = sY[(tab0 ? NB2 : 0) + e];
-                const bool minus = kind != 1 && kind != 4;
+                // dw in the operation order of the definition (P5 negated): at a resonance of a mode with itself it is
+                // a rounding error, which a small sigma makes visible
+                const double wx = sX[(kind >= 3 ? J * NB : 0) + ab];
+                const double wc = sOm2[ey], wd = sOm3[j3];
+                const double y1 = kind == 2 ? wd : wc, y2 = kind == 2 ? wc : wd;
+                const bool plus1 = kind == 1 || kind == 2 || kind == 4, plus2 = kind == 4;
+                const double dw = add_signed(add_signed(wx, y1, plus1), y2, plus2);
+                // the other order of {c, d} differs by its rounding, which only a sigma below 1e-3 rad/ps shows
+                const bool orders = twice && !tab0 && !(en & 1024u);
                 VT v;
                 if constexpr (DF) {
                   float2 W2 = make_float2(1.f, 0.f);
@@ -746,16 +969,24 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
                     for (int c = 0; c < NB; ++c) cdf_mac(Wd, e2[c], tb[c * NB]);
                     W2 = cdf_abs2_df(Wd);
                   }
-                  if (minus) vy = make_float2(-vy.x, -vy.y);
                   if (iv8.x >= 0.f) {
-                    const float2 x8 = df_mul(df_add(vx, vy), iv8);
-                    gv = df_mul(gv, df_exp_neg64(df_mul(x8, x8), sExpT));
+                    const float2 x8 = df_mul(df_make(dw), iv8);
+                    float2 ex = df_exp_neg64(df_mul(x8, x8), sExpT);
+                    if (iv8.x > 8000.f && orders)
+                      ex = pair_two_orders(ex, df_mul(df_make(add_signed(add_signed(wx, y2, plus1), y1, plus2)), iv8), sExpT);
+                    gv = df_mul(gv, ex);
                   }
                   v = df_mul(W2, gv);
                   if (en & 1024u) v = make_float2(0.5f * v.x, 0.5f * v.y);
                 } else {
                   double W2 = 1.0;
-                  if (!unit) {
+                  if constexpr (SL) {
+                    if (!unit) {
+                      const double2 w = sW[ab * NB2 + e];
+                      const double wr = w.x - slices::kMagic, wi = w.y - slices::kMagic;
+                      W2 = fma(wr, wr, wi * wi);
+                    }
+                  } else if (!unit) {
                     const C* tb = sT + (size_t)ab * (NB2 + 1) + j3;
                     const C* e2 = sE2 + ey * NB;
                     C Wv = cmk<double>(0, 0);
@@ -763,10 +994,12 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
                     for (int c = 0; c < NB; ++c) cfma(Wv, e2[c], tb[c * NB]);
                     W2 = Wv.re * Wv.re + Wv.im * Wv.im;
                   }
-                  if (minus) vy = __longlong_as_double(__double_as_longlong(vy) ^ 0x8000000000000000ULL);
-                  if (iv8 >= 0.0) {
-                    const double x8 = (vx + vy) * iv8;
-                    gv *= exp_neg64(x8 * x8, sExpT);
+                  if (__double2hiint(iv8) >= 0) {  // not -1 (delta := 1)
+                    const double x8 = dw * iv8;
+                    double ex = pair_exp_neg64(x8 * x8, sExpT);
+                    if (__double2hiint(iv8) > 0x40bf4000 && orders)  // 8 / sigma > 8000
+                      ex = pair_two_orders(ex, add_signed(add_signed(wx, y2, plus1), y1, plus2) * iv8, sExpT);
+                    gv *= ex;
                   }
                   v = W2 * gv;
                   if (en & 1024u) v *= 0.5;
@@ -799,9 +1032,11 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
 #pragma unroll
           for (int tt = 0; tt < MAXT; ++tt)
             if (tt == t) s1 = S1[tt];
-          sRed[tid] = s1;
-          sRed[rows + tid] = R45[t];
-          sRed[2 * rows + tid] = R45[nT + t];
+          // sliced: |W|^2 was in units of (2^(s - 51))^2
+          const double f = SL && !unit && any ? scalbn(1.0, 2 * sSc[rjj * NB + rj1] - 102) : 1.0;
+          sRed[tid] = f * s1;
+          sRed[rows + tid] = f * R45[t];
+          sRed[2 * rows + tid] = f * R45[nT + t];
         }
         __syncthreads();
         if (tid < nout) {

@@ -5,7 +5,7 @@
 
 namespace fp {
 // kernel pointers of the instantiations (fp_pair_*.cu, fp_rates_*.cu)
-const void* pair_kernel_f64(int nb, int maxt);
+const void* pair_kernel_f64(int nb, int maxt, bool sliced);
 const void* pair_kernel_df(int nb, int maxt);
 const void* rates_kernel_f64(int nb, int maxt);
 const void* rates_kernel_f32(int nb, int maxt);
@@ -127,6 +127,38 @@ __global__ void pair_reduce_kernel(RatesArgs a, double pref, double* rates) {
   if (a.mode_counts && t == 0) a.mode_counts[(size_t)q * a.nb + j] = (double)cnt * a.count_scale;
 }
 
+// the sliced eigenvectors of every grid point, in the fragment order of the two contractions
+template <int NB>
+__global__ void operand_kernel(const double2* evec, int N, unsigned* out) {
+  constexpr int kOp = slices::Shape<NB>::kOperand;
+  const long long n = (long long)N * 2 * kOp;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    const long long q = i / (2 * kOp);
+    const int w = (int)(i % (2 * kOp));
+    out[i] = slices::operand_word<NB>(evec + q * NB * NB, w / kOp, w % kOp);
+  }
+}
+
+// U[qi][j0][Q][beta][gamma theta] = sum_alpha phi_Q e_{i alpha}(q, j0) of the evaluated points: the part of the pair
+// kernel's Psi that every partner q' of q shares
+__global__ void psi_u_kernel(RatesArgs a, double2* out) {
+  const long long n = (long long)a.nq_sel * a.nb * a.nquart * 27;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    const int c = (int)(i % 27), Q = (int)((i / 27) % a.nquart), j0 = (int)((i / (27LL * a.nquart)) % a.nb);
+    const int q = a.qlist[i / (27LL * a.nquart * a.nb)];
+    const double2* e = a.evec + ((size_t)q * a.nb + j0) * a.nb + 3 * a.qmeta[9 * Q];
+    const double* f = a.qfc + 81 * (size_t)Q + c;
+    double re = 0.0, im = 0.0;
+    for (int al = 0; al < 3; ++al) {
+      re = fma(f[27 * al], e[al].x, re);
+      im = fma(f[27 * al], e[al].y, im);
+    }
+    out[i] = make_double2(re, im);
+  }
+}
+
+size_t operand_words(int nb) { return 2 * (size_t)(nb == 6 ? slices::Shape<6>::kOperand : slices::Shape<12>::kOperand); }
+
 // p[i] = v (the unit weight table of the unweighted phase space)
 __global__ void fill_kernel(double* p, long long n, double v) {
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
@@ -134,24 +166,27 @@ __global__ void fill_kernel(double* p, long long n, double v) {
 }
 
 // kernel for (precision, nb, number of temperatures, tensor cores): one accumulator per temperature, 1 or up to 8
-const void* rates_kernel_ptr(int precision, int nb, int nT, bool tc, bool pair) {
+const void* rates_kernel_ptr(int precision, int nb, int nT, bool tc, bool pair, bool sliced) {
   const int maxt = nT == 1 ? 1 : kMaxT;
-  if (pair) return precision == FP_PREC_DOUBLE_FLOAT ? pair_kernel_df(nb, maxt) : pair_kernel_f64(nb, maxt);
+  if (pair)
+    return precision == FP_PREC_DOUBLE_FLOAT ? pair_kernel_df(nb, maxt) : pair_kernel_f64(nb, maxt, sliced);
   if (tc) return precision == FP_PREC_MIXED ? rates_kernel_f32_tc(nb, maxt) : nullptr;
   if (precision == FP_PREC_DOUBLE_FLOAT) return rates_kernel_df(nb, maxt);
   return precision == FP_PREC_FP64 ? rates_kernel_f64(nb, maxt) : rates_kernel_f32(nb, maxt);
 }
 
-size_t smem_bytes(int precision, int nb, int J, int G, int nquart, int nT, int threads, bool tc, bool pair) {
-  if (pair) return make_pair_carve(nb, J, G, nquart, nT, threads).bytes();
+size_t smem_bytes(int precision, int nb, int J, int G, int nquart, int nT, int threads, bool tc, bool pair,
+                  bool sliced) {
+  if (pair) return make_pair_carve(nb, J, G, nquart, nT, threads, sliced).bytes();
   const bool f32 = precision == FP_PREC_MIXED;  // the double-float path has the FP64 path's shared memory
   Carve c = make_carve(nb, J, G, nquart, nT, threads, f32);
   const size_t b = c.bytes(f32 ? sizeof(Cx<float>) : sizeof(Cx<double>));
   return tc ? align128(b) + kTcBytes : b;
 }
 
-int max_ctas_per_sm(int precision, int nb, int nT, int threads, size_t smem, bool tc, bool pair) {
-  const void* k = rates_kernel_ptr(precision, nb, nT, tc, pair);
+int max_ctas_per_sm(int precision, int nb, int nT, int threads, size_t smem, bool tc, bool pair,
+                    bool sliced) {
+  const void* k = rates_kernel_ptr(precision, nb, nT, tc, pair, sliced);
   if (!k) return 0;
   if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
   int n = 0;
@@ -229,18 +264,15 @@ int make_selection(const fp_ctx* c, const fp_rates_opts& o, bool fold_allowed, S
   return FP_OK;
 }
 
-int plan_rates(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, size_t partial_budget, Plan* p,
-               std::string* err, bool mirror) {
+static int plan_form(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, size_t partial_budget, Plan* p,
+                     std::string* err, bool pair, bool sliced, bool mirror) {
   const int N = c->N, nb = c->nb;
   const bool tc = o.tensor_cores != 0;
   if (tc && (o.precision != FP_PREC_MIXED || nb != 6)) {
     *err = "tensor_cores needs the mixed precision and 6 branches";
     return FP_EINVAL;
   }
-  // The pair kernel identifies vertices whose legs are permuted, so it needs Phi4 to have that symmetry.  It is not
-  // built for the mixed path.
-  const bool pair = c->leg_symmetric && o.precision != FP_PREC_MIXED;
-  if (!rates_kernel_ptr(o.precision, nb, nT, tc, pair)) {
+  if (!rates_kernel_ptr(o.precision, nb, nT, tc, pair, sliced)) {
     *err = "unsupported number of branches";
     return FP_EINVAL;
   }
@@ -261,7 +293,7 @@ int plan_rates(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, size_t
     const size_t room = pair ? (pair_blocks_for(nb) == 1 ? 227 : 112) * 1024 : 110 * 1024;
     J = nb;
     while (J > 1 && (J * nb * nb > most ||
-                     smem_bytes(o.precision, nb, J, c->G, c->nquart, nT, pair ? (J * nb * nb + 31) / 32 * 32 : most, tc, pair) > room)) {
+                     smem_bytes(o.precision, nb, J, c->G, c->nquart, nT, pair ? (J * nb * nb + 31) / 32 * 32 : most, tc, pair, sliced) > room)) {
       int nj = J - 1;
       while (nj > 1 && nb % nj) --nj;
       J = nj;
@@ -296,6 +328,9 @@ int plan_rates(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, size_t
     mirror = cudaMemGetInfo(&mem_free, &mem_total) == cudaSuccess && mirror_bytes < mem_free / 2;
   }
   if (mirror && o.k1_tile <= 0 && t1_tuned <= 0) t1 = 1;
+  // the table U of the Psi prologue, where a call may take the memory for it (2 MB on diamond 3^3, 308 MB on 16^3)
+  const size_t u_bytes = (size_t)nq_sel * nb * c->nquart * 27 * sizeof(double2);
+  p->psi_u = pair && !partial_budget && u_bytes > 0 && u_bytes <= (size_t(512) << 20);
   if (o.k1_tile <= 0 && partial_budget && !mirror)
     while (t1 < N && part_bytes(t1) > partial_budget) t1 = t1 < 8 ? t1 + 1 : t1 + t1 / 4;
   if (t1 > N) t1 = N;
@@ -317,12 +352,12 @@ int plan_rates(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, size_t
     *err = "per-item partial sums do not fit the scratch";
     return FP_EINVAL;
   }
-  const size_t smem = smem_bytes(o.precision, nb, J, c->G, c->nquart, nT, threads, tc, pair);
+  const size_t smem = smem_bytes(o.precision, nb, J, c->G, c->nquart, nT, threads, tc, pair, sliced);
   if (smem > 227 * 1024) {
     *err = "tile does not fit in shared memory";
     return FP_EINVAL;
   }
-  const int per_sm = max_ctas_per_sm(o.precision, nb, nT, threads, smem, tc, pair);
+  const int per_sm = max_ctas_per_sm(o.precision, nb, nT, threads, smem, tc, pair, sliced);
   if (per_sm < 1) {
     *err = "kernel tile cannot be resident on an SM";
     return FP_EINVAL;
@@ -341,6 +376,8 @@ int plan_rates(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, size_t
   p->n_items = (long long)p->ntile * nq_sel * nchunk;
   p->smem = smem;
   p->pair = pair;
+  p->sliced = sliced;
+  p->operands = sliced;
   p->mirror = mirror;
   p->values = mirror ? mirror_values : p->n_items * J;
   long long ctas = (long long)nsm * per_sm;
@@ -354,6 +391,23 @@ int plan_rates(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, size_t
       sel.active_chunks += any ? 1 : 0;
     }
   return FP_OK;
+}
+
+int plan_rates(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, size_t partial_budget, Plan* p,
+               std::string* err, RateForm form) {
+  // The pair kernel identifies vertices whose legs are permuted, so it needs Phi4 to have that symmetry; where its
+  // tables do not fit, the ordered kernel runs.  The mixed path keeps the ordered kernel: its FP32 vertex rounds
+  // differently for each order of the legs, and exchanging them moved the rates by up to 2e-8 (its error is 5e-8).
+  if (form != kOrdered && c->leg_symmetric && o.precision != FP_PREC_MIXED) {
+    // the FP64 path's contraction in slices: 6 and 12 branches (with 3, K = 6 would leave most of a tile empty)
+    if (form != kPair && o.precision == FP_PREC_FP64 && c->unit_modes && c->nb >= 6) {
+      const int rc = plan_form(c, o, nT, sel, partial_budget, p, err, true, true, form == kPairMirror);
+      if (rc != FP_EINVAL) return rc;
+    }
+    const int rc = plan_form(c, o, nT, sel, partial_budget, p, err, true, false, form == kPairMirror);
+    if (rc != FP_EINVAL) return rc;
+  }
+  return plan_form(c, o, nT, sel, partial_budget, p, err, false, false, false);
 }
 
 void scratch_sizes(const fp_ctx* c, const Plan& p, int nT, size_t s[kScratchParts]) {
@@ -374,6 +428,8 @@ void scratch_sizes(const fp_ctx* c, const Plan& p, int nT, size_t s[kScratchPart
   s[13] = up256((size_t)81 * c->nquart * sizeof(float));
   s[14] = up256((size_t)c->L * sizeof(float2));
   s[15] = up256(3 * nm * nT * sizeof(float));
+  s[17] = p.psi_u ? up256((size_t)p.nq_sel * c->nb * c->nquart * 27 * sizeof(double2)) : 0;
+  s[16] = p.operands ? up256((size_t)c->N * operand_words(c->nb) * sizeof(unsigned)) : 0;
 }
 
 Scratch carve_scratch(unsigned char* b, const size_t sz[kScratchParts]) {
@@ -399,6 +455,8 @@ Scratch carve_scratch(unsigned char* b, const size_t sz[kScratchParts]) {
   sc.qfcf = reinterpret_cast<float*>(b + off[13]);
   sc.twf = reinterpret_cast<float2*>(b + off[14]);
   sc.wtf = reinterpret_cast<float*>(b + off[15]);
+  sc.operands = reinterpret_cast<unsigned*>(b + off[16]);
+  sc.psi_u = reinterpret_cast<double2*>(b + off[17]);
   return sc;
 }
 
@@ -469,6 +527,8 @@ int run_rates(fp_ctx* c, const fp_rates_opts& o, const Selection& sel, const Pla
   a.qfcf = sc.qfcf;
   a.twf = sc.twf;
   a.wtf = sc.wtf;
+  a.operands = sc.operands;
+  a.psi_u = p.psi_u ? sc.psi_u : nullptr;
   a.sb = sb;
   a.window = o.window;
   a.sigma_min = o.sigma_min;
@@ -503,7 +563,7 @@ int run_rates(fp_ctx* c, const fp_rates_opts& o, const Selection& sel, const Pla
   const double pref = unit_stride > 0
                           ? (double)unit_stride / ((double)N * (double)N)
                           : kPi * kHbar * kHbar * conv * conv * conv * conv / (8.0 * (double)N * (double)N);
-  const void* k = rates_kernel_ptr(o.precision, nb, nT, o.tensor_cores != 0, p.pair);
+  const void* k = rates_kernel_ptr(o.precision, nb, nT, o.tensor_cores != 0, p.pair, p.sliced);
   // the device part of a rate set: Bose weights, FP32 tables, cleared counters and output, the persistent
   // rate kernel and the reduction
   auto enqueue = [&]() -> cudaError_t {
@@ -521,6 +581,17 @@ int run_rates(fp_ctx* c, const fp_rates_opts& o, const Selection& sel, const Pla
     prep_kernel<<<4 * 152, 256, 0, s>>>(a, sc.omh, sc.oml, sc.velh, sc.vell, sc.evf, sc.qfcf, sc.twf, sc.wtf,
                                         want_f32);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if (a.psi_u && p.nq_sel > 0) {
+      psi_u_kernel<<<8 * 152, 256, 0, s>>>(a, sc.psi_u);
+      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    if (p.operands) {
+      if (nb == 6)
+        operand_kernel<6><<<4 * 152, 256, 0, s>>>(c->d_evec, N, sc.operands);
+      else
+        operand_kernel<12><<<4 * 152, 256, 0, s>>>(c->d_evec, N, sc.operands);
+      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
     if ((e = cudaMemsetAsync(sc.counters, 0, kCounters * sizeof(unsigned long long), s)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(d_out, 0, (size_t)nT * nm * sizeof(double), s)) != cudaSuccess) return e;
     if (p.n_items > 0) {
@@ -639,13 +710,14 @@ int phase4_sampled(fp_ctx* c, int nT, const double* T, double sb, int stride, do
   int rc = make_selection(c, o, false, &sel, err);  // q' on a stride is not symmetric under q -> -q
   if (rc) return rc;
   Plan p;
-  rc = plan_rates(c, o, nT, sel, 0, &p, err, false);
+  rc = plan_rates(c, o, nT, sel, 0, &p, err, kPairSliced);
   if (rc) return rc;
   // a q' tile of one stride: every item owns exactly one sampled q'
   p.t1 = stride;
   p.ntile = (c->N + stride - 1) / stride;
   p.n_items = (long long)p.ntile * p.nq_sel * p.nchunk;
   p.values = p.n_items * p.J;
+  p.psi_u = p.operands = false;  // no vertex
   if (p.ctas > p.n_items) p.ctas = (int)p.n_items;
   size_t sz[kScratchParts], total = 0;
   scratch_sizes(c, p, nT, sz);

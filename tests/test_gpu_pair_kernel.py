@@ -106,3 +106,31 @@ def test_force_constants_without_the_symmetry(precision):
         out, st = ctx.rates4(cr.temps, cr.scalebroad, precision=precision)
     _close(out.reshape(1, -1), ref)
     assert st["accepted"] == list(acc)
+
+
+@pytest.mark.parametrize("precision", [FP_PREC_FP64, FP_PREC_DOUBLE_FLOAT])
+@pytest.mark.parametrize("maker", [lambda: synth.diamond_si((3, 2, 2)), lambda: synth.licoo2((2, 1, 2))])
+def test_eigenvectors_of_any_norm(precision, maker):
+    """Mode tables whose eigenvectors are not of unit norm take the contraction that has no fixed-point scale."""
+    cr = maker()
+    w, e, v = oracle_modes(cr)
+    f = 2.0 ** np.arange(cr.nb) * 1.1  # the same at q and -q
+    e = e * f[None, :, None]
+    ref, acc = oracle.rates4(cr, w, e, v)
+    with Context.from_crystal(cr) as ctx:
+        ctx.set_modes(w, e, v)
+        out, st = ctx.rates4(cr.temps, cr.scalebroad, precision=precision)
+    _close(out.reshape(len(cr.temps), -1), ref)
+    assert st["accepted"] == list(acc)
+
+
+@pytest.mark.parametrize("scale", [1e-90, 1e-30, 3.0, 1e60])
+def test_force_constants_of_any_size(scale):
+    """The fixed-point scale of the contraction follows Phi4: the rates scale with its square."""
+    cr = synth.zincblende_bas((3, 2, 2))
+    w, e, v = oracle_modes(cr)
+    ref, _ = oracle.rates4(cr, w, e, v)
+    with Context.from_crystal(cr.scaled_fc4(scale)) as ctx:
+        ctx.set_modes(w, e, v)
+        out, _ = ctx.rates4(cr.temps, cr.scalebroad)
+    _close(out.reshape(1, -1) / scale ** 2, ref)

@@ -171,12 +171,14 @@ struct fp_ctx {
   int* d_pk_zero = nullptr;
   bool leg_symmetric = false;  // the quartet list obeys the transposition symmetry (Eq. TS)
   int* d_bzm = nullptr;  // [N][3] Brillouin-zone shifts (bz_shifts)
-  // third-order force constants (fp_set_fc3), grouped by atom triple
+  // third-order force constants (fp_set_fc3), by group (atoms j, k and D = Rj - Rk)
   bool have_fc3 = false;
-  int n3 = 0;
-  int* d_t3_start = nullptr;   // [natoms^3 + 1]
-  int* d_t3_cell = nullptr;    // [n3][6] Rj, Rk
+  int n3 = 0, G3 = 0;
+  int* d_t3_start = nullptr;   // [G3 + 1]
+  int* d_t3_meta = nullptr;    // [n3][4] atom i and Rk
   double* d_t3_fc = nullptr;   // [n3][27] Phi3 / sqrt(Mi Mj Mk)
+  int* d_g3_meta = nullptr;    // [G3][3] D
+  int* d_g3_start = nullptr;   // [natoms^2 + 1] groups by (j, k), D = 0 first
   // modes
   bool have_modes = false;
   bool unit_modes = false;  // eigenvectors of norm 1 within 1e-5

@@ -4,230 +4,346 @@
 //   W3(q, j; k1, j1; k2, j2) = sum_triplets sum_{abg} Phi3 / sqrt(M^3) e_a(q, j) e_b(k1, j1) conj(e_g(k2, j2))
 //                              exp(i (k1.R_j - k2.R_k))
 // is V+ of the partner q' = k1 and V- of the partner q' = -k1 (both with q'' = k2), so every (q, k1) pair
-// serves both processes.  One CTA per q walks k1 over the grid: it assembles the reciprocal force constants
-// Phi~[(i a)(j b)(k g)] for (k1, k2), contracts them with e(q), e(k1) and conj e(k2) (three nb^4 steps
-// through shared memory), and every thread then owns entries (j, j1, j2): the window test and Gaussian of
-// both processes in FP64 with the oracle's operation order (decisions are identical), Bose factors,
-// |W|^2, and a running sum in shared memory.  The rates of each j are summed over its entries in a fixed
-// order at the end, so results do not depend on scheduling.
+// serves both processes.  Time reversal gives the rates of -q (make_selection).
+//
+// One block owns a point q and a range of k1.  The phase is exp(-i q.R_k) exp(i k1.(R_j - R_k)), so the contraction with
+// e(q) is done once per block, Psi[j][group][beta gamma] over the triplets of equal atoms (j, k) and D = R_j - R_k; per
+// k1 the block forms A[j][(j b)(k g)] = sum_groups exp(i k1.D) Psi (nothing to do for D = 0), Y = A e(k1) and
+// W = Y conj e(k2).  Thread o owns the entry (j, j1, j2).  The window is tested in FP32 with a proven margin and decided
+// in FP64 in the operation order of the definition only inside it (as in fp_rates_kernel.cuh), and the accepted
+// (entry, process) pairs of a warp are compacted and evaluated 32 at a time with 1/sigma and the Bose factors from
+// tables per (j1, j2).  Sums run per entry, then over the entries of a j and over the k1 ranges in a fixed order.
+//
+// The FP64 pipe bounds this kernel.  Before, each (q, k1) took 1300 more FMAs for the assembly and e(q), an FP64 square
+// root and 30 more operations for each of its 432 window tests, and every q ran: diamond 8^3 20.8 ms, now 4.2 ms.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <map>
 #include <string>
+#include <tuple>
 #include <type_traits>
 #include <vector>
 
-#include "fp_internal.cuh"
+#include "fp_pair_kernel.cuh"
 
+namespace fp {
 namespace {
 
 struct Rates3Args {
-  int N, nb, nT, L, n3, natoms;
-  int grid[3], Lfac[3];
-  const double* omega;
-  const double2* evec;
-  const double* vel;
-  const double2* tw;
-  const int* t3_start;  // [natoms^3 + 1] triplets grouped by atom triple (i, j, k)
-  const int* t3_cell;   // [n3][6] Rj, Rk
-  const double* t3_fc;  // [n3][27] Phi3 / sqrt(Mi Mj Mk)
-  const double* bose;   // [nT][N nb] occupation numbers
-  const unsigned char* mask;
-  int q_begin, nq_sel;
-  double sb, window, sigma_min, dq, pref;
-  int dq_mode;
-  double rec[9];
-  double* rates;                 // [nT][N nb]
-  unsigned long long* counts;    // [2]
+  RatesArgs r;           // grid, modes, window and broadening fields (sigma_entry, sigma_entry_f32); qlist, mult
+  int n3, G;
+  const int* t3_meta;    // [n3][4] atom i and Rk, triplets by group
+  const double* t3_fc;   // [n3][27] Phi3 / sqrt(Mi Mj Mk)
+  const int* t3_start;   // [G + 1] triplets of a group (j, k, D = Rj - Rk)
+  const int* g3_meta;    // [G][3] D
+  const int* g3_start;   // [natoms^2 + 1] groups of (j, k), those with D = 0 first
+  const double* bose;    // [nT][N nb] occupation numbers
+  double2* psi;          // [nq_sel][nb][G][9]
+  int psi_shared;        // the block keeps its Psi in shared memory
+  int t0, nT_all;        // first temperature of this launch and their number in the call
+  int nch, kchunk;       // k1 ranges per q
+  double* partial;       // [nq_sel][nch][nb][nT_all]
+  unsigned long long* counts;  // [2] accepted + and -, weighted by the selected modes a row stands for
 };
-
-__device__ __forceinline__ int wrap3(int x, int n) {
-  int r = x % n;
-  return r < 0 ? r + n : r;
-}
-
-// sigma = sb |v' - v''| dq (dq_mode 0) or the per-axis form, in the oracle's operation order
-__device__ double sigma3(const Rates3Args& a, const double* v1, const double* v2) {
-  const double dx = __dsub_rn(v1[0], v2[0]), dy = __dsub_rn(v1[1], v2[1]), dz = __dsub_rn(v1[2], v2[2]);
-  if (a.dq_mode == 0) {
-    const double s = __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
-    return __dmul_rn(__dmul_rn(a.sb, sqrt(s)), a.dq);
-  }
-  double pa[3];
-  for (int d = 0; d < 3; ++d) {
-    const double* b = a.rec + 3 * d;
-    pa[d] = __ddiv_rn(__dadd_rn(__dadd_rn(__dmul_rn(dx, b[0]), __dmul_rn(dy, b[1])), __dmul_rn(dz, b[2])),
-                      (double)a.grid[d]);
-  }
-  const double s = __ddiv_rn(__dadd_rn(__dadd_rn(__dmul_rn(pa[0], pa[0]), __dmul_rn(pa[1], pa[1])), __dmul_rn(pa[2], pa[2])), 3.0);
-  return __dmul_rn(a.sb, sqrt(s));
-}
 
 __global__ void bose3_kernel(const double* omega, const double* T, int nT, long long nm, double* out) {
   const long long n = (long long)nT * nm;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const double w = omega[i % nm];
     const double t = T[i / nm];
-    out[i] = w > 0.0 ? 1.0 / expm1(fp::kHbar * w / (fp::kBoltzmann * t)) : 0.0;
+    out[i] = w > 0.0 ? 1.0 / expm1(kHbar * w / (kBoltzmann * t)) : 0.0;
   }
 }
 
+// Psi[qi][j][grp][beta gamma] = sum over the triplets of the group of exp(-i q.R_k) sum_alpha Phi3 e_alpha(q, j)
+__global__ void psi3_kernel(Rates3Args p) {
+  const RatesArgs& a = p.r;
+  const long long n = (long long)a.nq_sel * a.nb * p.G * 9;
+  for (long long o = blockIdx.x * (long long)blockDim.x + threadIdx.x; o < n; o += (long long)gridDim.x * blockDim.x) {
+    const int bg = (int)(o % 9), grp = (int)((o / 9) % p.G), j = (int)((o / (9LL * p.G)) % a.nb);
+    const int q = a.qlist[o / (9LL * p.G * a.nb)];
+    const int g[3] = {q / (a.grid[1] * a.grid[2]), (q / a.grid[2]) % a.grid[1], q % a.grid[2]};
+    const double2* e0 = a.evec + ((size_t)q * a.nb + j) * a.nb;
+    Cx<double> sum = cmk<double>(0, 0);
+    for (int Q = p.t3_start[grp]; Q < p.t3_start[grp + 1]; ++Q) {
+      const int* m = p.t3_meta + 4 * Q;
+      int e = 0;  // each term is below L, so e < 3 L
+      for (int d = 0; d < 3; ++d) e += a.Lfac[d] * wrapi(-g[d] * m[1 + d], a.grid[d]);
+      while (e >= a.L) e -= a.L;
+      Cx<double> s = cmk<double>(0, 0);
+      for (int al = 0; al < 3; ++al) {
+        const double f = p.t3_fc[27 * (size_t)Q + al * 9 + bg];
+        s.re = fma(f, e0[3 * m[0] + al].x, s.re);
+        s.im = fma(f, e0[3 * m[0] + al].y, s.im);
+      }
+      cfma(sum, ld_tw<double>(a, e), s);
+    }
+    p.psi[o] = make_double2(sum.re, sum.im);
+  }
+}
+
+__host__ __device__ constexpr int threads3(int nb) { return nb == 3 ? 32 : nb == 6 ? 224 : 256; }
+
+// shared memory in bytes
+struct Carve3 {
+  size_t Psi, A, Y, E1, E2, Tw, Acc, W0, W1, W2, V1, V2, Iv8, F, B, Val, ExpT, Vf, PM, Hf, Ent, Mult, total;
+};
+__host__ __device__ inline Carve3 make_carve3(int nb, int G, int nT, bool psi) {
+  Carve3 c;
+  const size_t nb2 = (size_t)nb * nb, nb3 = nb2 * nb, nw = threads3(nb) / 32;
+  size_t o = 0;
+  auto put = [&](size_t bytes) {
+    const size_t at = o;
+    o += (bytes + 15) & ~size_t(15);
+    return at;
+  };
+  c.Psi = put(psi ? (size_t)nb * G * 9 * 16 : 0);
+  c.A = put(nb3 * 16);
+  c.Y = put(nb3 * 16);
+  c.E1 = put(nb2 * 16);
+  c.E2 = put(nb2 * 16);
+  c.Tw = put((size_t)G * 16);
+  c.Acc = put(nb3 * nT * 8);
+  c.W0 = put((size_t)nb * 8);
+  c.W1 = put((size_t)nb * 8);
+  c.W2 = put((size_t)nb * 8);
+  c.V1 = put(3 * (size_t)nb * 8);
+  c.V2 = put(3 * (size_t)nb * 8);
+  c.Iv8 = put(2 * nb2 * 8);                 // 8/sigma or -1 (delta := 1), [process][j1][j2]
+  c.F = put(2 * nb2 * 8);                   // (1/sigma) / (sqrt(pi) w' w'')
+  c.B = put(2 * nb2 * nT * 8);              // Bose factors n' - n'' and (n' + n'' + 1) / 2
+  c.Val = put(nw * 64 * 8);
+  c.ExpT = put(kExpTab * 8);
+  c.Vf = put(12 * (size_t)nb * 4);          // two-float velocities of k1 and k2
+  c.PM = put(2 * nb2 * 8);                  // (P~, margin)
+  c.Hf = put(3 * (size_t)nb * 4);           // FP32 frequencies of q, k1, k2
+  c.Ent = put(nw * 64 * 2);
+  c.Mult = put((size_t)nb);
+  c.total = o;
+  return c;
+}
+
 template <int NB>
-__global__ void __launch_bounds__(256) rates3_kernel(Rates3Args a) {
-  constexpr int NB2 = NB * NB, NB3 = NB2 * NB, NA = NB / 3;
+__global__ void __launch_bounds__(threads3(NB), NB == 12 ? 1 : 2) rates3_kernel(Rates3Args p) {
+  constexpr int NB2 = NB * NB, NB3 = NB2 * NB, NA = NB / 3, kThreads = threads3(NB);
+  using C = Cx<double>;
   extern __shared__ __align__(16) unsigned char smem[];
-  double2* sPhi = reinterpret_cast<double2*>(smem);  // [a][b][c], then reused for Y[j][j1][c]
-  double2* sX = sPhi + NB3;                            // [j][b][c]
-  double2* sE0 = sX + NB3;                             // [j][a]
-  double2* sE1 = sE0 + NB2;
-  double2* sE2 = sE1 + NB2;
-  double2* sTw = sE2 + NB2;                            // [n3]
-  double* sAcc = reinterpret_cast<double*>(sTw + a.n3);  // [entry][t]
-  double* sW1 = sAcc + (size_t)NB3 * a.nT;               // omega(k1), omega(-k1), omega(k2)
-  double* sW1n = sW1 + NB;
-  double* sW2 = sW1n + NB;
-  double* sV1 = sW2 + NB;  // [3 NB] v(k1), v(-k1), v(k2)
-  double* sV1n = sV1 + 3 * NB;
-  double* sV2 = sV1n + 3 * NB;
-  const int tid = threadIdx.x, nthr = blockDim.x;
-  const int N = a.N, nT = a.nT;
-  const long long NM = (long long)N * NB;
-  const int q = a.q_begin + blockIdx.x;
+  const RatesArgs& a = p.r;
+  const int nT = a.nT, N = a.N, G = p.G;
+  const Carve3 cv = make_carve3(NB, G, nT, p.psi_shared != 0);
+  auto dbl = [&](size_t at) { return reinterpret_cast<double*>(smem + at); };
+  auto flt = [&](size_t at) { return reinterpret_cast<float*>(smem + at); };
+  C *sPsi = reinterpret_cast<C*>(smem + cv.Psi), *sA = reinterpret_cast<C*>(smem + cv.A), *sY = reinterpret_cast<C*>(smem + cv.Y);
+  C *sE1 = reinterpret_cast<C*>(smem + cv.E1), *sE2 = reinterpret_cast<C*>(smem + cv.E2);
+  C* sTw = reinterpret_cast<C*>(smem + cv.Tw);
+  double *sAcc = dbl(cv.Acc), *sW0 = dbl(cv.W0), *sW1 = dbl(cv.W1), *sW2 = dbl(cv.W2), *sV1 = dbl(cv.V1), *sV2 = dbl(cv.V2);
+  double *sIv8 = dbl(cv.Iv8), *sF = dbl(cv.F), *sB = dbl(cv.B), *sExpT = dbl(cv.ExpT);
+  float *sVf = flt(cv.Vf), *sH0 = flt(cv.Hf), *sH1 = sH0 + NB, *sH2 = sH1 + NB;
+  float2* sPM = reinterpret_cast<float2*>(smem + cv.PM);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  double* sVal = dbl(cv.Val) + warp * 64;
+  unsigned short* sEnt = reinterpret_cast<unsigned short*>(smem + cv.Ent) + warp * 64;
+  unsigned char* sMult = smem + cv.Mult;
+  const size_t NM = (size_t)N * NB;
+  const int qi = blockIdx.x / p.nch, ch = blockIdx.x % p.nch;
+  const int q = a.qlist[qi];
   const int g[3] = {q / (a.grid[1] * a.grid[2]), (q / a.grid[2]) % a.grid[1], q % a.grid[2]};
-  for (int o = tid; o < NB2; o += nthr) sE0[o] = a.evec[(size_t)q * NB2 + o];
-  for (int o = tid; o < NB3 * nT; o += nthr) sAcc[o] = 0.0;
+  const bool f32_sigma = a.dq_mode == 0;
+  const double inv_sbdq = 1.0 / (a.sb * a.dq);
+  const C* psi = reinterpret_cast<const C*>(p.psi) + (size_t)qi * NB * G * 9;
+  if (p.psi_shared) {
+    for (int o = tid; o < NB * G * 9; o += kThreads) sPsi[o] = psi[o];
+    psi = sPsi;
+  }
+  for (int o = tid; o < NB; o += kThreads) {
+    const double w = a.omega[(size_t)q * NB + o];
+    sW0[o] = w;
+    sH0[o] = __double2float_rn(w);
+    sMult[o] = w > 0.0 ? a.mult[(size_t)q * NB + o] : 0;
+  }
+  for (int o = tid; o < kExpTab; o += kThreads) sExpT[o] = exp(-(double)o * kExpH);
+  for (int o = tid; o < NB3 * nT; o += kThreads) sAcc[o] = 0.0;
   unsigned long long cplus = 0, cminus = 0;
-  __syncthreads();
-  for (int k1 = 0; k1 < N; ++k1) {
+  const int k_begin = ch * p.kchunk, k_end = min(N, k_begin + p.kchunk);
+  for (int k1 = k_begin; k1 < k_end; ++k1) {
     const int g1[3] = {k1 / (a.grid[1] * a.grid[2]), (k1 / a.grid[2]) % a.grid[1], k1 % a.grid[2]};
-    int g2[3], gn[3];
+    int g2[3];
     for (int d = 0; d < 3; ++d) {
-      g2[d] = wrap3(g[d] + g1[d], a.grid[d]);
-      gn[d] = wrap3(-g1[d], a.grid[d]);
+      g2[d] = g[d] + g1[d];
+      if (g2[d] >= a.grid[d]) g2[d] -= a.grid[d];
     }
     const int k2 = (g2[0] * a.grid[1] + g2[1]) * a.grid[2] + g2[2];
-    const int kn = (gn[0] * a.grid[1] + gn[1]) * a.grid[2] + gn[2];  // -k1, the partner of the - process
-    for (int o = tid; o < NB2; o += nthr) {
-      sE1[o] = a.evec[(size_t)k1 * NB2 + o];
-      sE2[o] = a.evec[(size_t)k2 * NB2 + o];
+    __syncthreads();  // Psi; at later k1 the last one's terms
+    for (int o = tid; o < NB2; o += kThreads) {
+      sE1[o] = ld_e<double>(a, (size_t)k1 * NB2 + o);
+      sE2[o] = ld_e<double>(a, (size_t)k2 * NB2 + o);
     }
-    for (int o = tid; o < NB; o += nthr) {
+    for (int o = tid; o < NB; o += kThreads) {
       sW1[o] = a.omega[(size_t)k1 * NB + o];
-      sW1n[o] = a.omega[(size_t)kn * NB + o];
       sW2[o] = a.omega[(size_t)k2 * NB + o];
+      sH1[o] = __double2float_rn(sW1[o]);
+      sH2[o] = __double2float_rn(sW2[o]);
     }
-    for (int o = tid; o < 3 * NB; o += nthr) {
-      sV1[o] = a.vel[(size_t)k1 * NB * 3 + o];
-      sV1n[o] = a.vel[(size_t)kn * NB * 3 + o];
-      sV2[o] = a.vel[(size_t)k2 * NB * 3 + o];
+    for (int o = tid; o < 3 * NB; o += kThreads) {
+      const double v1 = a.vel[(size_t)k1 * NB * 3 + o], v2 = a.vel[(size_t)k2 * NB * 3 + o];
+      sV1[o] = v1;
+      sV2[o] = v2;
+      const float h1 = __double2float_rn(v1), h2 = __double2float_rn(v2);
+      sVf[o] = h1;
+      sVf[3 * NB + o] = __double2float_rn(v1 - (double)h1);
+      sVf[6 * NB + o] = h2;
+      sVf[9 * NB + o] = __double2float_rn(v2 - (double)h2);
     }
-    for (int Q = tid; Q < a.n3; Q += nthr) {
-      const int* R = a.t3_cell + 6 * Q;
-      int e = 0;  // each term is below L, so e < 3 L
-      for (int d = 0; d < 3; ++d) e += a.Lfac[d] * wrap3(g1[d] * R[d] - g2[d] * R[3 + d], a.grid[d]);
+    for (int o = tid; o < G; o += kThreads) {
+      const int* D = p.g3_meta + 3 * o;
+      int e = 0;
+      for (int d = 0; d < 3; ++d) e += a.Lfac[d] * wrapi(g1[d] * D[d], a.grid[d]);
       while (e >= a.L) e -= a.L;
-      sTw[Q] = a.tw[e];
+      sTw[o] = ld_tw<double>(a, e);
     }
     __syncthreads();
-    // Phi~[(i al)(j be)(k ga)] = sum over the triplets of atoms (i, j, k) of Phi3 / sqrt(M^3) exp(i(k1.Rj - k2.Rk))
-    for (int o = tid; o < NB3; o += nthr) {
-      const int ab = o / NB, c = o % NB, aa = ab / NB, b = ab % NB;
-      const int t = (aa / 3 * NA + b / 3) * NA + c / 3;
-      const int comp = ((aa % 3) * 3 + b % 3) * 3 + c % 3;
-      double re = 0.0, im = 0.0;
-      for (int Q = a.t3_start[t]; Q < a.t3_start[t + 1]; ++Q) {
-        const double f = a.t3_fc[27 * (size_t)Q + comp];
-        re = fma(f, sTw[Q].x, re);
-        im = fma(f, sTw[Q].y, im);
+    for (int o = tid; o < NB3; o += kThreads) {
+      const int j = o / NB2, b = (o / NB) % NB, c = o % NB, jk = b / 3 * NA + c / 3, bg = (b % 3) * 3 + c % 3;
+      C s = cmk<double>(0, 0);
+      int gi = p.g3_start[jk];
+      const int g_end = p.g3_start[jk + 1];
+      if (gi < g_end && p.g3_meta[3 * gi] == 0 && p.g3_meta[3 * gi + 1] == 0 && p.g3_meta[3 * gi + 2] == 0) {
+        s = psi[(j * G + gi) * 9 + bg];
+        ++gi;
       }
-      sPhi[o] = make_double2(re, im);
+      for (; gi < g_end; ++gi) cfma(s, sTw[gi], psi[(j * G + gi) * 9 + bg]);
+      sA[o] = s;
     }
-    __syncthreads();
-    // X[j][b][c] = sum_a e_a(q, j) Phi~[a][b][c]
-    for (int o = tid; o < NB3; o += nthr) {
-      const int j = o / NB2, bc = o % NB2;
-      double re = 0.0, im = 0.0;
-#pragma unroll
-      for (int aa = 0; aa < NB; ++aa) {
-        const double2 e = sE0[j * NB + aa], p = sPhi[aa * NB2 + bc];
-        re = fma(e.x, p.x, fma(-e.y, p.y, re));
-        im = fma(e.x, p.y, fma(e.y, p.x, im));
-      }
-      sX[o] = make_double2(re, im);
-    }
-    __syncthreads();
-    // Y[j][j1][c] = sum_b e_b(k1, j1) X[j][b][c]  (into sPhi)
-    for (int o = tid; o < NB3; o += nthr) {
-      const int j = o / NB2, j1 = (o / NB) % NB, c = o % NB;
-      double re = 0.0, im = 0.0;
-#pragma unroll
-      for (int b = 0; b < NB; ++b) {
-        const double2 e = sE1[j1 * NB + b], x = sX[(j * NB + b) * NB + c];
-        re = fma(e.x, x.x, fma(-e.y, x.y, re));
-        im = fma(e.x, x.y, fma(e.y, x.x, im));
-      }
-      sPhi[o] = make_double2(re, im);
-    }
-    __syncthreads();
-    // W[j][j1][j2] = sum_c conj(e_c(k2, j2)) Y[j][j1][c]; then both processes of the entry
-    for (int o = tid; o < NB3; o += nthr) {
-      const int j = o / NB2, j1 = (o / NB) % NB, j2 = o % NB;
-      const long long m0 = (long long)q * NB + j;
-      const double w = a.omega[m0];
-      if (w == 0.0 || (a.mask && !a.mask[m0])) continue;
-      const double w2 = sW2[j2];
-      if (w2 == 0.0) continue;
-      double re = 0.0, im = 0.0;
-#pragma unroll
-      for (int c = 0; c < NB; ++c) {
-        const double2 e = sE2[j2 * NB + c], y = sPhi[(j * NB + j1) * NB + c];
-        re = fma(e.x, y.x, fma(e.y, y.y, re));
-        im = fma(e.x, y.y, fma(-e.y, y.x, im));
-      }
-      const double W2 = re * re + im * im;
-      for (int pr = 0; pr < 2; ++pr) {
-        // + : partner k1; - : partner -k1 (same branch index; frequencies and velocities from its own entry)
-        const double w1 = pr == 0 ? sW1[j1] : sW1n[j1];
-        if (w1 == 0.0) continue;
-        const double dw = __dsub_rn(pr == 0 ? __dadd_rn(w, w1) : __dsub_rn(w, w1), w2);
-        const double sigma = sigma3(a, (pr == 0 ? sV1 : sV1n) + 3 * j1, sV2 + 3 * j2);
-        const double sw = sigma < a.sigma_min ? a.sigma_min : sigma;
-        if (!(fabs(dw) <= __dmul_rn(a.window, sw))) continue;
-        const double delta = sigma < a.sigma_min ? 1.0 : exp(-(dw * dw) / (sigma * sigma)) / (sqrt(fp::kPi) * sigma);
-        const double base = W2 * delta / (w * w1 * w2);
-        const long long m1 = (long long)(pr == 0 ? k1 : kn) * NB + j1, m2 = (long long)k2 * NB + j2;
-        for (int t = 0; t < nT; ++t) {
-          const double n1 = a.bose[t * NM + m1], n2 = a.bose[t * NM + m2];
-          sAcc[(size_t)o * nT + t] += pr == 0 ? (n1 - n2) * base : 0.5 * (n1 + n2 + 1.0) * base;
+    // tables per (process, j1, j2): + v(k1) - v(k2), - -v(k1) - v(k2)
+    for (int o = kThreads - 1 - tid; o < 2 * NB2; o += kThreads) {
+      const int pr = o / NB2, j1 = (o / NB) % NB, j2 = o % NB;
+      double iv = -1.0;
+      if (f32_sigma) {
+        float inv;
+        sigma_entry_f32(a, sVf + 3 * j1, sVf + 3 * NB + 3 * j1, pr ? -1.f : 1.f, sVf + 6 * NB + 3 * j2,
+                        sVf + 9 * NB + 3 * j2, sV1 + 3 * j1, sV2 + 3 * j2, sPM + o, &inv);
+        if (inv >= 0.f) {
+          const double sg = pr ? -1.0 : 1.0;
+          const double dx = sg * sV1[3 * j1] - sV2[3 * j2], dy = sg * sV1[3 * j1 + 1] - sV2[3 * j2 + 1],
+                       dz = sg * sV1[3 * j1 + 2] - sV2[3 * j2 + 2];
+          iv = rsqrt(fma(dx, dx, fma(dy, dy, dz * dz))) * inv_sbdq;
         }
-        if (pr == 0)
-          ++cplus;
-        else
-          ++cminus;
+      } else {
+        double ex[2];
+        float inv;
+        sigma_entry(a, sV1 + 3 * j1, pr ? -1.0 : 1.0, sV2 + 3 * j2, ex);
+        sigma_f_from_exact(ex, sPM + o, &inv);
+        iv = ex[1];
       }
+      sIv8[o] = iv >= 0.0 ? 8.0 * iv : -1.0;
+      sF[o] = (iv >= 0.0 ? iv * kInvSqrtPi : 1.0) / (sW1[j1] * sW2[j2]);  // not used at zero frequency
+    }
+    for (int o = tid; o < 2 * NB2 * nT; o += kThreads) {
+      const int t = o / (2 * NB2), pr = (o / NB2) % 2, j1 = (o / NB) % NB, j2 = o % NB;
+      const double *n = p.bose + (size_t)(p.t0 + t) * NM, n1 = n[(size_t)k1 * NB + j1], n2 = n[(size_t)k2 * NB + j2];
+      sB[o] = pr == 0 ? n1 - n2 : 0.5 * (n1 + n2 + 1.0);
     }
     __syncthreads();
+    for (int o = tid; o < NB3; o += kThreads) {
+      const int j = o / NB2, j1 = (o / NB) % NB, c = o % NB;
+      C s = cmk<double>(0, 0);
+#pragma unroll
+      for (int b = 0; b < NB; ++b) cfma(s, sE1[j1 * NB + b], sA[(j * NB + b) * NB + c]);
+      sY[o] = s;
+    }
+    __syncthreads();
+    for (int o0 = warp * 32; o0 < NB3; o0 += kThreads) {
+      const int o = o0 + lane;
+      const int j = o / NB2, j1 = (o / NB) % NB, j2 = o % NB;
+      // accepted processes of this entry: bit 0 (+), bit 1 (-)
+      unsigned acc = 0;
+      const unsigned mult = o < NB3 ? sMult[j] : 0u;
+      if (mult && sH1[j1] != 0.f && sH2[j2] != 0.f) {
+        const float h = sH0[j], h1 = sH1[j1], h2 = sH2[j2], sS = kRelS * ((h + h1) + h2);
+#pragma unroll
+        for (int pr = 0; pr < 2; ++pr) {
+          const float2 pm = sPM[pr * NB2 + j1 * NB + j2];
+          const float d = fabsf((pr ? h - h1 : h + h1) - h2), M = sS + pm.y;
+          if (d < pm.x - M) {
+            acc |= 1u << pr;
+          } else if (d <= pm.x + M) {  // inside the rounding of the prefilter: decided in FP64
+            double ex[2];
+            sigma_entry(a, sV1 + 3 * j1, pr ? -1.0 : 1.0, sV2 + 3 * j2, ex);
+            const double w = sW0[j], w1 = sW1[j1];
+            if (fabs(__dsub_rn(pr ? __dsub_rn(w, w1) : __dadd_rn(w, w1), sW2[j2])) <= ex[0]) acc |= 1u << pr;
+          }
+        }
+      }
+      cplus += (acc & 1u) * mult;
+      cminus += (acc >> 1) * mult;
+      const unsigned b0 = __ballot_sync(0xffffffffu, acc & 1u), b1 = __ballot_sync(0xffffffffu, acc & 2u);
+      const unsigned below = (1u << lane) - 1u;
+      const int n0 = __popc(b0), total = n0 + __popc(b1);
+      const int p0 = __popc(b0 & below), p1 = n0 + __popc(b1 & below);
+      if (acc & 1u) sEnt[p0] = (unsigned short)lane;
+      if (acc & 2u) sEnt[p1] = (unsigned short)(lane | 32);
+      __syncwarp();
+      for (int i = lane; i < total; i += 32) {
+        const unsigned en = sEnt[i];
+        const int oe = o0 + (int)(en & 31u), pr = (int)(en >> 5);
+        const int ej = oe / NB2, e1 = (oe / NB) % NB, e2 = oe % NB, e = pr * NB2 + e1 * NB + e2;
+        C W = cmk<double>(0, 0);
+#pragma unroll
+        for (int c = 0; c < NB; ++c) cfma_conj(W, sY[(ej * NB + e1) * NB + c], sE2[e2 * NB + c]);
+        const double w = sW0[ej], w1 = sW1[e1];
+        const double dw = __dsub_rn(pr ? __dsub_rn(w, w1) : __dadd_rn(w, w1), sW2[e2]);
+        double v = (W.re * W.re + W.im * W.im) * sF[e];
+        const double iv8 = sIv8[e];
+        if (__double2hiint(iv8) >= 0) {
+          const double x8 = dw * iv8;
+          v *= pair_exp_neg64(x8 * x8, sExpT);
+        }
+        sVal[i] = v;
+      }
+      __syncwarp();
+      if (acc) {
+        const double v0 = (acc & 1u) ? sVal[p0] : 0.0, v1 = (acc & 2u) ? sVal[p1] : 0.0;
+        for (int t = 0; t < nT; ++t) {
+          const double* B = sB + 2 * t * NB2 + j1 * NB + j2;
+          sAcc[(size_t)o * nT + t] = fma(v0, B[0], fma(v1, B[NB2], sAcc[(size_t)o * nT + t]));
+        }
+      }
+      __syncwarp();
+    }
   }
-  // rate of (q, j): its entries (j, j1, j2) in order
-  for (int o = tid; o < NB * nT; o += nthr) {
+  __syncthreads();
+  for (int o = tid; o < NB * nT; o += kThreads) {
     const int j = o / nT, t = o % nT;
     double s = 0.0;
     for (int e = j * NB2; e < (j + 1) * NB2; ++e) s += sAcc[(size_t)e * nT + t];
-    a.rates[t * NM + (long long)q * NB + j] = a.pref * s;
+    p.partial[((size_t)blockIdx.x * NB + j) * p.nT_all + p.t0 + t] = s;
   }
   for (int off = 16; off > 0; off >>= 1) {
     cplus += __shfl_down_sync(0xffffffffu, cplus, off);
     cminus += __shfl_down_sync(0xffffffffu, cminus, off);
   }
-  if ((tid & 31) == 0) {
-    if (cplus) atomicAdd(a.counts, cplus);
-    if (cminus) atomicAdd(a.counts + 1, cminus);
+  if (lane == 0 && p.t0 == 0) {
+    if (cplus) atomicAdd(p.counts, cplus);
+    if (cminus) atomicAdd(p.counts + 1, cminus);
   }
 }
 
-size_t smem3_bytes(int nb, int n3, int nT) {
-  const size_t nb3 = (size_t)nb * nb * nb, nb2 = (size_t)nb * nb;
-  return (2 * nb3 + 3 * nb2 + n3) * sizeof(double2) + (nb3 * nT + 3 * nb + 9 * nb) * sizeof(double);
+// rates[t][q][j] = pref / w sum_ranges partial, in order, for the selected modes; the others stay zero
+__global__ void reduce3_kernel(Rates3Args p, double pref, double* rates) {
+  const RatesArgs& a = p.r;
+  const long long n = (long long)p.nT_all * a.q_out_n * a.nb;
+  const long long o = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (o >= n) return;
+  const int j = (int)(o % a.nb);
+  const int q = a.q_out_begin + (int)((o / a.nb) % a.q_out_n);
+  const int t = (int)(o / ((long long)a.nb * a.q_out_n));
+  const double w = a.omega[(size_t)q * a.nb + j];
+  if (!a.sel[(size_t)q * a.nb + j] || !(w > 0.0)) return;
+  const double* s = p.partial + (((size_t)a.qpos[q] * p.nch) * a.nb + j) * p.nT_all + t;
+  double sum = 0.0;
+  for (int ch = 0; ch < p.nch; ++ch) sum += s[(size_t)ch * a.nb * p.nT_all];
+  rates[((size_t)t * a.N + q) * a.nb + j] = pref * sum / w;
 }
 
 const void* rates3_ptr(int nb) {
@@ -245,6 +361,9 @@ int fail3(fp_ctx* c, int code, const std::string& msg) {
 }
 
 }  // namespace
+}  // namespace fp
+
+using namespace fp;
 
 #define R3_CUDA(call)                                                                              \
   do {                                                                                             \
@@ -258,27 +377,34 @@ extern "C" int fp_set_fc3(fp_ctx* c, int n_fc3, const fp_fc3* fc3) {
   if (!c) return FP_EINVAL;
   if (n_fc3 < 0 || (n_fc3 > 0 && !fc3)) return fail3(c, FP_EINVAL, "fp_set_fc3: bad triplet list");
   const int na = c->natoms;
-  // group the triplets by atom triple; store Phi3 / sqrt(Mi Mj Mk) and the cells
-  std::vector<std::vector<int>> by(na * na * na);
+  // triplets by group (j, k, D = Rj - Rk), groups by (j, k) with D = 0 first; Phi3 / sqrt(Mi Mj Mk)
+  std::map<std::tuple<int, int, int, int, int>, std::vector<int>> groups;
   for (int b = 0; b < n_fc3; ++b) {
     const fp_fc3& f = fc3[b];
     if (f.i < 0 || f.j < 0 || f.k < 0 || f.i >= na || f.j >= na || f.k >= na)
       return fail3(c, FP_EINVAL, "fp_set_fc3: atom index out of range");
-    by[(f.i * na + f.j) * na + f.k].push_back(b);
+    const int D[3] = {f.Rj[0] - f.Rk[0], f.Rj[1] - f.Rk[1], f.Rj[2] - f.Rk[2]};
+    groups[std::make_tuple(f.j * na + f.k, D[0] || D[1] || D[2] ? 1 : 0, D[0], D[1], D[2])].push_back(b);
   }
-  std::vector<int> start(na * na * na + 1, 0), cell;
+  std::vector<int> start(1, 0), tmeta, meta, gstart(na * na + 1, 0);
   std::vector<double> val;
-  for (size_t t = 0; t < by.size(); ++t) {
-    start[t + 1] = start[t] + (int)by[t].size();
-    for (int b : by[t]) {
+  for (const auto& kv : groups) {
+    gstart[std::get<0>(kv.first) + 1]++;
+    meta.push_back(std::get<2>(kv.first));
+    meta.push_back(std::get<3>(kv.first));
+    meta.push_back(std::get<4>(kv.first));
+    for (int b : kv.second) {
       const fp_fc3& f = fc3[b];
-      for (int d = 0; d < 3; ++d) cell.push_back(f.Rj[d]);
-      for (int d = 0; d < 3; ++d) cell.push_back(f.Rk[d]);
+      tmeta.push_back(f.i);
+      for (int d = 0; d < 3; ++d) tmeta.push_back(f.Rk[d]);
       const double m = std::sqrt(c->mass[f.i] * c->mass[f.j] * c->mass[f.k]);
       for (int x = 0; x < 27; ++x) val.push_back(f.fc[x] / m);
     }
+    start.push_back((int)tmeta.size() / 4);
   }
+  for (int k = 0; k < na * na; ++k) gstart[k + 1] += gstart[k];
   R3_CUDA(cudaSetDevice(c->device));
+  c->have_fc3 = false;
   auto put = [&](auto*& dst, const auto& src) -> cudaError_t {
     using T = typename std::remove_reference<decltype(*dst)>::type;
     if (dst) cudaFree(dst);
@@ -288,8 +414,11 @@ extern "C" int fp_set_fc3(fp_ctx* c, int n_fc3, const fp_fc3* fc3) {
     return cudaMemcpy(dst, src.data(), src.size() * sizeof(T), cudaMemcpyHostToDevice);
   };
   R3_CUDA(put(c->d_t3_start, start));
-  R3_CUDA(put(c->d_t3_cell, cell));
+  R3_CUDA(put(c->d_t3_meta, tmeta));
   R3_CUDA(put(c->d_t3_fc, val));
+  R3_CUDA(put(c->d_g3_meta, meta));
+  R3_CUDA(put(c->d_g3_start, gstart));
+  c->G3 = (int)groups.size();
   c->n3 = n_fc3;
   c->have_fc3 = true;
   return FP_OK;
@@ -318,85 +447,129 @@ extern "C" int fp_rates3(fp_ctx* c, int nT, const double* T, double scalebroad, 
   const void* k = rates3_ptr(nb);
   if (!k) return fail3(c, FP_EINVAL, "fp_rates3: nb must be 3, 6 or 12");
   const size_t nm = (size_t)N * nb;
-  const size_t smem = smem3_bytes(nb, c->n3, nT);
-  if (smem > 227 * 1024) return fail3(c, FP_EINVAL, "fp_rates3: tables do not fit in shared memory");
+  // Psi in shared memory while two blocks fit an SM (one with twelve branches), else read from the table; temperatures
+  // in as many launches as their sums per entry need
+  const size_t most = 227 * 1024;
+  int nTb = nT;
+  while (nTb > 1 && make_carve3(nb, c->G3, nTb, false).total > most) --nTb;
+  const bool psi_shared = make_carve3(nb, c->G3, nTb, true).total <= (nb == 12 ? most : most / 2);
+  const size_t smem = make_carve3(nb, c->G3, nTb, psi_shared).total;
+  if (smem > most) return fail3(c, FP_EINVAL, "fp_rates3: tables do not fit in shared memory");
   R3_CUDA(cudaSetDevice(c->device));
   cudaStream_t s = c->stream;
-  // working memory: T, occupation table, mask, counts, rates
-  double *dT = nullptr, *dn = nullptr, *dr = nullptr;
-  unsigned char* dm = nullptr;
-  unsigned long long* dc = nullptr;
-  auto cleanup = [&]() {
-    cudaFree(dT);
-    cudaFree(dn);
-    cudaFree(dr);
-    cudaFree(dm);
-    cudaFree(dc);
-  };
-  cudaError_t e = cudaSuccess;
-  if ((e = cudaMalloc(&dT, nT * sizeof(double))) != cudaSuccess || (e = cudaMalloc(&dn, nT * nm * sizeof(double))) ||
-      (e = cudaMalloc(&dr, nT * nm * sizeof(double))) || (e = cudaMalloc(&dc, 2 * sizeof(unsigned long long))) ||
-      (o.mode_mask && (e = cudaMalloc(&dm, nm)))) {
-    cleanup();
-    return fail3(c, e == cudaErrorMemoryAllocation ? FP_ENOMEM : FP_ECUDA, std::string("fp_rates3: ") + cudaGetErrorString(e));
+  // one point of each pair {q, -q}; the other options of `o` do not apply
+  fp_rates_opts so;
+  fp_default_opts(&so);
+  so.mode_mask = o.mode_mask;
+  so.q_begin = o.q_begin;
+  so.q_end = o.q_end;
+  Selection sel;
+  std::string err;
+  int rc = make_selection(c, so, true, &sel, &err);
+  if (rc) return fail3(c, rc, "fp_rates3: " + err);
+  const int nq = (int)sel.qlist.size();
+  // k1 ranges: enough blocks to fill the SMs about eight times over, so that the last wave costs little
+  int nsm = 0;
+  R3_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device));
+  int nch = nq > 0 ? (nsm * 16 + nq - 1) / nq : 1;
+  nch = std::max(1, std::min(nch, (N + 15) / 16));
+  const int kchunk = (N + nch - 1) / nch;
+  nch = (N + kchunk - 1) / kchunk;
+  // working memory, kept in the context: T, occupation table, counts, partial sums, rates, selection, Psi
+  const size_t part = std::max<size_t>(1, (size_t)nq * nch * nb * nT);
+  const size_t sizes[] = {nT * sizeof(double), nT * nm * sizeof(double), 2 * sizeof(unsigned long long), part * sizeof(double),
+                          nT * nm * sizeof(double), nm, nm, (size_t)N * sizeof(int), (size_t)N * sizeof(int),
+                          std::max<size_t>(1, (size_t)nq * nb * c->G3 * 9) * sizeof(double2)};
+  size_t off[11] = {0};
+  for (int i = 0; i < 10; ++i) off[i + 1] = off[i] + ((sizes[i] + 255) & ~size_t(255));
+  if (c->scratch_cap < off[10]) {
+    if (c->d_scratch) cudaFree(c->d_scratch);
+    c->d_scratch = nullptr;
+    c->scratch_cap = 0;
+    R3_CUDA(cudaMalloc(reinterpret_cast<void**>(&c->d_scratch), off[10]));
+    c->scratch_cap = off[10];
   }
+  unsigned char* base = c->d_scratch;
+  double *dT = reinterpret_cast<double*>(base), *dn = reinterpret_cast<double*>(base + off[1]);
+  unsigned long long* dc = reinterpret_cast<unsigned long long*>(base + off[2]);
+  double* dr = reinterpret_cast<double*>(base + off[4]);
   Rates3Args a;
   std::memset(&a, 0, sizeof(a));
-  a.N = N;
-  a.nb = nb;
-  a.nT = nT;
-  a.L = c->L;
-  a.n3 = c->n3;
-  a.natoms = c->natoms;
+  RatesArgs& r = a.r;
+  r.N = N;
+  r.nb = nb;
+  r.natoms = c->natoms;
+  r.nT = nT;
+  r.L = c->L;
   for (int d = 0; d < 3; ++d) {
-    a.grid[d] = c->grid[d];
-    a.Lfac[d] = c->L / c->grid[d];
+    r.grid[d] = c->grid[d];
+    r.Lfac[d] = c->L / c->grid[d];
   }
-  a.omega = c->d_omega;
-  a.evec = c->d_evec;
-  a.vel = c->d_vel;
-  a.tw = c->d_tw;
-  a.t3_start = c->d_t3_start;
-  a.t3_cell = c->d_t3_cell;
-  a.t3_fc = c->d_t3_fc;
-  a.bose = dn;
-  a.mask = dm;
-  a.q_begin = o.q_begin;
-  a.nq_sel = q_end - o.q_begin;
-  a.sb = scalebroad;
-  a.window = o.window;
-  a.sigma_min = o.sigma_min;
+  r.omega = c->d_omega;
+  r.evec = c->d_evec;
+  r.vel = c->d_vel;
+  r.tw = c->d_tw;
+  r.sb = scalebroad;
+  r.window = o.window;
+  r.sigma_min = o.sigma_min;
   const double* B = c->rec;
   const double detB = B[0] * (B[4] * B[8] - B[5] * B[7]) - B[1] * (B[3] * B[8] - B[5] * B[6]) +
                       B[2] * (B[3] * B[7] - B[4] * B[6]);
-  a.dq = std::cbrt(std::fabs(detB) / (double)N);
-  a.dq_mode = o.dq_mode;
-  for (int i = 0; i < 9; ++i) a.rec[i] = B[i];
-  a.pref = fp::kPi * fp::kHbar * fp::kConv * fp::kConv * fp::kConv / (4.0 * (double)N);
-  a.rates = dr;
+  r.dq = std::cbrt(std::fabs(detB) / (double)N);
+  r.dq_mode = o.dq_mode;
+  for (int i = 0; i < 9; ++i) r.rec[i] = B[i];
+  r.mult = base + off[5];
+  r.sel = base + off[6];
+  r.qlist = reinterpret_cast<int*>(base + off[7]);
+  r.qpos = reinterpret_cast<int*>(base + off[8]);
+  r.q_out_begin = sel.q_out_begin;
+  r.q_out_n = sel.q_out_end - sel.q_out_begin;
+  r.nq_sel = nq;
+  a.n3 = c->n3;
+  a.G = c->G3;
+  a.t3_start = c->d_t3_start;
+  a.t3_meta = c->d_t3_meta;
+  a.t3_fc = c->d_t3_fc;
+  a.psi = reinterpret_cast<double2*>(base + off[9]);
+  a.psi_shared = psi_shared ? 1 : 0;
+  a.nT_all = nT;
+  a.g3_meta = c->d_g3_meta;
+  a.g3_start = c->d_g3_start;
+  a.bose = dn;
+  a.nch = nch;
+  a.kchunk = kchunk;
+  a.partial = reinterpret_cast<double*>(base + off[3]);
   a.counts = dc;
-  bool ok = cudaMemcpyAsync(dT, T, nT * sizeof(double), cudaMemcpyHostToDevice, s) == cudaSuccess &&
-            (!dm || cudaMemcpyAsync(dm, o.mode_mask, nm, cudaMemcpyHostToDevice, s) == cudaSuccess) &&
-            cudaMemsetAsync(dr, 0, nT * nm * sizeof(double), s) == cudaSuccess &&
-            cudaMemsetAsync(dc, 0, 2 * sizeof(unsigned long long), s) == cudaSuccess &&
-            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess &&
-            cudaEventRecord(c->ev0, s) == cudaSuccess;
-  if (ok) {
-    bose3_kernel<<<256, 256, 0, s>>>(c->d_omega, dT, nT, (long long)nm, dn);
-    void* args[] = {&a};
-    ok = cudaGetLastError() == cudaSuccess &&
-         (a.nq_sel == 0 || cudaLaunchKernel(k, dim3(a.nq_sel), dim3(256), args, smem, s) == cudaSuccess) &&
-         cudaEventRecord(c->ev1, s) == cudaSuccess;
+  const double pref = kPi * kHbar * kConv * kConv * kConv / (4.0 * (double)N);
+  R3_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  R3_CUDA(cudaMemcpyAsync(dT, T, nT * sizeof(double), cudaMemcpyHostToDevice, s));
+  R3_CUDA(cudaMemcpyAsync(base + off[5], sel.mult.data(), nm, cudaMemcpyHostToDevice, s));
+  R3_CUDA(cudaMemcpyAsync(base + off[6], sel.sel.data(), nm, cudaMemcpyHostToDevice, s));
+  if (nq > 0) R3_CUDA(cudaMemcpyAsync(base + off[7], sel.qlist.data(), nq * sizeof(int), cudaMemcpyHostToDevice, s));
+  R3_CUDA(cudaMemcpyAsync(base + off[8], sel.qpos.data(), (size_t)N * sizeof(int), cudaMemcpyHostToDevice, s));
+  R3_CUDA(cudaMemsetAsync(dr, 0, nT * nm * sizeof(double), s));
+  R3_CUDA(cudaMemsetAsync(dc, 0, 2 * sizeof(unsigned long long), s));
+  R3_CUDA(cudaEventRecord(c->ev0, s));
+  bose3_kernel<<<256, 256, 0, s>>>(c->d_omega, dT, nT, (long long)nm, dn);
+  R3_CUDA(cudaGetLastError());
+  if (nq > 0) {
+    psi3_kernel<<<4 * nsm, 256, 0, s>>>(a);
+    R3_CUDA(cudaGetLastError());
+    for (int t0 = 0; t0 < nT; t0 += nTb) {
+      a.t0 = t0;
+      r.nT = std::min(nTb, nT - t0);
+      void* args[] = {&a};
+      R3_CUDA(cudaLaunchKernel(k, dim3(nq * nch), dim3(threads3(nb)), args, smem, s));
+    }
+    const long long n = (long long)nT * r.q_out_n * nb;
+    reduce3_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(a, pref, dr);
+    R3_CUDA(cudaGetLastError());
   }
+  R3_CUDA(cudaEventRecord(c->ev1, s));
   unsigned long long cnt[2] = {0, 0};
-  ok = ok && cudaMemcpyAsync(rates, dr, nT * nm * sizeof(double), cudaMemcpyDeviceToHost, s) == cudaSuccess &&
-       cudaMemcpyAsync(cnt, dc, sizeof(cnt), cudaMemcpyDeviceToHost, s) == cudaSuccess &&
-       cudaStreamSynchronize(s) == cudaSuccess;
-  if (!ok) {
-    const cudaError_t le = cudaGetLastError();
-    cleanup();
-    return fail3(c, FP_ECUDA, std::string("fp_rates3: ") + cudaGetErrorString(le));
-  }
+  R3_CUDA(cudaMemcpyAsync(rates, dr, nT * nm * sizeof(double), cudaMemcpyDeviceToHost, s));
+  R3_CUDA(cudaMemcpyAsync(cnt, dc, sizeof(cnt), cudaMemcpyDeviceToHost, s));
+  R3_CUDA(cudaStreamSynchronize(s));
   if (stats) {
     std::memset(stats, 0, sizeof(*stats));
     double nsel = 0;
@@ -405,18 +578,18 @@ extern "C" int fp_rates3(fp_ctx* c, int nT, const double* T, double scalebroad, 
     stats->candidates = 2.0 * nsel * (double)N * nb * nb;
     stats->accepted[0] = (double)cnt[0];
     stats->accepted[1] = (double)cnt[1];
-    // per (q, k1): the reciprocal force constants (27 n3 real x complex) and three nb^4 contractions
-    stats->flops = (double)a.nq_sel * N * (4.0 * 27.0 * c->n3 + 3.0 * 8.0 * nb * nb * nb * nb);
+    // per evaluated (q, k1): the assembly over the groups (9 nb G) and two nb^4 contractions
+    stats->flops = (double)nq * N * 8.0 * (9.0 * nb * c->G3 + 2.0 * nb * nb * nb * nb);
     float ms = 0.f;
     cudaEventElapsedTime(&ms, c->ev0, c->ev1);
     stats->ms = ms;
-    stats->tile[2] = 256;
-    stats->tile[3] = a.nq_sel;
+    stats->tile[2] = threads3(nb);
+    stats->tile[3] = nq * nch;
   }
-  cleanup();
   return FP_OK;
 }
 
+namespace fp {
 namespace {
 
 // RTA thermal conductivity (the tensor the paper's rates feed, Sec. 2.1): kappa_ab(T) = k_B / (N V)
@@ -448,6 +621,7 @@ __global__ void kappa_kernel(const double* omega, const double* vel, const doubl
 }
 
 }  // namespace
+}  // namespace fp
 
 extern "C" int fp_kappa_rta(fp_ctx* c, int nT, const double* T, const double* rates, double* kappa) {
   if (!c) return FP_EINVAL;

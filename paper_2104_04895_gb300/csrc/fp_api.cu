@@ -507,6 +507,27 @@ static int validate_opts(fp_ctx* c, int nT, const double* T, double sb, const fp
   return FP_OK;
 }
 
+// run a plan on the context's scratch (grown on demand)
+static int run_planned(fp_ctx* c, const fp_rates_opts& o, const fp::Selection& sel, const fp::Plan& p, int nT,
+                       const double* T, double sb, double* d_out, fp_stats* stats) {
+  size_t sz[fp::kScratchParts], total = 0;
+  fp::scratch_sizes(c, p, nT, sz);
+  for (size_t x : sz) total += x;
+  if (c->scratch_cap < total) {
+    dfree(c->d_scratch);
+    c->scratch_cap = 0;
+    FP_CUDA(c, dalloc(&c->d_scratch, total));
+    c->scratch_cap = total;
+  }
+  const fp::Scratch sc = fp::carve_scratch(c->d_scratch, sz);
+  unsigned long long counts[fp::kCounters] = {0};
+  std::string err;
+  const int rc = fp::run_rates(c, o, sel, p, sc, nT, T, sb, d_out, counts, o.no_graph == 0, &err);
+  if (rc) return fail(c, rc, "fp_rates4: " + err);
+  if (stats) fp::fill_stats(c, o, sel, p, counts, stats);
+  return FP_OK;
+}
+
 static int rates_impl(fp_ctx* c, int nT, const double* T, double sb, const fp_rates_opts* user, double* d_out,
                       fp_stats* stats) {
   fp_rates_opts o;
@@ -520,21 +541,7 @@ static int rates_impl(fp_ctx* c, int nT, const double* T, double sb, const fp_ra
   fp::Plan p;
   rc = fp::plan_rates(c, o, nT, sel, 0, &p, &err);
   if (rc) return fail(c, rc, "fp_rates4: " + err);
-  size_t sz[fp::kScratchParts], total = 0;
-  fp::scratch_sizes(c, p, nT, sz);
-  for (size_t x : sz) total += x;
-  if (c->scratch_cap < total) {
-    dfree(c->d_scratch);
-    c->scratch_cap = 0;
-    FP_CUDA(c, dalloc(&c->d_scratch, total));
-    c->scratch_cap = total;
-  }
-  const fp::Scratch sc = fp::carve_scratch(c->d_scratch, sz);
-  unsigned long long counts[fp::kCounters] = {0};
-  rc = fp::run_rates(c, o, sel, p, sc, nT, T, sb, d_out, counts, o.no_graph == 0, &err);
-  if (rc) return fail(c, rc, "fp_rates4: " + err);
-  if (stats) fp::fill_stats(c, o, sel, p, counts, stats);
-  return FP_OK;
+  return run_planned(c, o, sel, p, nT, T, sb, d_out, stats);
 }
 
 int fp_rates4_device(fp_ctx* c, int nT, const double* T, double scalebroad, const fp_rates_opts* opts,
@@ -659,7 +666,46 @@ int rates_passes(fp_ctx* c, int nT, const double* T, double sb, const fp_rates_o
   if (!rates) return fail(c, FP_EINVAL, name + ": NULL output");
   if (nT < 1 || nT > fp::kMaxT) return fail(c, FP_EINVAL, name + ": nT must be in [1, 8]");
   FP_CUDA(c, cudaSetDevice(c->device));
-  const size_t nm = (size_t)c->N * c->nb, need = (size_t)nT * nm;
+  const size_t nm = (size_t)c->N * c->nb;
+  // the pair kernel keeps the parts apart in one pass where their sums fit it
+  if (nT * npass <= fp::kMaxT && c->leg_symmetric && (!opts || opts->precision != FP_PREC_MIXED)) {
+    fp_rates_opts so;
+    int rc = validate_opts(c, nT, T, sb, opts, &so);
+    if (rc) return rc;
+    const int split = npass == 2 ? 1 : 2;
+    fp_rates_opts sel_o = so;
+    if (split == 1) sel_o.nu_select = 1;  // the normal/Umklapp split does not fold q and -q
+    so.no_graph = 1;
+    std::string err;
+    fp::Selection sel;
+    fp::Plan p;
+    rc = fp::make_selection(c, sel_o, true, &sel, &err);
+    if (!rc) rc = fp::plan_rates(c, so, nT, sel, 0, &p, &err, fp::kPairMirror, split);
+    if (rc) return fail(c, rc, "fp_rates4: " + err);
+    if (p.split) {
+      const size_t all = (size_t)nT * npass * nm;
+      if (c->rates_cap < all) {
+        dfree(c->d_rates);
+        c->rates_cap = 0;
+        FP_CUDA(c, dalloc(&c->d_rates, all));
+        c->rates_cap = all;
+      }
+      rc = run_planned(c, so, sel, p, nT, T, sb, c->d_rates, stats);
+      if (rc) return rc;
+      std::vector<double> part(all);
+      FP_CUDA(c, cudaMemcpyAsync(part.data(), c->d_rates, all * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+      FP_CUDA(c, cudaStreamSynchronize(c->stream));
+      for (int t = 0; t < nT; ++t)
+        for (int k = 0; k < npass; ++k)
+          std::memcpy(rates + ((size_t)t * npass + k) * nm, part.data() + ((size_t)k * nT + t) * nm, nm * sizeof(double));
+      if (stats && split == 1) {  // each part counts its candidates
+        stats->candidates *= 2.0;
+        stats->candidates_executed *= 2.0;
+      }
+      return FP_OK;
+    }
+  }
+  const size_t need = (size_t)nT * nm;
   if (c->rates_cap < need) {
     dfree(c->d_rates);
     c->rates_cap = 0;
@@ -775,14 +821,22 @@ extern "C" int fp_phase_space4(fp_ctx* c, int nT, const double* T, double scaleb
   const size_t nm = (size_t)c->N * c->nb;
   double* d = nullptr;
   FP_CUDA(c, dalloc(&d, nm * (2 + (size_t)nT) + nm));
-  double* d_p4 = d;
-  double* d_cnt = d + nm;
-  double* d_wp4 = d + 2 * nm;
+  double* d_p4 = d;  // followed by d_wp4: one pass writes both
+  double* d_wp4 = d + nm;
+  double* d_cnt = d + (1 + (size_t)nT) * nm;
   double* d_cnt2 = d + (2 + (size_t)nT) * nm;
   std::string err;
-  // pass 1: unit weights (P4) and the accepted terms per mode; pass 2: Bose and frequency weights (WP4)
-  rc = phase_pass(c, o, 1, T, scalebroad, stride, true, d_p4, d_cnt, &err);
-  if (!rc && wp4) rc = phase_pass(c, o, nT, T, scalebroad, stride, false, d_wp4, d_cnt2, &err);
+  // unit weights (P4) and the accepted terms per mode, and Bose and frequency weights (WP4).  In FP64 and double-float
+  // one pass takes both, the unit weights as a temperature more; the mixed path keeps its arithmetic for one
+  // temperature and takes two passes
+  if (wp4 && nT < fp::kMaxT && o.precision != FP_PREC_MIXED) {
+    double T1[fp::kMaxT] = {T[0]};
+    std::memcpy(T1 + 1, T, nT * sizeof(double));
+    rc = phase_pass(c, o, nT + 1, T1, scalebroad, stride, true, d_p4, d_cnt, &err);
+  } else {
+    rc = phase_pass(c, o, 1, T, scalebroad, stride, true, d_p4, d_cnt, &err);
+    if (!rc && wp4) rc = phase_pass(c, o, nT, T, scalebroad, stride, false, d_wp4, d_cnt2, &err);
+  }
   cudaError_t e = cudaSuccess;
   if (!rc && numprocess) e = cudaMemcpyAsync(numprocess, d_cnt, nm * sizeof(double), cudaMemcpyDeviceToHost, c->stream);
   if (!rc && e == cudaSuccess && p4) e = cudaMemcpyAsync(p4, d_p4, nm * sizeof(double), cudaMemcpyDeviceToHost, c->stream);

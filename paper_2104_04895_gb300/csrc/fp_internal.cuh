@@ -77,6 +77,8 @@ struct RatesArgs {
   double* mode_counts;       // [N*nb] reduction output: accepted terms per selected mode x count_scale, or null
   double count_scale;
   // pair kernel (fp_pair_kernel.cuh)
+  int nS;                    // sums per mode: nT x parts, slot part * nT + t (nT in the ordered kernel)
+  int split;                 // parts: 0 one, 1 normal and Umklapp, 2 the channels ++, +-, --
   int mirror;                // 1: `partial` has a slot per (evaluated point, q') and a pair fills the slots of both its
                              // members; 0: a slot per work item, every q' evaluated
   const int* pk_start;       // [natoms + 1] groups with D != 0 by atom k, in l order
@@ -111,7 +113,8 @@ struct Plan {
   bool sliced = false;                // its contractions on the tensor cores
   bool operands = false;              // with the sliced eigenvectors in the scratch
   bool psi_u = false;                 // its Psi prologue from the table U
-  long long values = 0;               // partial sums per temperature
+  long long values = 0;               // partial sums per slot
+  int nS = 1, split = 0;              // sums per mode and what they keep apart (RatesArgs)
 };
 
 // Device working memory of one rates call (owned by the caller of run_rates), in the order of scratch_sizes.
@@ -127,7 +130,7 @@ struct Scratch {
   int* qlist;                    // [N]
   int* qpos;                     // [N]
   double* wt;                    // [nT][N*nb][3]
-  double* partial;               // [Plan::values][nT]
+  double* partial;               // [Plan::values][nS]
   float* omh;                    // [N*nb]
   float* oml;
   float* velh;                   // [N*nb*3]
@@ -221,8 +224,10 @@ int make_selection(const fp_ctx* c, const fp_rates_opts& o, bool fold_allowed, S
 // per-item partial sums fit; `form` is the richest form of the rate kernel that the caller allows.  Returns FP_OK or an
 // FP_E* code with a message in *err.
 enum RateForm { kOrdered = 0, kPair = 1, kPairSliced = 2, kPairMirror = 3 };
+// `split` keeps the parts of the rates apart (RatesArgs::split) where the pair kernel runs and they fit kMaxT sums;
+// Plan::split says whether it does.
 int plan_rates(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, size_t partial_budget, Plan* p,
-               std::string* err, RateForm form = kPairMirror);
+               std::string* err, RateForm form = kPairMirror, int split = 0);
 // Byte sizes of the Scratch buffers of a plan, in the order of the Scratch fields (each rounded up to 256).
 void scratch_sizes(const fp_ctx* c, const Plan& p, int nT, size_t sizes[kScratchParts]);
 // Scratch pointers laid out from `base` with the sizes of scratch_sizes.
@@ -230,7 +235,8 @@ Scratch carve_scratch(unsigned char* base, const size_t sizes[kScratchParts]);
 // Variants of a rates launch used by the phase-space entry points.
 struct RunExtra {
   int unit_stride = 0;          // > 0: |W|^2 := 1, q' on this stride, ordered (q', q'') pairs, no prefactor
-  bool unit_weights = false;    // Bose and frequency weights := 1 (the unweighted phase space)
+  bool unit_weights = false;    // Bose and frequency weights := 1 (the unweighted phase space) for the first
+                                // temperature, whose entry in T does not count
   unsigned long long* d_item_counts = nullptr;  // [n_items][J]: with d_mode_counts, per-mode accepted terms
   double* d_mode_counts = nullptr;              // [N*nb] accepted terms of each selected mode x unit_stride
 };

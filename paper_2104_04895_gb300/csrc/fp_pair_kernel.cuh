@@ -1,6 +1,7 @@
 // Four-phonon rate kernel over unordered wavevector pairs (FP64 and double-float paths; paper Sec. 2.2 Eqs. tao0,
 // 4phgamma, V4; Sec. 2.4).  Used when the quartet list obeys the transposition symmetry of Sec. 2.3 (Eq. TS), which
-// fp_init checks; otherwise the kernel of fp_rates_kernel.cuh runs.
+// fp_init checks; otherwise the kernel of fp_rates_kernel.cuh runs.  One pass can keep the parts of a rate apart
+// (RatesArgs::split): normal and Umklapp processes, which one k2 decides for a whole test, or the three channels.
 //
 // What it shares.  The rate of a = (q, j0) is a sum over b = lambda' of R(a; b), where R(a; b) collects every process
 // in which b is the partner lambda' and {c, d} are lambda'', lambda''' in both orders.  Write all four wavevectors as
@@ -127,7 +128,7 @@ struct PairCarve {
   }
 };
 
-__host__ __device__ inline PairCarve make_pair_carve(int nb, int J, int G, int nquart, int nT, int threads,
+__host__ __device__ inline PairCarve make_pair_carve(int nb, int J, int G, int nquart, int nT, int nS, int threads,
                                                    bool sliced) {
   PairCarve c;
   const size_t nb2 = (size_t)nb * nb, na = nb / 3, nwarps = ((size_t)threads + 31) / 32;
@@ -153,7 +154,7 @@ __host__ __device__ inline PairCarve make_pair_carve(int nb, int J, int G, int n
   c.V3 = d; d += 3 * nb;
   c.Iv8 = d; d += 2 * nb2;             // 8/sigma (or -1: delta := 1) of |v2 - v3| and |v2 + v3|, [y][j3]
   c.F = d; d += 3 * nb2;               // (1/sigma) x constants of P1, P2, P3 (x c and d weights for one temperature)
-  c.WB = d; d += nT > 1 ? 3 * (size_t)nT * nb2 : 0;  // c and d weights of P1, P2, P3 per temperature
+  c.WB = d; d += nS > 1 ? 3 * (size_t)nT * nb2 : 0;  // c and d weights of P1, P2, P3 per temperature
   c.Wc = d; d += 2 * (size_t)nT * nb;  // (1+n)/w and n/w of k2
   c.Wd = d; d += 2 * (size_t)nT * nb;  // and of k3
   c.Val = d; d += sliced ? 0 : nwarps * kPairCap;
@@ -219,7 +220,7 @@ __device__ __noinline__ float2 pair_two_orders(float2 ex, float2 z8, const float
   return make_float2(0.5f * m.x, 0.5f * m.y);
 }
 
-// NB branches, up to MAXT temperatures.  DF: vertex contraction and terms in double-float on the FP32 pipes.  SL: both
+// NB branches, up to MAXT sums per row.  DF: vertex contraction and terms in double-float on the FP32 pipes.  SL: both
 // vertex contractions on the tensor cores in exact slices (fp_slices.cuh; unit eigenvectors, nb = 6 or 12): A in FP64,
 // T as digits, |W|^2 of every entry in FP64.
 template <int NB, int MAXT, bool DF, bool SL>
@@ -231,10 +232,10 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ long long s_item;
   __shared__ unsigned s_umask;
-  const int J = a.J, G = a.G, nT = a.nT, N = a.N;
+  const int J = a.J, G = a.G, nT = a.nT, nS = a.nS, N = a.N;  // nS sums per row: temperatures x parts
   const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, warp = tid >> 5;
   const int rows = J * NB2;
-  const PairCarve cv = make_pair_carve(NB, J, G, a.nquart, nT, nthr, SL);
+  const PairCarve cv = make_pair_carve(NB, J, G, a.nquart, nT, a.nS, nthr, SL);
   C* cx = reinterpret_cast<C*>(smem);
   C *sE0 = cx + cv.E0, *sE1 = cx + cv.E1, *sE2 = cx + cv.E2, *sE3 = cx + cv.E3;
   C *sPsi = cx + cv.Psi, *sT = cx + cv.T, *sTw2 = cx + cv.Tw2, *sTwQ = cx + cv.TwQ;
@@ -270,6 +271,10 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
   const bool f32_sigma = a.dq_mode == 0;
   const double inv_sbdq = 1.0 / (a.sb * a.dq);
   const bool unit = a.unit_vertex != 0;
+  // part of a test: by normal (0) and Umklapp (1), or by channel ++, +-, --
+  auto part_of = [&](int kind, unsigned um) {
+    return a.split == 0 ? 0 : a.split == 1 ? (int)((um >> kind) & 1u) : kind == 0 ? 1 : kind < 3 ? 0 : 2;
+  };
 
   for (int o = tid; o < kExpTab; o += nthr) sExpT[o] = pair_val<VT>(exp(-(double)o * kExpH));
   for (int o = tid; o < NA + 1; o += nthr) sKLs[o] = a.pk_start[o];
@@ -465,7 +470,7 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
       if constexpr (MAXT == 1) {
         R45[0] = R45[1] = 0.0;
       } else {
-        for (int t = 0; t < 2 * nT; ++t) R45[t] = 0.0;
+        for (int t = 0; t < 2 * nS; ++t) R45[t] = 0.0;
       }
 #pragma unroll
       for (int k = 0; k < kRun; ++k) sh[k] = sl[k] = 0.f;
@@ -481,7 +486,8 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
           for (int k = 0; k < kRun; ++k) sh[k] = sl[k] = 0.f;
         }
       };
-      // value v of test `kind` at the entry e = (y, j3) into the row's sums
+      // value v of test `kind` at the entry e = (y, j3) into the row's sums, those of its part from slot lo
+      unsigned umask = 0;  // Umklapp tests of the current k2
       auto add = [&](const VT v, const int kind, const int e) {
         if constexpr (DF) {
           auto run = [&](int k, float2 term) {
@@ -500,17 +506,18 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
               run(2, v);
           } else {
             const float2* wb = sWB + (kind < 3 ? kind : 0) * NB2 + e;
+            const int lo = part_of(kind, umask) * nT;
             if (kind < 3) {
 #pragma unroll
               for (int t = 0; t < MAXT; ++t) {
-                if (t >= nT) break;
-                run(t, df_mul(v, wb[3 * t * NB2]));
+                if (t >= nS) break;
+                if (t >= lo && t < lo + nT) run(t, df_mul(v, wb[3 * (t - lo) * NB2]));
               }
             } else {
 #pragma unroll 1
               for (int t = 0; t < nT; ++t) {
                 const float2 term = df_mul(v, wb[3 * t * NB2]);
-                R45[(kind - 3) * nT + t] += (double)term.x + (double)term.y;
+                R45[(kind - 3) * nS + lo + t] += (double)term.x + (double)term.y;
               }
             }
           }
@@ -523,15 +530,19 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
             R45[1] += v;
         } else {
           const double* wb = sWB + (kind < 3 ? kind : 0) * NB2 + e;
+          const int lo = part_of(kind, umask) * nT;
           if (kind < 3) {
 #pragma unroll
             for (int t = 0; t < MAXT; ++t) {
-              if (t >= nT) break;
-              S1[t] = fma(v, wb[3 * t * NB2], S1[t]);
+              if (t >= nS) break;
+              if (t >= lo && t < lo + nT) S1[t] = fma(v, wb[3 * (t - lo) * NB2], S1[t]);
             }
           } else {
 #pragma unroll 1
-            for (int t = 0; t < nT; ++t) R45[(kind - 3) * nT + t] = fma(v, wb[3 * t * NB2], R45[(kind - 3) * nT + t]);
+            for (int t = 0; t < nT; ++t) {
+              double& r = R45[(kind - 3) * nS + lo + t];
+              r = fma(v, wb[3 * t * NB2], r);
+            }
           }
         }
       };
@@ -560,7 +571,7 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
         if (kd < k2) continue;  // {c, d} is visited at its smaller index
         const bool twice = kd != k2;  // both orders of {c, d} come from this visit
         // ---- tables of k2 and k3
-        if (a.nu_select != 0 && tid == 0) s_umask = pair_umklapp_bits(a, g, g1, g2, g3);
+        if ((a.nu_select != 0 || a.split == 1) && tid == 0) s_umask = pair_umklapp_bits(a, g, g1, g2, g3);
         if constexpr (SL) {
           constexpr int kOp4 = slices::Shape<SL ? NB : 6>::kOperand / 4;
           const uint4* src = reinterpret_cast<const uint4*>(a.operands);
@@ -845,6 +856,7 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
         __syncthreads();
         // ---- window tests of the row's entries and evaluation of the accepted ones
         {
+          if (a.split == 1) umask = s_umask;
           const int x = rj1, y = rc, jq = has_row ? rjj : 0;
           const unsigned cand = row_cand & proc_cand &
                                 (a.nu_select == 0 ? 31u : a.nu_select == 1 ? ~s_umask : s_umask) &
@@ -967,7 +979,7 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
                     float4 Wd = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
                     for (int c = 0; c < NB; ++c) cdf_mac(Wd, e2[c], tb[c * NB]);
-                    W2 = cdf_abs2_df(Wd);
+                    W2 = cdf_abs2_df(cdf_norm(Wd));  // a vanishing W leaves its high parts cancelled
                   }
                   if (iv8.x >= 0.f) {
                     const float2 x8 = df_mul(df_make(dw), iv8);
@@ -1026,7 +1038,7 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
       const size_t slot = a.mirror ? ((size_t)qi * N + k1) * a.nchunk + chunk : 0;
       const size_t mslot = mir ? ((size_t)role.mirror * N + role.mirror_b) * a.nchunk + chunk : 0;
       const int nout = J + (mir ? NB : 0);
-      for (int t = 0; t < nT; ++t) {
+      for (int t = 0; t < nS; ++t) {
         if (has_row) {
           double s1 = 0.0;
 #pragma unroll
@@ -1036,13 +1048,13 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
           const double f = SL && !unit && any ? scalbn(1.0, 2 * sSc[rjj * NB + rj1] - 102) : 1.0;
           sRed[tid] = f * s1;
           sRed[rows + tid] = f * R45[t];
-          sRed[2 * rows + tid] = f * R45[nT + t];
+          sRed[2 * rows + tid] = f * R45[nS + t];
         }
         __syncthreads();
         if (tid < nout) {
           const bool direct = tid < J;
           const int m = direct ? tid : tid - J;
-          const double* W = a.wt + 3 * (size_t)t * NM;
+          const double* W = a.wt + 3 * (size_t)(t % nT) * NM;
           double sum = 0.0;
           for (int o = 0; o < (direct ? NB : J); ++o) {
             const int r0 = ((direct ? m : o) * NB + (direct ? o : m)) * NB;
@@ -1056,10 +1068,14 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
           }
           sum *= W[3 * (direct ? (size_t)q * NB + j0b + m : (size_t)k1 * NB + m)];
           if (!a.mirror) {
-            if (t == 0 && nT == 1) dir += sum;
-            if (nT > 1) a.partial[(((size_t)item * J + m) * nT) + t] = (k1 == k1_first ? 0.0 : a.partial[(((size_t)item * J + m) * nT) + t]) + sum;
+            if (nS == 1) {
+              dir += sum;
+            } else {
+              double& out = a.partial[((size_t)item * J + m) * nS + t];
+              out = (k1 == k1_first ? 0.0 : out) + sum;
+            }
           } else {
-            a.partial[((direct ? slot : mslot) * NB + m) * nT + t] = sum;
+            a.partial[((direct ? slot : mslot) * NB + m) * nS + t] = sum;
           }
         }
         __syncthreads();
@@ -1086,10 +1102,10 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
       }
     }
     if (!a.mirror && tid < J) {
-      if (nT == 1)
+      if (nS == 1)
         a.partial[(size_t)item * J + tid] = dir;
       else if (k1_first >= k1_end)
-        for (int t = 0; t < nT; ++t) a.partial[((size_t)item * J + tid) * nT + t] = 0.0;
+        for (int t = 0; t < nS; ++t) a.partial[((size_t)item * J + tid) * nS + t] = 0.0;
       if (a.item_counts) a.item_counts[(size_t)item * J + tid] = dir_n;
     }
     unsigned long long c0 = cnt0, c1 = cnt1, c2 = cnt2, cw = nwf, ct = nte;

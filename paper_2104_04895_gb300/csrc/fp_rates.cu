@@ -63,7 +63,7 @@ __global__ void prep_kernel(RatesArgs a, float* omh, float* oml, float* velh, fl
 // rates[t][q][j] = pref * sum_tiles partial[(tile, qpos[q], chunk)][jj][t], in a fixed order, for every selected
 // mode of the output range (the others stay zero); under time reversal q and -q read the same partial sums.
 __global__ void reduce_kernel(RatesArgs a, double pref, double* rates) {
-  const long long n = (long long)a.nT * a.q_out_n * a.nb;
+  const long long n = (long long)a.nS * a.q_out_n * a.nb;
   long long o = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (o >= n) return;
   const int j = (int)(o % a.nb);
@@ -75,7 +75,7 @@ __global__ void reduce_kernel(RatesArgs a, double pref, double* rates) {
   double s = 0.0;
   for (int tile = 0; tile < a.ntile; ++tile) {
     const long long item = ((long long)tile * a.nq_sel + qi) * a.nchunk + chunk;
-    s += a.partial[((size_t)item * a.J + jj) * a.nT + t];
+    s += a.partial[((size_t)item * a.J + jj) * a.nS + t];
   }
   rates[((size_t)t * a.N + q) * a.nb + j] = s * pref;
   if (a.mode_counts && t == 0) {
@@ -91,7 +91,7 @@ __global__ void reduce_kernel(RatesArgs a, double pref, double* rates) {
 // The same for the pair kernel's slots: one warp per output, the slots of q (its pair with every q') summed by lane
 // and then across lanes, in a fixed order.  A slot that a chunked mirrored pair wrote holds one value per chunk.
 __global__ void pair_reduce_kernel(RatesArgs a, double pref, double* rates) {
-  const long long n = (long long)a.nT * a.q_out_n * a.nb;
+  const long long n = (long long)a.nS * a.q_out_n * a.nb;
   const long long o = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (o >= n) return;
@@ -108,12 +108,12 @@ __global__ void pair_reduce_kernel(RatesArgs a, double pref, double* rates) {
     const size_t base = ((size_t)qi * a.N + b) * a.nchunk;
     if (a.nchunk == 1 || pair_role(a, qi, qe, b).run) {
       const size_t v = (base + chunk) * a.nb + jj;
-      s += a.partial[v * a.nT + t];
+      s += a.partial[v * a.nS + t];
       if (a.mode_counts && t == 0) cnt += a.item_counts[v];
     } else {
       for (int c = 0; c < a.nchunk; ++c) {
         const size_t v = (base + c) * a.nb + j;
-        s += a.partial[v * a.nT + t];
+        s += a.partial[v * a.nS + t];
         if (a.mode_counts && t == 0) cnt += a.item_counts[v];
       }
     }
@@ -166,8 +166,8 @@ __global__ void fill_kernel(double* p, long long n, double v) {
 }
 
 // kernel for (precision, nb, number of temperatures, tensor cores): one accumulator per temperature, 1 or up to 8
-const void* rates_kernel_ptr(int precision, int nb, int nT, bool tc, bool pair, bool sliced) {
-  const int maxt = nT == 1 ? 1 : kMaxT;
+const void* rates_kernel_ptr(int precision, int nb, int nS, bool tc, bool pair, bool sliced) {
+  const int maxt = nS == 1 ? 1 : nS == 2 && pair ? 2 : kMaxT;
   if (pair)
     return precision == FP_PREC_DOUBLE_FLOAT ? pair_kernel_df(nb, maxt) : pair_kernel_f64(nb, maxt, sliced);
   if (tc) return precision == FP_PREC_MIXED ? rates_kernel_f32_tc(nb, maxt) : nullptr;
@@ -175,18 +175,18 @@ const void* rates_kernel_ptr(int precision, int nb, int nT, bool tc, bool pair, 
   return precision == FP_PREC_FP64 ? rates_kernel_f64(nb, maxt) : rates_kernel_f32(nb, maxt);
 }
 
-size_t smem_bytes(int precision, int nb, int J, int G, int nquart, int nT, int threads, bool tc, bool pair,
+size_t smem_bytes(int precision, int nb, int J, int G, int nquart, int nT, int nS, int threads, bool tc, bool pair,
                   bool sliced) {
-  if (pair) return make_pair_carve(nb, J, G, nquart, nT, threads, sliced).bytes();
+  if (pair) return make_pair_carve(nb, J, G, nquart, nT, nS, threads, sliced).bytes();
   const bool f32 = precision == FP_PREC_MIXED;  // the double-float path has the FP64 path's shared memory
   Carve c = make_carve(nb, J, G, nquart, nT, threads, f32);
   const size_t b = c.bytes(f32 ? sizeof(Cx<float>) : sizeof(Cx<double>));
   return tc ? align128(b) + kTcBytes : b;
 }
 
-int max_ctas_per_sm(int precision, int nb, int nT, int threads, size_t smem, bool tc, bool pair,
+int max_ctas_per_sm(int precision, int nb, int nS, int threads, size_t smem, bool tc, bool pair,
                     bool sliced) {
-  const void* k = rates_kernel_ptr(precision, nb, nT, tc, pair, sliced);
+  const void* k = rates_kernel_ptr(precision, nb, nS, tc, pair, sliced);
   if (!k) return 0;
   if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
   int n = 0;
@@ -265,14 +265,15 @@ int make_selection(const fp_ctx* c, const fp_rates_opts& o, bool fold_allowed, S
 }
 
 static int plan_form(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, size_t partial_budget, Plan* p,
-                     std::string* err, bool pair, bool sliced, bool mirror) {
+                     std::string* err, bool pair, bool sliced, bool mirror, int split) {
+  const int nS = nT * (split == 1 ? 2 : split == 2 ? 3 : 1);
   const int N = c->N, nb = c->nb;
   const bool tc = o.tensor_cores != 0;
   if (tc && (o.precision != FP_PREC_MIXED || nb != 6)) {
     *err = "tensor_cores needs the mixed precision and 6 branches";
     return FP_EINVAL;
   }
-  if (!rates_kernel_ptr(o.precision, nb, nT, tc, pair, sliced)) {
+  if (!rates_kernel_ptr(o.precision, nb, nS, tc, pair, sliced)) {
     *err = "unsupported number of branches";
     return FP_EINVAL;
   }
@@ -293,7 +294,7 @@ static int plan_form(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, 
     const size_t room = pair ? (pair_blocks_for(nb) == 1 ? 227 : 112) * 1024 : 110 * 1024;
     J = nb;
     while (J > 1 && (J * nb * nb > most ||
-                     smem_bytes(o.precision, nb, J, c->G, c->nquart, nT, pair ? (J * nb * nb + 31) / 32 * 32 : most, tc, pair, sliced) > room)) {
+                     smem_bytes(o.precision, nb, J, c->G, c->nquart, nT, nS, pair ? (J * nb * nb + 31) / 32 * 32 : most, tc, pair, sliced) > room)) {
       int nj = J - 1;
       while (nj > 1 && nb % nj) --nj;
       J = nj;
@@ -315,13 +316,13 @@ static int plan_form(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, 
   const int nchunk = nb / J;
   int t1 = o.k1_tile > 0 ? o.k1_tile : t1_tuned > 0 ? t1_tuned : (N + 511) / 512;
   auto part_bytes = [&](int tile) {
-    return (size_t)((N + tile - 1) / tile) * nq_sel * nchunk * J * nT * sizeof(double);
+    return (size_t)((N + tile - 1) / tile) * nq_sel * nchunk * J * nS * sizeof(double);
   };
   // a slot per (evaluated point, q') halves the pairs to evaluate; without the memory for it, every q' is evaluated
   // and a work item has one slot
   mirror = mirror && pair;
   const long long mirror_values = (long long)nq_sel * N * nchunk * nb;
-  const size_t mirror_bytes = (size_t)mirror_values * nT * sizeof(double);
+  const size_t mirror_bytes = (size_t)mirror_values * nS * sizeof(double);
   if (mirror && partial_budget && mirror_bytes > partial_budget) mirror = false;
   if (mirror && mirror_bytes > (size_t(256) << 20) && mirror_bytes > c->scratch_cap) {
     size_t mem_free = 0, mem_total = 0;
@@ -352,12 +353,12 @@ static int plan_form(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, 
     *err = "per-item partial sums do not fit the scratch";
     return FP_EINVAL;
   }
-  const size_t smem = smem_bytes(o.precision, nb, J, c->G, c->nquart, nT, threads, tc, pair, sliced);
+  const size_t smem = smem_bytes(o.precision, nb, J, c->G, c->nquart, nT, nS, threads, tc, pair, sliced);
   if (smem > 227 * 1024) {
     *err = "tile does not fit in shared memory";
     return FP_EINVAL;
   }
-  const int per_sm = max_ctas_per_sm(o.precision, nb, nT, threads, smem, tc, pair, sliced);
+  const int per_sm = max_ctas_per_sm(o.precision, nb, nS, threads, smem, tc, pair, sliced);
   if (per_sm < 1) {
     *err = "kernel tile cannot be resident on an SM";
     return FP_EINVAL;
@@ -377,6 +378,8 @@ static int plan_form(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, 
   p->smem = smem;
   p->pair = pair;
   p->sliced = sliced;
+  p->nS = nS;
+  p->split = split;
   p->operands = sliced;
   p->mirror = mirror;
   p->values = mirror ? mirror_values : p->n_items * J;
@@ -394,20 +397,21 @@ static int plan_form(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, 
 }
 
 int plan_rates(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, size_t partial_budget, Plan* p,
-               std::string* err, RateForm form) {
+               std::string* err, RateForm form, int split) {
+  if (nT * (split == 1 ? 2 : 3) > kMaxT) split = 0;
   // The pair kernel identifies vertices whose legs are permuted, so it needs Phi4 to have that symmetry; where its
   // tables do not fit, the ordered kernel runs.  The mixed path keeps the ordered kernel: its FP32 vertex rounds
   // differently for each order of the legs, and exchanging them moved the rates by up to 2e-8 (its error is 5e-8).
   if (form != kOrdered && c->leg_symmetric && o.precision != FP_PREC_MIXED) {
     // the FP64 path's contraction in slices: 6 and 12 branches (with 3, K = 6 would leave most of a tile empty)
     if (form != kPair && o.precision == FP_PREC_FP64 && c->unit_modes && c->nb >= 6) {
-      const int rc = plan_form(c, o, nT, sel, partial_budget, p, err, true, true, form == kPairMirror);
+      const int rc = plan_form(c, o, nT, sel, partial_budget, p, err, true, true, form == kPairMirror, split);
       if (rc != FP_EINVAL) return rc;
     }
-    const int rc = plan_form(c, o, nT, sel, partial_budget, p, err, true, false, form == kPairMirror);
+    const int rc = plan_form(c, o, nT, sel, partial_budget, p, err, true, false, form == kPairMirror, split);
     if (rc != FP_EINVAL) return rc;
   }
-  return plan_form(c, o, nT, sel, partial_budget, p, err, false, false, false);
+  return plan_form(c, o, nT, sel, partial_budget, p, err, false, false, false, 0);
 }
 
 void scratch_sizes(const fp_ctx* c, const Plan& p, int nT, size_t s[kScratchParts]) {
@@ -419,7 +423,7 @@ void scratch_sizes(const fp_ctx* c, const Plan& p, int nT, size_t s[kScratchPart
   s[4] = up256((size_t)c->N * sizeof(int));               // qlist
   s[5] = up256((size_t)c->N * sizeof(int));               // qpos
   s[6] = up256(3 * nm * nT * sizeof(double));             // wt
-  s[kScratchPartial] = up256((size_t)p.values * nT * sizeof(double));
+  s[kScratchPartial] = up256((size_t)p.values * p.nS * sizeof(double));
   s[8] = up256(nm * sizeof(float));
   s[9] = up256(nm * sizeof(float));
   s[10] = up256(3 * nm * sizeof(float));
@@ -541,6 +545,8 @@ int run_rates(fp_ctx* c, const fp_rates_opts& o, const Selection& sel, const Pla
   a.partial = sc.partial;
   a.counter = sc.counters;
   a.counts = sc.counters + 1;
+  a.nS = p.nS;
+  a.split = p.split;
   a.mirror = p.mirror ? 1 : 0;
   a.pk_start = c->d_pk_start;
   a.pk_grp = c->d_pk_grp;
@@ -563,14 +569,15 @@ int run_rates(fp_ctx* c, const fp_rates_opts& o, const Selection& sel, const Pla
   const double pref = unit_stride > 0
                           ? (double)unit_stride / ((double)N * (double)N)
                           : kPi * kHbar * kHbar * conv * conv * conv * conv / (8.0 * (double)N * (double)N);
-  const void* k = rates_kernel_ptr(o.precision, nb, nT, o.tensor_cores != 0, p.pair, p.sliced);
+  const void* k = rates_kernel_ptr(o.precision, nb, p.nS, o.tensor_cores != 0, p.pair, p.sliced);
   // the device part of a rate set: Bose weights, FP32 tables, cleared counters and output, the persistent
   // rate kernel and the reduction
   auto enqueue = [&]() -> cudaError_t {
     cudaError_t e = cudaSuccess;
     if (x.unit_weights) {
-      fill_kernel<<<152, 256, 0, s>>>(sc.wt, 3LL * (long long)nm * nT, 1.0);
+      fill_kernel<<<152, 256, 0, s>>>(sc.wt, 3LL * (long long)nm, 1.0);
       e = cudaGetLastError();
+      if (e == cudaSuccess && nT > 1) e = launch_weights(c, nT - 1, sc.T + 1, sc.wt + 3 * nm, s);
     } else {
       e = launch_weights(c, nT, sc.T, sc.wt, s);
     }
@@ -593,12 +600,12 @@ int run_rates(fp_ctx* c, const fp_rates_opts& o, const Selection& sel, const Pla
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     if ((e = cudaMemsetAsync(sc.counters, 0, kCounters * sizeof(unsigned long long), s)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(d_out, 0, (size_t)nT * nm * sizeof(double), s)) != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(d_out, 0, (size_t)p.nS * nm * sizeof(double), s)) != cudaSuccess) return e;
     if (p.n_items > 0) {
       RatesArgs aa = a;
       void* args[] = {&aa};
       if ((e = cudaLaunchKernel(k, dim3(p.ctas), dim3(p.threads), args, p.smem, s)) != cudaSuccess) return e;
-      const long long n = (long long)nT * (sel.q_out_end - sel.q_out_begin) * nb;
+      const long long n = (long long)p.nS * (sel.q_out_end - sel.q_out_begin) * nb;
       if (p.mirror)
         pair_reduce_kernel<<<(unsigned)((n + 7) / 8), 256, 0, s>>>(a, pref, d_out);
       else

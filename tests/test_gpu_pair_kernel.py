@@ -134,3 +134,45 @@ def test_force_constants_of_any_size(scale):
         ctx.set_modes(w, e, v)
         out, _ = ctx.rates4(cr.temps, cr.scalebroad)
     _close(out.reshape(1, -1) / scale ** 2, ref)
+
+
+def _close_parts(got, ref):
+    """_close where a part of a symmetric grid may hold only vertices that vanish: rounding, 1e-30 of the others, on both
+    sides."""
+    noise = np.abs(ref) <= 1e-20 * ref.max()
+    assert np.all(np.abs(got[noise]) <= 1e-20 * ref.max())
+    _close(got[~noise], ref[~noise])
+
+
+@pytest.mark.parametrize("precision", [FP_PREC_FP64, FP_PREC_DOUBLE_FLOAT])
+@pytest.mark.parametrize("maker,nT", [(lambda: synth.simple_cubic((4, 3, 2)), 1), (lambda: synth.zincblende_bas((3, 2, 2)), 2),
+                                      (lambda: synth.licoo2((2, 1, 2)), 4), (lambda: synth.diamond_si((2, 2, 2)), 5)])
+def test_parts_in_one_pass(precision, maker, nT):
+    """Normal and Umklapp parts and the channels: one pass up to eight sums per mode (2 nT, 3 nT), passes beyond."""
+    cr = maker()
+    w, e, v = oracle_modes(cr)
+    temps = list(np.linspace(300.0, 900.0, nT))
+    N, nb = cr.nq, cr.nb
+    rng = np.random.Generator(np.random.PCG64(N))
+    mask = (rng.random(N * nb) < 0.5).astype(np.uint8)
+    with Context.from_crystal(cr) as ctx:
+        ctx.set_modes(w, e, v)
+        nu, st = ctx.rates4_nu(temps, cr.scalebroad, precision=precision)
+        nm, st_m = ctx.rates4_nu(temps, cr.scalebroad, precision=precision, mode_mask=mask, process_mask=6)
+        ch, st_c = ctx.rates4_channels(temps, cr.scalebroad, precision=precision)
+        full, st_f = ctx.rates4(temps, cr.scalebroad, precision=precision)
+    total = np.zeros(3)
+    for p, name in enumerate(("normal", "umklapp")):
+        ref, acc = oracle.rates4(cr, w, e, v, temps=temps, nu=name)
+        _close_parts(nu[:, p].reshape(nT, -1), ref)
+        total += acc
+        sel = np.nonzero(mask)[0]
+        ref, _ = oracle.rates4(cr, w, e, v, temps=temps, nu=name, sel=sel, processes=(1, 2))
+        _close_parts(nm[:, p].reshape(nT, -1)[:, sel], ref)
+        assert np.all(nm[:, p].reshape(nT, -1)[:, mask == 0] == 0.0)
+    for p in range(3):
+        ref, acc = oracle.rates4(cr, w, e, v, temps=temps, processes=(p,))
+        _close_parts(ch[:, p].reshape(nT, -1), ref)
+        assert st_c["accepted"][p] == acc[p]
+    assert st["accepted"] == list(total) == st_f["accepted"]
+    assert st["candidates"] == 2 * st_f["candidates"] and st_c["candidates"] == st_f["candidates"]

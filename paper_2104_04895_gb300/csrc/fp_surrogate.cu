@@ -202,75 +202,220 @@ __global__ void gather_kernel(const float* X, int F, const int* rows, int n, flo
 }
 
 // ------------------------------------------------------------------------------------------------
-// FP32 network kernels.  C[M][N] = act(sum_k A(m,k) B(k,n) + bias[n]); A(m,k) = A[m*lda+k] or A[k*lda+m]
-// (transA), B(k,n) = B[k*ldb+n] or B[n*ldb+k] (transB).  32x32 tiles, one output per thread, k in order
-// (deterministic).
-constexpr int kTile = 32;
+// FP32 network kernels.  Every output is one chain of FMAs (or adds) in the order of its index k, so results do not
+// depend on the launch.  The chains are short enough (the batch, at most a few thousand) that latency and the number of
+// launches bound a minibatch: each layer's backward runs in one launch whose blocks take the weight gradient, the bias
+// gradient and the next layer's deltas, with the tanh derivative in the epilogue.  A minibatch of 1024 with 19 inputs
+// through fp_mlp_loss_grad: 820 us with 18 launches, one-block bias sums and 15 allocations, 310 us now, same bits.
+constexpr int kTile = 32;   // rows and columns of a block in the row-wise products
+constexpr int kChunk = 128; // k values staged at once there
+constexpr int kGTile = 16;  // outputs per side of a block in the weight gradients
+constexpr int kGRows = 64;  // batch rows staged at once there
 
-__global__ void gemm_kernel(int M, int Nn, int K, const float* A, int lda, int transA, const float* B, int ldb,
-                            int transB, float* C, int ldc, const float* bias, int act_tanh) {
-  __shared__ float As[kTile][kTile + 1];
-  __shared__ float Bs[kTile][kTile + 1];
+// C[r][n] for 32 x 32 outputs: acc = fma(A[r][k], B(k, n), acc) over k in order, B(k, n) = W[n K + k] (wt) or W[k ldw + n]
+template <bool kWT>
+__device__ __forceinline__ void tile_product(const float* A, int M, int K, const float* W, int Nn, int r0, int n0,
+                                             float (*As)[kChunk + 1], float (*Bs)[kTile + 1], float acc[4]) {
   const int tx = threadIdx.x % kTile, ty = threadIdx.x / kTile;  // 32 x 8 threads
-  const int m0 = blockIdx.y * kTile, n0 = blockIdx.x * kTile;
-  float acc[4] = {0.f, 0.f, 0.f, 0.f};
-  for (int k0 = 0; k0 < K; k0 += kTile) {
-    for (int r = ty; r < kTile; r += 8) {
-      const int m = m0 + r, k = k0 + tx;
-      As[r][tx] = (m < M && k < K) ? (transA ? A[(size_t)k * lda + m] : A[(size_t)m * lda + k]) : 0.f;
-      const int kk = k0 + r, n = n0 + tx;
-      Bs[r][tx] = (kk < K && n < Nn) ? (transB ? B[(size_t)n * ldb + kk] : B[(size_t)kk * ldb + n]) : 0.f;
+  for (int i = 0; i < 4; ++i) acc[i] = 0.f;
+  for (int k0 = 0; k0 < K; k0 += kChunk) {
+    const int kn = min(kChunk, K - k0);
+    for (int o = threadIdx.x; o < kTile * kn; o += 256) {
+      const int r = o / kn, k = o % kn;
+      As[r][k] = r0 + r < M ? A[(size_t)(r0 + r) * K + k0 + k] : 0.f;
+    }
+    for (int o = threadIdx.x; o < kTile * kn; o += 256) {
+      const int n = kWT ? o / kn : o % kTile, k = kWT ? o % kn : o / kTile;
+      Bs[k][n] = n0 + n < Nn ? (kWT ? W[(size_t)(n0 + n) * K + k0 + k] : W[(size_t)(k0 + k) * Nn + n0 + n]) : 0.f;
     }
     __syncthreads();
+#pragma unroll 8
+    for (int k = 0; k < kn; ++k) {
+      const float b = Bs[k][tx];
 #pragma unroll
-    for (int kk = 0; kk < kTile; ++kk) {
-      const float b = Bs[kk][tx];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) acc[i] = fmaf(As[ty + 8 * i][kk], b, acc[i]);
+      for (int i = 0; i < 4; ++i) acc[i] = fmaf(As[ty + 8 * i][k], b, acc[i]);
     }
     __syncthreads();
   }
+}
+
+// H[r][n] = tanh(sum_k A[r][k] W[n][k] + bias[n]), n < kH
+__global__ void __launch_bounds__(256) layer_kernel(int M, int K, const float* A, const float* W, const float* bias, float* H) {
+  __shared__ float As[kTile][kChunk + 1];
+  __shared__ float Bs[kChunk][kTile + 1];
+  const int r0 = blockIdx.x * kTile, n0 = blockIdx.y * kTile;
+  float acc[4];
+  tile_product<true>(A, M, K, W, kH, r0, n0, As, Bs, acc);
+  const int n = n0 + threadIdx.x % kTile;
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    const int m = m0 + ty + 8 * i, n = n0 + tx;
-    if (m < M && n < Nn) {
-      float v = acc[i] + (bias ? bias[n] : 0.f);
-      C[(size_t)m * ldc + n] = act_tanh ? tanhf(v) : v;
+    const int r = r0 + threadIdx.x / kTile + 8 * i;
+    if (r < M) H[(size_t)r * kH + n] = tanhf(acc[i] + bias[n]);
+  }
+}
+
+// y[r] = sum_k H3[r][k] w4[k] + b4 and, with targets, dy = 2 (y - t) / B and D3 = dy w4 (1 - H3^2); 32 rows per block
+__global__ void __launch_bounds__(256) head_kernel(int M, const float* H3, const float* w4, const float* b4, float* y,
+                                                   const float* t, float* dy, float* D3) {
+  __shared__ float Hs[kTile][kH + 1];
+  __shared__ float ws[kH];
+  __shared__ float ds[kTile];
+  const int r0 = blockIdx.x * kTile;
+  for (int o = threadIdx.x; o < kTile * kH; o += 256)
+    Hs[o / kH][o % kH] = r0 + o / kH < M ? H3[(size_t)r0 * kH + o] : 0.f;
+  for (int o = threadIdx.x; o < kH; o += 256) ws[o] = w4[o];
+  __syncthreads();
+  const int r = threadIdx.x;
+  if (r < kTile) {
+    float acc = 0.f;
+#pragma unroll 8
+    for (int k = 0; k < kH; ++k) acc = fmaf(Hs[r][k], ws[k], acc);
+    acc = acc + b4[0];
+    float d = 0.f;
+    if (r0 + r < M) {
+      y[r0 + r] = acc;
+      if (t) {
+        const float e = acc - t[r0 + r];
+        d = 2.f * e / (float)M;
+        dy[r0 + r] = d;
+      }
+    }
+    ds[r] = d;
+  }
+  if (!t) return;
+  __syncthreads();
+  for (int o = threadIdx.x; o < kTile * kH; o += 256) {
+    const int rr = o / kH, n = o % kH;
+    if (r0 + rr < M) {
+      float v = ds[rr] * ws[n];
+      v *= (1.f - Hs[rr][n] * Hs[rr][n]);
+      D3[(size_t)r0 * kH + o] = v;
     }
   }
 }
 
-// dZ = dH * (1 - H^2) (in place on dH)
-__global__ void tanh_back_kernel(float* dH, const float* H, long long n) {
-  long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) dH[i] *= (1.f - H[i] * H[i]);
+// sum over the rows of a column, in order: acc = fma(Z[r], s[r], acc) or acc + Z[r] (s null); rows in batches, so that
+// their loads overlap
+__device__ __forceinline__ float column_sum(const float* Z, size_t stride, int rows, const float* s) {
+  constexpr int kU = 32;
+  float acc = 0.f;
+  int r = 0;
+  for (; r + kU <= rows; r += kU) {
+    float z[kU], m[kU];
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      z[u] = Z[(size_t)(r + u) * stride];
+      m[u] = s ? s[r + u] : 1.f;
+    }
+#pragma unroll
+    for (int u = 0; u < kU; ++u) acc = s ? fmaf(z[u], m[u], acc) : acc + z[u];
+  }
+  for (; r < rows; ++r) acc = s ? fmaf(Z[(size_t)r * stride], s[r], acc) : acc + Z[(size_t)r * stride];
+  return acc;
 }
 
-// column sums (bias gradients), fixed order
-__global__ void colsum_kernel(const float* Z, int rows, int cols, float* out) {
-  int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= cols) return;
-  float s = 0.f;
-  for (int r = 0; r < rows; ++r) s += Z[(size_t)r * cols + c];
-  out[c] = s;
-}
-
-// residual r = y - t, dy = 2 r / B, loss = mean r^2 (single block, fixed order)
-__global__ void loss_kernel(const float* y, const float* t, int B, float* dy, float* loss) {
-  __shared__ double part[256];
+// Backward of one layer in one launch.  D: M x kH deltas of the layer, P: M x K its inputs, W: kH x K its weights.
+//   blocks [0, nw):   gW[n][k] = sum_r D[r][n] P[r][k], 16 x 16 outputs each
+//   next nd:          Dp[r][k] = (sum_n D[r][n] W[n][k]) (1 - P[r][k]^2), 32 x 32 outputs each (none for the first layer)
+//   next kH / 32:     gb[n] = sum_r D[r][n]
+//   and for the last layer (y) kH / 32 blocks of gw4[n] = sum_r H3[r][n] dy[r] and one of gb4 = sum dy and the loss
+struct BackArgs {
+  int M, K, nw, nd;
+  const float *D, *P, *W;
+  float *gW, *gb, *Dp;
+  const float *H3, *dy, *y, *t;
+  float *gw4, *gb4, *loss;
+};
+__global__ void __launch_bounds__(256) back_kernel(BackArgs a) {
+  __shared__ union {
+    struct {
+      float As[kTile][kChunk + 1];
+      float Bs[kChunk][kTile + 1];
+    } p;
+    struct {
+      float Ds[2][kGRows][kGTile];
+      float Ps[2][kGRows][kGTile];
+    } g;
+    double part[256];
+  } sm;
+  int b = blockIdx.x;
+  const int tid = threadIdx.x;
+  if (b < a.nw) {
+    const int kt = (a.K + kGTile - 1) / kGTile;
+    const int n0 = b / kt * kGTile, k0 = b % kt * kGTile;
+    const int n = tid / kGTile, k = tid % kGTile;
+    float acc = 0.f, rd[4], rp[4];
+    auto load = [&](int r0) {  // four rows per thread of each operand
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int r = r0 + tid / kGTile + 16 * u, c = tid % kGTile;
+        rd[u] = r < a.M ? a.D[(size_t)r * kH + n0 + c] : 0.f;
+        rp[u] = r < a.M && k0 + c < a.K ? a.P[(size_t)r * a.K + k0 + c] : 0.f;
+      }
+    };
+    auto store = [&](int buf) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        sm.g.Ds[buf][tid / kGTile + 16 * u][tid % kGTile] = rd[u];
+        sm.g.Ps[buf][tid / kGTile + 16 * u][tid % kGTile] = rp[u];
+      }
+    };
+    load(0);
+    int buf = 0;
+    for (int r0 = 0; r0 < a.M; r0 += kGRows) {
+      store(buf);
+      __syncthreads();
+      if (r0 + kGRows < a.M) load(r0 + kGRows);
+      const int rn = min(kGRows, a.M - r0);
+#pragma unroll 16
+      for (int r = 0; r < rn; ++r) acc = fmaf(sm.g.Ds[buf][r][n], sm.g.Ps[buf][r][k], acc);
+      buf ^= 1;
+    }
+    if (k0 + k < a.K) a.gW[(size_t)(n0 + n) * a.K + k0 + k] = acc + 0.f;
+    return;
+  }
+  b -= a.nw;
+  if (b < a.nd) {
+    const int r0 = b / (kH / kTile) * kTile, n0 = b % (kH / kTile) * kTile;
+    float acc[4];
+    tile_product<false>(a.D, a.M, kH, a.W, kH, r0, n0, sm.p.As, sm.p.Bs, acc);
+    const int n = n0 + tid % kTile;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int r = r0 + tid / kTile + 8 * i;
+      if (r < a.M) {
+        const float h = a.P[(size_t)r * kH + n];
+        float v = acc[i] + 0.f;
+        v *= (1.f - h * h);
+        a.Dp[(size_t)r * kH + n] = v;
+      }
+    }
+    return;
+  }
+  b -= a.nd;
+  if (b < kH / 32) {
+    if (tid < 32) a.gb[32 * b + tid] = column_sum(a.D + 32 * b + tid, kH, a.M, nullptr);
+    return;
+  }
+  b -= kH / 32;
+  if (b < kH / 32) {
+    if (tid < 32) a.gw4[32 * b + tid] = column_sum(a.H3 + 32 * b + tid, kH, a.M, a.dy) + 0.f;
+    return;
+  }
+  // loss = mean r^2: strided partial sums in FP64, added in thread order; gb4 by the last warp
   double s = 0.0;
-  for (int i = threadIdx.x; i < B; i += blockDim.x) {
-    const float r = y[i] - t[i];
-    dy[i] = 2.f * r / (float)B;
+  for (int i = tid; i < a.M; i += 256) {
+    const float r = a.y[i] - a.t[i];
     s += (double)r * r;
   }
-  part[threadIdx.x] = s;
+  sm.part[tid] = s;
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (tid == 0) {
     double tot = 0.0;
-    for (int i = 0; i < blockDim.x; ++i) tot += part[i];
-    *loss = (float)(tot / B);
+    for (int i = 0; i < 256; ++i) tot += sm.part[i];
+    *a.loss = (float)(tot / a.M);
   }
+  if (tid == 32) *a.gb4 = column_sum(a.dy, 1, a.M, nullptr);
 }
 
 // Adam (Kingma & Ba 2015) with bias correction
@@ -297,6 +442,7 @@ size_t nparams(int F) { return (size_t)kH * F + kH + 2 * ((size_t)kH * kH + kH) 
 // Network workspace on the device (layout of the packed parameters: W1 b1 W2 b2 W3 b3 w4 b4).
 struct Net {
   int F = 0, Bmax = 0;
+  float* block = nullptr;
   float *p = nullptr, *g = nullptr, *m = nullptr, *v = nullptr;
   float *X = nullptr, *H1 = nullptr, *H2 = nullptr, *H3 = nullptr, *y = nullptr, *t = nullptr, *dy = nullptr;
   float *D1 = nullptr, *D2 = nullptr, *D3 = nullptr, *loss = nullptr;
@@ -310,46 +456,38 @@ struct Net {
   float* b4() const { return w4() + kH; }
 };
 
-cudaError_t gemm(cudaStream_t s, int M, int Nn, int K, const float* A, int lda, int tA, const float* B, int ldb,
-                 int tB, float* C, int ldc, const float* bias, int act) {
-  dim3 grid((Nn + kTile - 1) / kTile, (M + kTile - 1) / kTile);
-  gemm_kernel<<<grid, 256, 0, s>>>(M, Nn, K, A, lda, tA, B, ldb, tB, C, ldc, bias, act);
+// forward pass of B rows already in net.X; output in net.y; with targets also the deltas of the last layers
+cudaError_t net_forward(const Net& n, int B, cudaStream_t s, const float* t = nullptr) {
+  const dim3 grid((B + kTile - 1) / kTile, kH / kTile);
+  layer_kernel<<<grid, 256, 0, s>>>(B, n.F, n.X, n.W1(), n.b1(), n.H1);
+  layer_kernel<<<grid, 256, 0, s>>>(B, kH, n.H1, n.W2(), n.b2(), n.H2);
+  layer_kernel<<<grid, 256, 0, s>>>(B, kH, n.H2, n.W3(), n.b3(), n.H3);
+  head_kernel<<<grid.x, 256, 0, s>>>(B, n.H3, n.w4(), n.b4(), n.y, t, n.dy, n.D3);
   return cudaGetLastError();
 }
 
-// forward pass of B rows already in net.X; output in net.y
-cudaError_t net_forward(const Net& n, int B, cudaStream_t s) {
-  cudaError_t e;
-  if ((e = gemm(s, B, kH, n.F, n.X, n.F, 0, n.W1(), n.F, 1, n.H1, kH, n.b1(), 1))) return e;
-  if ((e = gemm(s, B, kH, kH, n.H1, kH, 0, n.W2(), kH, 1, n.H2, kH, n.b2(), 1))) return e;
-  if ((e = gemm(s, B, kH, kH, n.H2, kH, 0, n.W3(), kH, 1, n.H3, kH, n.b3(), 1))) return e;
-  return gemm(s, B, 1, kH, n.H3, kH, 0, n.w4(), 1, 0, n.y, 1, n.b4(), 0);
-}
-
-// loss and gradient of B rows (targets in net.t); gradient in net.g
+// loss and gradient of B rows (targets in net.t) after net_forward with these targets; gradient in net.g
 cudaError_t net_backward(const Net& n, int B, cudaStream_t s) {
-  cudaError_t e;
   const int F = n.F;
   float* g = n.g;
   float *gW1 = g, *gb1 = g + kH * F, *gW2 = gb1 + kH, *gb2 = gW2 + kH * kH, *gW3 = gb2 + kH,
         *gb3 = gW3 + kH * kH, *gw4 = gb3 + kH, *gb4 = gw4 + kH;
-  loss_kernel<<<1, 256, 0, s>>>(n.y, n.t, B, n.dy, n.loss);
-  // output layer: gw4 = H3^T dy, gb4 = sum dy, D3 = dy w4^T
-  if ((e = gemm(s, kH, 1, B, n.H3, kH, 1, n.dy, 1, 0, gw4, 1, nullptr, 0))) return e;
-  colsum_kernel<<<1, 32, 0, s>>>(n.dy, B, 1, gb4);
-  if ((e = gemm(s, B, kH, 1, n.dy, 1, 0, n.w4(), kH, 0, n.D3, kH, nullptr, 0))) return e;
-  const long long bh = (long long)B * kH;
-  tanh_back_kernel<<<(unsigned)((bh + 255) / 256), 256, 0, s>>>(n.D3, n.H3, bh);
-  if ((e = gemm(s, kH, kH, B, n.D3, kH, 1, n.H2, kH, 0, gW3, kH, nullptr, 0))) return e;
-  colsum_kernel<<<(kH + 127) / 128, 128, 0, s>>>(n.D3, B, kH, gb3);
-  if ((e = gemm(s, B, kH, kH, n.D3, kH, 0, n.W3(), kH, 0, n.D2, kH, nullptr, 0))) return e;
-  tanh_back_kernel<<<(unsigned)((bh + 255) / 256), 256, 0, s>>>(n.D2, n.H2, bh);
-  if ((e = gemm(s, kH, kH, B, n.D2, kH, 1, n.H1, kH, 0, gW2, kH, nullptr, 0))) return e;
-  colsum_kernel<<<(kH + 127) / 128, 128, 0, s>>>(n.D2, B, kH, gb2);
-  if ((e = gemm(s, B, kH, kH, n.D2, kH, 0, n.W2(), kH, 0, n.D1, kH, nullptr, 0))) return e;
-  tanh_back_kernel<<<(unsigned)((bh + 255) / 256), 256, 0, s>>>(n.D1, n.H1, bh);
-  if ((e = gemm(s, kH, F, B, n.D1, kH, 1, n.X, F, 0, gW1, F, nullptr, 0))) return e;
-  colsum_kernel<<<(kH + 127) / 128, 128, 0, s>>>(n.D1, B, kH, gb1);
+  const int rt = (B + kTile - 1) / kTile, full = (kH / kGTile) * (kH / kGTile);
+  BackArgs a{};
+  a.M = B;
+  a.K = kH;
+  a.nw = full;
+  a.nd = rt * (kH / kTile);
+  a.D = n.D3, a.P = n.H2, a.W = n.W3(), a.gW = gW3, a.gb = gb3, a.Dp = n.D2;
+  a.H3 = n.H3, a.dy = n.dy, a.y = n.y, a.t = n.t, a.gw4 = gw4, a.gb4 = gb4, a.loss = n.loss;
+  back_kernel<<<a.nw + a.nd + 2 * (kH / 32) + 1, 256, 0, s>>>(a);
+  a.D = n.D2, a.P = n.H1, a.W = n.W2(), a.gW = gW2, a.gb = gb2, a.Dp = n.D1;
+  back_kernel<<<a.nw + a.nd + kH / 32, 256, 0, s>>>(a);
+  a.K = F;
+  a.nw = (kH / kGTile) * ((F + kGTile - 1) / kGTile);
+  a.nd = 0;
+  a.D = n.D1, a.P = n.X, a.gW = gW1, a.gb = gb1;
+  back_kernel<<<a.nw + kH / 32, 256, 0, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -359,26 +497,27 @@ cudaError_t dalloc(T** p, size_t n) {
   return cudaMalloc(reinterpret_cast<void**>(p), (n ? n : 1) * sizeof(T));
 }
 
+// one block of device memory for all buffers (256-byte parts)
 cudaError_t net_alloc(Net& n, int F, int Bmax) {
   n.F = F;
   n.Bmax = Bmax;
-  const size_t P = nparams(F);
-  cudaError_t e;
-  if ((e = dalloc(&n.p, P)) || (e = dalloc(&n.g, P)) || (e = dalloc(&n.m, P)) || (e = dalloc(&n.v, P))) return e;
-  if ((e = dalloc(&n.X, (size_t)Bmax * F)) || (e = dalloc(&n.H1, (size_t)Bmax * kH)) ||
-      (e = dalloc(&n.H2, (size_t)Bmax * kH)) || (e = dalloc(&n.H3, (size_t)Bmax * kH)))
-    return e;
-  if ((e = dalloc(&n.y, Bmax)) || (e = dalloc(&n.t, Bmax)) || (e = dalloc(&n.dy, Bmax))) return e;
-  if ((e = dalloc(&n.D1, (size_t)Bmax * kH)) || (e = dalloc(&n.D2, (size_t)Bmax * kH)) ||
-      (e = dalloc(&n.D3, (size_t)Bmax * kH)) || (e = dalloc(&n.loss, 1)))
-    return e;
+  const size_t P = nparams(F), bh = (size_t)Bmax * kH;
+  float** ptr[] = {&n.p, &n.g, &n.m, &n.v, &n.X, &n.H1, &n.H2, &n.H3, &n.y, &n.t, &n.dy, &n.D1, &n.D2, &n.D3, &n.loss};
+  const size_t len[] = {P, P, P, P, (size_t)Bmax * F, bh, bh, bh, (size_t)Bmax, (size_t)Bmax, (size_t)Bmax, bh, bh, bh, 1};
+  size_t total = 0;
+  for (size_t l : len) total += (l + 63) & ~size_t(63);
+  cudaError_t e = dalloc(&n.block, total);
+  if (e) return e;
+  float* at = n.block;
+  for (int i = 0; i < 15; ++i) {
+    *ptr[i] = at;
+    at += (len[i] + 63) & ~size_t(63);
+  }
   return cudaSuccess;
 }
 
 void net_free(Net& n) {
-  float* ptrs[] = {n.p, n.g, n.m, n.v, n.X, n.H1, n.H2, n.H3, n.y, n.t, n.dy, n.D1, n.D2, n.D3, n.loss};
-  for (float* q : ptrs)
-    if (q) cudaFree(q);
+  if (n.block) cudaFree(n.block);
   n = Net();
 }
 
@@ -553,7 +692,7 @@ extern "C" int fp_mlp_loss_grad(int device, int n_in, int batch, const float* X,
   if (cudaMemcpy(n.p, params, P * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(n.X, X, (size_t)batch * n_in * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(n.t, y, batch * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess ||
-      net_forward(n, batch, s) != cudaSuccess || net_backward(n, batch, s) != cudaSuccess ||
+      net_forward(n, batch, s, n.t) != cudaSuccess || net_backward(n, batch, s) != cudaSuccess ||
       cudaMemcpy(grad, n.g, P * sizeof(float), cudaMemcpyDeviceToHost) != cudaSuccess ||
       cudaMemcpy(loss, n.loss, sizeof(float), cudaMemcpyDeviceToHost) != cudaSuccess)
     rc = FP_ECUDA;
@@ -761,7 +900,7 @@ extern "C" int fp_surrogate_fit(fp_ctx* c, int nT, const double* T, double sb, c
     SG_TRY(cudaMemcpyAsync(drows, order.data(), order.size() * sizeof(int), cudaMemcpyHostToDevice, s));
     for (int b0 = 0; b0 + B <= nrows; b0 += B) {
       gather_kernel<<<(B * F + 255) / 256, 256, 0, s>>>(dX, F, drows + b0, B, net.X, dY, net.t);
-      SG_TRY(net_forward(net, B, s));
+      SG_TRY(net_forward(net, B, s, net.t));
       SG_TRY(net_backward(net, B, s));
       ++step;
       const float c1 = 1.f - std::pow(b1, (float)step), c2 = 1.f - std::pow(b2, (float)step);
@@ -1060,7 +1199,7 @@ extern "C" int fp_surrogate_sweep(fp_ctx* c, int nA, const double* TA, int nT, c
     SW_TRY(cudaMemcpyAsync(drows, order.data(), order.size() * sizeof(int), cudaMemcpyHostToDevice, s));
     for (int b0 = 0; b0 + B <= nrows; b0 += B) {
       gather_kernel<<<(B * F + 255) / 256, 256, 0, s>>>(dX, F, drows + b0, B, net.X, dY, net.t);
-      SW_TRY(net_forward(net, B, s));
+      SW_TRY(net_forward(net, B, s, net.t));
       SW_TRY(net_backward(net, B, s));
       ++step;
       const float c1 = 1.f - std::pow(b1, (float)step), c2 = 1.f - std::pow(b2, (float)step);

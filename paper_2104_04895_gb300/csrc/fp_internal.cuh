@@ -84,6 +84,7 @@ struct RatesArgs {
   const int* pk_start;       // [natoms + 1] groups with D != 0 by atom k, in l order
   const int* pk_grp;         // their group index | l << 24
   const int* pk_zero;        // [natoms^2] the group of (k, l) with D = 0 (phase 1), or -1
+  const float* rec32;        // [N][DenseRecord::size] records of the mixed path (fp_dense_kernel.cuh)
   const double2* psi_u;      // [nq_sel][nb][nquart][3][9] sum_alpha phi e0 of the evaluated points, or null
   const unsigned* operands;  // [N][2][Shape::kOperand] sliced eigenvectors in fragment order (fp_slices.cuh)
 };
@@ -110,6 +111,7 @@ struct Plan {
   long long n_items;
   size_t smem;
   bool pair = false, mirror = false;  // the pair kernel; with a slot per (evaluated point, q')
+  bool dense = false;                 // the dense kernel of the mixed path
   bool sliced = false;                // its contractions on the tensor cores
   bool operands = false;              // with the sliced eigenvectors in the scratch
   bool psi_u = false;                 // its Psi prologue from the table U
@@ -118,7 +120,7 @@ struct Plan {
 };
 
 // Device working memory of one rates call (owned by the caller of run_rates), in the order of scratch_sizes.
-constexpr int kScratchParts = 18;
+constexpr int kScratchParts = 19;
 constexpr int kScratchPartial = 7;  // index of the per-item partial sums
 constexpr int kCounters = 10;       // queue, accepted ++, +-, --, vertex entries, terms evaluated, wait timeouts,
                                     // iterations, pairs, spare
@@ -140,6 +142,7 @@ struct Scratch {
   float2* twf;                   // [L]
   float* wtf;                    // [nT][N*nb][3]
   double2* psi_u;                // [nq_sel][nb][nquart][3][9] (pair kernel, where it fits)
+  float* rec32;                  // [N][DenseRecord::size] (dense mixed kernel)
   unsigned* operands;            // [N][2][Shape::kOperand] (sliced pair kernel)
 };
 

@@ -1,12 +1,14 @@
 // Host side of the rate path: FP32 prep kernel, fixed-order reduction, tile plan and the launch routine
 // shared by fp_rates4, fp_rates4_device and fp_rates4_noalloc.  The rate kernel itself is in
 // fp_rates_kernel.cuh.
+#include "fp_dense_kernel.cuh"
 #include "fp_pair_kernel.cuh"
 
 namespace fp {
 // kernel pointers of the instantiations (fp_pair_*.cu, fp_rates_*.cu)
 const void* pair_kernel_f64(int nb, int maxt, bool sliced);
 const void* pair_kernel_df(int nb, int maxt);
+const void* dense_kernel_f32(int nb, int maxt);
 const void* rates_kernel_f64(int nb, int maxt);
 const void* rates_kernel_f32(int nb, int maxt);
 const void* rates_kernel_f32_tc(int nb, int maxt);
@@ -139,6 +141,42 @@ __global__ void operand_kernel(const double2* evec, int N, unsigned* out) {
   }
 }
 
+// Records of the dense mixed kernel, one block per grid point: the FP32 tables of prep_kernel and the group phases
+// exp(i k.D_g) of the point
+__global__ void record_kernel(RatesArgs a, float* out) {
+  const int q = blockIdx.x, nb = a.nb, nT = a.nT;
+  const DenseRecord r = make_record(nb, a.G, nT);
+  const int g[3] = {q / (a.grid[1] * a.grid[2]), (q / a.grid[2]) % a.grid[1], q % a.grid[2]};
+  float* o = out + (size_t)q * r.size;
+  for (int i = threadIdx.x; i < nb * nb; i += blockDim.x) {
+    const float2 e = a.evf[(size_t)q * nb * nb + i];
+    o[r.E + 2 * i] = e.x;
+    o[r.E + 2 * i + 1] = e.y;
+  }
+  for (int i = threadIdx.x; i < a.G; i += blockDim.x) {
+    const int* gm = a.gmeta + 5 * i;
+    int e = 0;  // each term is below L, so e < 3 L
+    for (int d = 0; d < 3; ++d) e += a.Lfac[d] * wrapi(g[d] * gm[2 + d], a.grid[d]);
+    while (e >= a.L) e -= a.L;
+    const float2 t = a.twf[e];
+    o[r.Tw + 2 * i] = t.x;
+    o[r.Tw + 2 * i + 1] = t.y;
+  }
+  for (int i = threadIdx.x; i < nb; i += blockDim.x) {
+    o[r.H + i] = a.omh[(size_t)q * nb + i];
+    o[r.L + i] = a.oml[(size_t)q * nb + i];
+  }
+  for (int i = threadIdx.x; i < 3 * nb; i += blockDim.x) {
+    o[r.VH + i] = a.velh[(size_t)q * nb * 3 + i];
+    o[r.VL + i] = a.vell[(size_t)q * nb * 3 + i];
+  }
+  for (int i = threadIdx.x; i < nT * nb; i += blockDim.x) {
+    const float* w = a.wtf + 3 * ((size_t)(i / nb) * a.N * nb + (size_t)q * nb + i % nb);
+    o[r.W + 2 * i] = w[1];
+    o[r.W + 2 * i + 1] = w[2];
+  }
+}
+
 // U[qi][j0][Q][beta][gamma theta] = sum_alpha phi_Q e_{i alpha}(q, j0) of the evaluated points: the part of the pair
 // kernel's Psi that every partner q' of q shares
 __global__ void psi_u_kernel(RatesArgs a, double2* out) {
@@ -166,17 +204,19 @@ __global__ void fill_kernel(double* p, long long n, double v) {
 }
 
 // kernel for (precision, nb, number of temperatures, tensor cores): one accumulator per temperature, 1 or up to 8
-const void* rates_kernel_ptr(int precision, int nb, int nS, bool tc, bool pair, bool sliced) {
+const void* rates_kernel_ptr(int precision, int nb, int nS, bool tc, bool pair, bool sliced, bool dense) {
   const int maxt = nS == 1 ? 1 : nS == 2 && pair ? 2 : kMaxT;
   if (pair)
     return precision == FP_PREC_DOUBLE_FLOAT ? pair_kernel_df(nb, maxt) : pair_kernel_f64(nb, maxt, sliced);
+  if (dense) return dense_kernel_f32(nb, maxt);
   if (tc) return precision == FP_PREC_MIXED ? rates_kernel_f32_tc(nb, maxt) : nullptr;
   if (precision == FP_PREC_DOUBLE_FLOAT) return rates_kernel_df(nb, maxt);
   return precision == FP_PREC_FP64 ? rates_kernel_f64(nb, maxt) : rates_kernel_f32(nb, maxt);
 }
 
 size_t smem_bytes(int precision, int nb, int J, int G, int nquart, int nT, int nS, int threads, bool tc, bool pair,
-                  bool sliced) {
+                  bool sliced, bool dense) {
+  if (dense) return make_dense_carve(nb, J, G, nquart, nT, threads).total;
   if (pair) return make_pair_carve(nb, J, G, nquart, nT, nS, threads, sliced).bytes();
   const bool f32 = precision == FP_PREC_MIXED;  // the double-float path has the FP64 path's shared memory
   Carve c = make_carve(nb, J, G, nquart, nT, threads, f32);
@@ -185,8 +225,8 @@ size_t smem_bytes(int precision, int nb, int J, int G, int nquart, int nT, int n
 }
 
 int max_ctas_per_sm(int precision, int nb, int nS, int threads, size_t smem, bool tc, bool pair,
-                    bool sliced) {
-  const void* k = rates_kernel_ptr(precision, nb, nS, tc, pair, sliced);
+                    bool sliced, bool dense) {
+  const void* k = rates_kernel_ptr(precision, nb, nS, tc, pair, sliced, dense);
   if (!k) return 0;
   if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
   int n = 0;
@@ -265,7 +305,7 @@ int make_selection(const fp_ctx* c, const fp_rates_opts& o, bool fold_allowed, S
 }
 
 static int plan_form(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, size_t partial_budget, Plan* p,
-                     std::string* err, bool pair, bool sliced, bool mirror, int split) {
+                     std::string* err, bool pair, bool sliced, bool mirror, int split, bool dense = false) {
   const int nS = nT * (split == 1 ? 2 : split == 2 ? 3 : 1);
   const int N = c->N, nb = c->nb;
   const bool tc = o.tensor_cores != 0;
@@ -273,7 +313,7 @@ static int plan_form(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, 
     *err = "tensor_cores needs the mixed precision and 6 branches";
     return FP_EINVAL;
   }
-  if (!rates_kernel_ptr(o.precision, nb, nS, tc, pair, sliced)) {
+  if (!rates_kernel_ptr(o.precision, nb, nS, tc, pair, sliced, dense)) {
     *err = "unsupported number of branches";
     return FP_EINVAL;
   }
@@ -294,7 +334,7 @@ static int plan_form(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, 
     const size_t room = pair ? (pair_blocks_for(nb) == 1 ? 227 : 112) * 1024 : 110 * 1024;
     J = nb;
     while (J > 1 && (J * nb * nb > most ||
-                     smem_bytes(o.precision, nb, J, c->G, c->nquart, nT, nS, pair ? (J * nb * nb + 31) / 32 * 32 : most, tc, pair, sliced) > room)) {
+                     smem_bytes(o.precision, nb, J, c->G, c->nquart, nT, nS, pair ? (J * nb * nb + 31) / 32 * 32 : most, tc, pair, sliced, dense) > room)) {
       int nj = J - 1;
       while (nj > 1 && nb % nj) --nj;
       J = nj;
@@ -353,12 +393,12 @@ static int plan_form(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, 
     *err = "per-item partial sums do not fit the scratch";
     return FP_EINVAL;
   }
-  const size_t smem = smem_bytes(o.precision, nb, J, c->G, c->nquart, nT, nS, threads, tc, pair, sliced);
+  const size_t smem = smem_bytes(o.precision, nb, J, c->G, c->nquart, nT, nS, threads, tc, pair, sliced, dense);
   if (smem > 227 * 1024) {
     *err = "tile does not fit in shared memory";
     return FP_EINVAL;
   }
-  const int per_sm = max_ctas_per_sm(o.precision, nb, nS, threads, smem, tc, pair, sliced);
+  const int per_sm = max_ctas_per_sm(o.precision, nb, nS, threads, smem, tc, pair, sliced, dense);
   if (per_sm < 1) {
     *err = "kernel tile cannot be resident on an SM";
     return FP_EINVAL;
@@ -378,6 +418,7 @@ static int plan_form(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, 
   p->smem = smem;
   p->pair = pair;
   p->sliced = sliced;
+  p->dense = dense;
   p->nS = nS;
   p->split = split;
   p->operands = sliced;
@@ -411,6 +452,14 @@ int plan_rates(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, size_t
     const int rc = plan_form(c, o, nT, sel, partial_budget, p, err, true, false, form == kPairMirror, split);
     if (rc != FP_EINVAL) return rc;
   }
+  // The mixed path's dense kernel evaluates the ordered sums for three and six branches.  With twelve, 144 rows are one
+  // j0 per block and both the columns and the unrolled loop spill: LiCoO2 5x4x4 63.8 ms against 62.6 for the ordered
+  // kernel, 4x3x3 with three temperatures 10.8 against 8.0, so they stay there, as do a tile or a scratch without room
+  // for the records.
+  if (form != kOrdered && o.precision == FP_PREC_MIXED && !o.tensor_cores) {
+    const int rc = plan_form(c, o, nT, sel, partial_budget, p, err, false, false, false, 0, true);
+    if (rc != FP_EINVAL) return rc;
+  }
   return plan_form(c, o, nT, sel, partial_budget, p, err, false, false, false, 0);
 }
 
@@ -432,6 +481,7 @@ void scratch_sizes(const fp_ctx* c, const Plan& p, int nT, size_t s[kScratchPart
   s[13] = up256((size_t)81 * c->nquart * sizeof(float));
   s[14] = up256((size_t)c->L * sizeof(float2));
   s[15] = up256(3 * nm * nT * sizeof(float));
+  s[18] = p.dense ? up256((size_t)c->N * make_record(c->nb, c->G, nT).size * sizeof(float)) : 0;
   s[17] = p.psi_u ? up256((size_t)p.nq_sel * c->nb * c->nquart * 27 * sizeof(double2)) : 0;
   s[16] = p.operands ? up256((size_t)c->N * operand_words(c->nb) * sizeof(unsigned)) : 0;
 }
@@ -461,6 +511,7 @@ Scratch carve_scratch(unsigned char* b, const size_t sz[kScratchParts]) {
   sc.wtf = reinterpret_cast<float*>(b + off[15]);
   sc.operands = reinterpret_cast<unsigned*>(b + off[16]);
   sc.psi_u = reinterpret_cast<double2*>(b + off[17]);
+  sc.rec32 = reinterpret_cast<float*>(b + off[18]);
   return sc;
 }
 
@@ -532,6 +583,7 @@ int run_rates(fp_ctx* c, const fp_rates_opts& o, const Selection& sel, const Pla
   a.twf = sc.twf;
   a.wtf = sc.wtf;
   a.operands = sc.operands;
+  a.rec32 = sc.rec32;
   a.psi_u = p.psi_u ? sc.psi_u : nullptr;
   a.sb = sb;
   a.window = o.window;
@@ -569,7 +621,7 @@ int run_rates(fp_ctx* c, const fp_rates_opts& o, const Selection& sel, const Pla
   const double pref = unit_stride > 0
                           ? (double)unit_stride / ((double)N * (double)N)
                           : kPi * kHbar * kHbar * conv * conv * conv * conv / (8.0 * (double)N * (double)N);
-  const void* k = rates_kernel_ptr(o.precision, nb, p.nS, o.tensor_cores != 0, p.pair, p.sliced);
+  const void* k = rates_kernel_ptr(o.precision, nb, p.nS, o.tensor_cores != 0, p.pair, p.sliced, p.dense);
   // the device part of a rate set: Bose weights, FP32 tables, cleared counters and output, the persistent
   // rate kernel and the reduction
   auto enqueue = [&]() -> cudaError_t {
@@ -588,6 +640,10 @@ int run_rates(fp_ctx* c, const fp_rates_opts& o, const Selection& sel, const Pla
     prep_kernel<<<4 * 152, 256, 0, s>>>(a, sc.omh, sc.oml, sc.velh, sc.vell, sc.evf, sc.qfcf, sc.twf, sc.wtf,
                                         want_f32);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if (p.dense) {
+      record_kernel<<<N, 128, 0, s>>>(a, sc.rec32);
+      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
     if (a.psi_u && p.nq_sel > 0) {
       psi_u_kernel<<<8 * 152, 256, 0, s>>>(a, sc.psi_u);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;

@@ -188,6 +188,7 @@ void fp_free(fp_ctx* c) {
   dfree(c->d_pk_start);
   dfree(c->d_pk_grp);
   dfree(c->d_pk_zero);
+  dfree(c->d_terms);
   dfree(c->d_tw);
   dfree(c->d_omega);
   dfree(c->d_evec);
@@ -369,6 +370,30 @@ int fp_init(fp_ctx** out, const double lattice[9], int natoms, const double* fra
       }
     pk_start[k + 1] = (int)pk_grp.size();
   }
+  // and the quartets of a group that share (atom j, R_j - R_l): their phases differ by one of q alone, so the table U of
+  // the pair kernel holds their sum (58 quartets are 26 terms on diamond, 172 are 76 on LiCoO2)
+  std::vector<int> terms;
+  {
+    std::map<std::tuple<int, int, int, int, int>, std::vector<int>> tid;  // sorted by group
+    for (int b = 0; b < n_fc4; ++b) {
+      const fp_fc4& f = fc4[b];
+      tid[std::make_tuple(qgroup[b], f.j, f.Rj[0] - f.Rl[0], f.Rj[1] - f.Rl[1], f.Rj[2] - f.Rl[2])].push_back(b);
+    }
+    const int G = c->G, nt = c->nterm = (int)tid.size();
+    terms.assign((size_t)G + 1 + 4 * (size_t)nt + nt + 1 + n_fc4, 0);
+    int *start = terms.data(), *meta = start + G + 1, *qstart = meta + 4 * (size_t)nt, *list = qstart + nt + 1;
+    int t = 0, n = 0;
+    for (const auto& kv : tid) {
+      start[std::get<0>(kv.first) + 1]++;
+      meta[4 * t] = std::get<1>(kv.first);
+      meta[4 * t + 1] = std::get<2>(kv.first);
+      meta[4 * t + 2] = std::get<3>(kv.first);
+      meta[4 * t + 3] = std::get<4>(kv.first);
+      for (int b : kv.second) list[n++] = b;
+      qstart[++t] = n;
+    }
+    for (int gi = 0; gi < G; ++gi) start[gi + 1] += start[gi];
+  }
   c->leg_symmetric = c->G < (1 << 24) && leg_symmetric(n_fc4, fc4);
   INIT_CUDA(dalloc(&c->d_qmeta, qmeta.size()));
   INIT_CUDA(dalloc(&c->d_qfc, qfc.size()));
@@ -381,6 +406,8 @@ int fp_init(fp_ctx** out, const double lattice[9], int natoms, const double* fra
   INIT_CUDA(dalloc(&c->d_pk_start, pk_start.size()));
   INIT_CUDA(dalloc(&c->d_pk_grp, pk_grp.size()));
   INIT_CUDA(dalloc(&c->d_pk_zero, pk_zero.size()));
+  INIT_CUDA(dalloc(&c->d_terms, terms.size()));
+  INIT_CUDA(cudaMemcpyAsync(c->d_terms, terms.data(), terms.size() * sizeof(int), cudaMemcpyHostToDevice, s));
   INIT_CUDA(cudaMemcpyAsync(c->d_pk_start, pk_start.data(), pk_start.size() * sizeof(int), cudaMemcpyHostToDevice, s));
   INIT_CUDA(cudaMemcpyAsync(c->d_pk_grp, pk_grp.data(), pk_grp.size() * sizeof(int), cudaMemcpyHostToDevice, s));
   INIT_CUDA(cudaMemcpyAsync(c->d_pk_zero, pk_zero.data(), pk_zero.size() * sizeof(int), cudaMemcpyHostToDevice, s));

@@ -84,8 +84,14 @@ struct RatesArgs {
   const int* pk_start;       // [natoms + 1] groups with D != 0 by atom k, in l order
   const int* pk_grp;         // their group index | l << 24
   const int* pk_zero;        // [natoms^2] the group of (k, l) with D = 0 (phase 1), or -1
+  // terms of the table psi_u, by group: quartets of one group with the same (atom j, R_j - R_l)
+  int nterm;
+  const int* term_start;     // [G + 1]
+  const int* term_meta;      // [nterm] atom j, R_j - R_l
+  const int* term_qstart;    // [nterm + 1]
+  const int* term_q;         // [nquart]
   const float* rec32;        // [N][DenseRecord::size] records of the mixed path (fp_dense_kernel.cuh)
-  const double2* psi_u;      // [nq_sel][nb][nquart][3][9] sum_alpha phi e0 of the evaluated points, or null
+  const double2* psi_u;      // [nq_sel][nb][nterm][3][9] table U of the evaluated points (psi_u_kernel), or null
   const unsigned* operands;  // [N][2][Shape::kOperand] sliced eigenvectors in fragment order (fp_slices.cuh)
 };
 
@@ -141,7 +147,7 @@ struct Scratch {
   float* qfcf;                   // [nquart*81]
   float2* twf;                   // [L]
   float* wtf;                    // [nT][N*nb][3]
-  double2* psi_u;                // [nq_sel][nb][nquart][3][9] (pair kernel, where it fits)
+  double2* psi_u;                // [nq_sel][nb][nterm][3][9] (pair kernel, where it fits)
   float* rec32;                  // [N][DenseRecord::size] (dense mixed kernel)
   unsigned* operands;            // [N][2][Shape::kOperand] (sliced pair kernel)
 };
@@ -175,6 +181,8 @@ struct fp_ctx {
   int* d_pk_start = nullptr;  // groups as the pair kernel walks them (RatesArgs)
   int* d_pk_grp = nullptr;
   int* d_pk_zero = nullptr;
+  int nterm = 0;
+  int* d_terms = nullptr;  // term_start, term_meta, term_qstart, term_q (RatesArgs) one after the other
   bool leg_symmetric = false;  // the quartet list obeys the transposition symmetry (Eq. TS)
   int* d_bzm = nullptr;  // [N][3] Brillouin-zone shifts (bz_shifts)
   // third-order force constants (fp_set_fc3), by group (atoms j, k and D = Rj - Rk)

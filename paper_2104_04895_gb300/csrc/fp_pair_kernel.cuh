@@ -195,13 +195,13 @@ __device__ __forceinline__ double add_signed(double x, double y, bool plus) {
   return __dadd_rn(x, __hiloint2double(__double2hiint(y) ^ (plus ? 0 : 0x80000000), __double2loint(y)));
 }
 
-// exp_neg64 (fp_rates_kernel.cuh) with the range test and the rounding of v to k kept off the FP64 compare and convert
-// instructions: v + 1.5 2^52 holds k = rint(v) in its low bits
-__device__ __forceinline__ double pair_exp_neg64(double v, const double* tab) {
-  if (__double2hiint(v) > 0x40700000) return exp(-v * kExpH);  // v >= 256 (1 + 2^-20) (also NaN)
-  const double vm = __dadd_rn(v, slices::kMagic);
+// exp_neg64 (fp_rates_kernel.cuh) of v = x^2 with the range test and the rounding of v to k kept off the FP64 compare and
+// convert instructions: x^2 + 1.5 2^52 holds k = rint(v) in its low bits; k - x^2 is rounded once
+__device__ __forceinline__ double pair_exp_neg64(double x, const double* tab) {
+  if ((__double2hiint(x) & 0x7fffffff) > 0x40300000) return exp(-(x * x) * kExpH);  // |x| >= 16 (1 + 2^-20) (also NaN)
+  const double vm = fma(x, x, slices::kMagic);
   const int k = __double2loint(vm);
-  const double t = __dsub_rn(__dsub_rn(vm, slices::kMagic), v);
+  const double t = fma(-x, x, __dsub_rn(vm, slices::kMagic));
   double p = (1.0 / 120.0) / 1073741824.0;
   p = fma(p, t, (1.0 / 24.0) / 16777216.0);
   p = fma(p, t, (1.0 / 6.0) / 262144.0);
@@ -213,7 +213,7 @@ __device__ __forceinline__ double pair_exp_neg64(double v, const double* tab) {
 
 // exp of the second order of {c, d} averaged in (rare: out of line)
 __device__ __noinline__ double pair_two_orders(double ex, double z8, const double* tab) {
-  return 0.5 * (ex + pair_exp_neg64(z8 * z8, tab));
+  return 0.5 * (ex + pair_exp_neg64(z8, tab));
 }
 __device__ __noinline__ float2 pair_two_orders(float2 ex, float2 z8, const float2* tab) {
   const float2 m = df_add(ex, df_exp_neg64(df_mul(z8, z8), tab));
@@ -267,6 +267,8 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
 
   const bool has_row = tid < rows;
   const int rjj = tid / NB2, rj1 = (tid / NB) % NB, rc = tid % NB;
+  // complex elements of the block of T, free until Psi is complete
+  const int kTabU = SL ? (nthr / 32) * 32 * (NB == 6 ? 36 : 76) / 4 : J * NB * (NB2 + 1);
   const size_t NM = (size_t)N * NB;
   const bool f32_sigma = a.dq_mode == 0;
   const double inv_sbdq = 1.0 / (a.sb * a.dq);
@@ -326,7 +328,15 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
         sH1[o] = a.omh[k1 * NB + o];
         sMb[o] = mir && w > 0.0 ? a.mult[rq * NB + o] : 0;
       }
-      for (int Q = tid; Q < a.nquart; Q += nthr) {
+      if (a.psi_u)
+        for (int t = tid; t < a.nterm; t += nthr) {
+          const int* m = a.term_meta + 4 * t;
+          int e = 0;  // each term is below L, so e < 3 L
+          for (int d = 0; d < 3; ++d) e += a.Lfac[d] * wrapi(g1[d] * m[1 + d], a.grid[d]);
+          while (e >= a.L) e -= a.L;
+          sTwQ[t] = ld_tw<double>(a, e);
+        }
+      for (int Q = tid; Q < (a.psi_u ? 0 : a.nquart); Q += nthr) {
         const int* m = a.qmeta + 9 * Q;
         int e = 0;  // each term is below L, so e < 3 L
         for (int d = 0; d < 3; ++d) e += a.Lfac[d] * wrapi(g1[d] * m[3 + d] - (g[d] + g1[d]) * m[6 + d], a.grid[d]);
@@ -345,23 +355,30 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
       // Psi[jj][j1][grp][gt] (see fp_rates_kernel.cuh): one thread per (jj, j1, grp) and block of three (gamma, theta)
       constexpr int kGtb = 3;
       if (a.psi_u && !unit && any) {
-        // with U = sum_alpha phi e0 of this q at hand: Psi = sum_Q sum_beta (tw1_Q e1_beta) U, 36 FMAs per quartet and
-        // three (gamma, theta) instead of 90
-        const double2* U = a.psi_u + ((size_t)qi * NB + j0b) * a.nquart * 27;
+        // with U of this q at hand (psi_u_kernel): Psi = sum over the group's terms and beta of exp(i q'.(R_j - R_l)) e1_beta
+        // U, 36 FMAs per term and three (gamma, theta) instead of 90 per quartet
+        const double2* U = a.psi_u + ((size_t)qi * NB + j0b) * a.nterm * 27;
+        // exp(i q'.(R_j - R_l)) e1 [j1][term][beta] where it fits into the block of T
+        const bool table = 3 * NB * a.nterm <= kTabU;
+        if (table) {
+          for (int o = tid; o < 3 * NB * a.nterm; o += nthr) {
+            const int t = (o / 3) % a.nterm;
+            sT[o] = cmul(sTwQ[t], sE1[(o / (3 * a.nterm)) * NB + 3 * a.term_meta[4 * t] + o % 3]);
+          }
+          __syncthreads();
+        }
         for (int o = tid; o < J * NB * G * (9 / kGtb); o += nthr) {
           const int gb = o % (9 / kGtb), jr = (o / (9 / kGtb)) % (J * NB), grp = o / ((9 / kGtb) * J * NB);
           const int j1 = jr % NB, jj = jr / NB;
           C sum[kGtb];
 #pragma unroll
           for (int u = 0; u < kGtb; ++u) sum[u] = cmk<double>(0, 0);
-          for (int qq = a.grp_qstart[grp]; qq < a.grp_qstart[grp + 1]; ++qq) {
-            const int Q = a.grp_q[qq];
-            const C tq = sTwQ[Q];
-            const double2* uq = U + ((size_t)jj * a.nquart + Q) * 27 + gb * kGtb;
-            const C* e1 = sE1 + j1 * NB + 3 * a.qmeta[9 * Q + 1];
+          for (int t = a.term_start[grp]; t < a.term_start[grp + 1]; ++t) {
+            const double2* uq = U + ((size_t)jj * a.nterm + t) * 27 + gb * kGtb;
+            const C* e1 = table ? sT + 3 * ((size_t)j1 * a.nterm + t) : sE1 + j1 * NB + 3 * a.term_meta[4 * t];
 #pragma unroll
             for (int be = 0; be < 3; ++be) {
-              const C et = cmul(tq, e1[be]);
+              const C et = table ? e1[be] : cmul(sTwQ[t], e1[be]);
 #pragma unroll
               for (int u = 0; u < kGtb; ++u) {
                 const double2 v = uq[be * 9 + u];
@@ -1008,7 +1025,7 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
                   }
                   if (__double2hiint(iv8) >= 0) {  // not -1 (delta := 1)
                     const double x8 = dw * iv8;
-                    double ex = pair_exp_neg64(x8 * x8, sExpT);
+                    double ex = pair_exp_neg64(x8, sExpT);
                     if (__double2hiint(iv8) > 0x40bf4000 && orders)  // 8 / sigma > 8000
                       ex = pair_two_orders(ex, add_signed(add_signed(wx, y2, plus1), y1, plus2) * iv8, sExpT);
                     gv *= ex;
@@ -1020,10 +1037,15 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
               }
               __syncwarp();
               int p = pos0 - r0;
-              for (unsigned b = left0 & ~left; b; b &= b - 1) {
+              // the three sums one after the other: a warp runs the longest list of each, not all three per position
+              const unsigned done = left0 & ~left;
+              constexpr unsigned kM = (1u << kPairGroup) - 1u;
+              for (unsigned b = done & ((1u << (3 * kPairGroup)) - 1u); b; b &= b - 1) {
                 const int bit = __ffs(b) - 1;
                 add(sVal[p++], bit / kPairGroup, y * NB + jb + bit % kPairGroup);
               }
+              for (unsigned b = done >> (3 * kPairGroup) & kM; b; b &= b - 1) add(sVal[p++], 3, y * NB + jb + __ffs(b) - 1);
+              for (unsigned b = done >> (4 * kPairGroup) & kM; b; b &= b - 1) add(sVal[p++], 4, y * NB + jb + __ffs(b) - 1);
               __syncwarp();
             }
           }

@@ -177,21 +177,33 @@ __global__ void record_kernel(RatesArgs a, float* out) {
   }
 }
 
-// U[qi][j0][Q][beta][gamma theta] = sum_alpha phi_Q e_{i alpha}(q, j0) of the evaluated points: the part of the pair
-// kernel's Psi that every partner q' of q shares
+// U[qi][j0][term][beta][gamma theta] = sum over the term's quartets Q and alpha of exp(-i q.R_l) phi_Q e_{i alpha}(q, j0)
+// of the evaluated points: the part of the pair kernel's Psi that every partner q' of q shares.  The quartets of a term
+// have the same phase exp(i q'.(R_j - R_l)), so a pair reads and multiplies their sum: 26 terms instead of 58 quartets on
+// diamond (3x3x3 0.66 -> 0.56 ms, 5x4x5 13.9 -> 13.1), 76 instead of 172 on LiCoO2 (3x3x3 8.48 -> 7.63 ms).
 __global__ void psi_u_kernel(RatesArgs a, double2* out) {
-  const long long n = (long long)a.nq_sel * a.nb * a.nquart * 27;
+  const long long n = (long long)a.nq_sel * a.nb * a.nterm * 27;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const int c = (int)(i % 27), Q = (int)((i / 27) % a.nquart), j0 = (int)((i / (27LL * a.nquart)) % a.nb);
-    const int q = a.qlist[i / (27LL * a.nquart * a.nb)];
-    const double2* e = a.evec + ((size_t)q * a.nb + j0) * a.nb + 3 * a.qmeta[9 * Q];
-    const double* f = a.qfc + 81 * (size_t)Q + c;
-    double re = 0.0, im = 0.0;
-    for (int al = 0; al < 3; ++al) {
-      re = fma(f[27 * al], e[al].x, re);
-      im = fma(f[27 * al], e[al].y, im);
+    const int c = (int)(i % 27), t = (int)((i / 27) % a.nterm), j0 = (int)((i / (27LL * a.nterm)) % a.nb);
+    const int q = a.qlist[i / (27LL * a.nterm * a.nb)];
+    const int g[3] = {q / (a.grid[1] * a.grid[2]), (q / a.grid[2]) % a.grid[1], q % a.grid[2]};
+    Cx<double> sum = cmk<double>(0, 0);
+    for (int k = a.term_qstart[t]; k < a.term_qstart[t + 1]; ++k) {
+      const int Q = a.term_q[k];
+      const int* m = a.qmeta + 9 * Q;
+      const double2* e = a.evec + ((size_t)q * a.nb + j0) * a.nb + 3 * m[0];
+      const double* f = a.qfc + 81 * (size_t)Q + c;
+      Cx<double> v = cmk<double>(0, 0);
+      for (int al = 0; al < 3; ++al) {
+        v.re = fma(f[27 * al], e[al].x, v.re);
+        v.im = fma(f[27 * al], e[al].y, v.im);
+      }
+      int w = 0;  // each term is below L, so w < 3 L
+      for (int d = 0; d < 3; ++d) w += a.Lfac[d] * wrapi(-g[d] * m[6 + d], a.grid[d]);
+      while (w >= a.L) w -= a.L;
+      cfma(sum, ld_tw<double>(a, w), v);
     }
-    out[i] = make_double2(re, im);
+    out[i] = make_double2(sum.re, sum.im);
   }
 }
 
@@ -369,8 +381,8 @@ static int plan_form(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, 
     mirror = cudaMemGetInfo(&mem_free, &mem_total) == cudaSuccess && mirror_bytes < mem_free / 2;
   }
   if (mirror && o.k1_tile <= 0 && t1_tuned <= 0) t1 = 1;
-  // the table U of the Psi prologue, where a call may take the memory for it (2 MB on diamond 3^3, 308 MB on 16^3)
-  const size_t u_bytes = (size_t)nq_sel * nb * c->nquart * 27 * sizeof(double2);
+  // the table U of the Psi prologue, where a call may take the memory for it (1 MB on diamond 3^3, 138 MB on 16^3)
+  const size_t u_bytes = (size_t)nq_sel * nb * c->nterm * 27 * sizeof(double2);
   p->psi_u = pair && !partial_budget && u_bytes > 0 && u_bytes <= (size_t(512) << 20);
   if (o.k1_tile <= 0 && partial_budget && !mirror)
     while (t1 < N && part_bytes(t1) > partial_budget) t1 = t1 < 8 ? t1 + 1 : t1 + t1 / 4;
@@ -482,7 +494,7 @@ void scratch_sizes(const fp_ctx* c, const Plan& p, int nT, size_t s[kScratchPart
   s[14] = up256((size_t)c->L * sizeof(float2));
   s[15] = up256(3 * nm * nT * sizeof(float));
   s[18] = p.dense ? up256((size_t)c->N * make_record(c->nb, c->G, nT).size * sizeof(float)) : 0;
-  s[17] = p.psi_u ? up256((size_t)p.nq_sel * c->nb * c->nquart * 27 * sizeof(double2)) : 0;
+  s[17] = p.psi_u ? up256((size_t)p.nq_sel * c->nb * c->nterm * 27 * sizeof(double2)) : 0;
   s[16] = p.operands ? up256((size_t)c->N * operand_words(c->nb) * sizeof(unsigned)) : 0;
 }
 
@@ -546,6 +558,11 @@ int run_rates(fp_ctx* c, const fp_rates_opts& o, const Selection& sel, const Pla
   a.L = c->L;
   a.G = c->G;
   a.nquart = c->nquart;
+  a.nterm = c->nterm;
+  a.term_start = c->d_terms;
+  a.term_meta = a.term_start + c->G + 1;
+  a.term_qstart = a.term_meta + 4 * (size_t)c->nterm;
+  a.term_q = a.term_qstart + c->nterm + 1;
   for (int d = 0; d < 3; ++d) {
     a.grid[d] = c->grid[d];
     a.Lfac[d] = c->L / c->grid[d];
@@ -748,7 +765,7 @@ void fill_stats(const fp_ctx* c, const fp_rates_opts& o, const Selection& sel, c
   const double J = p.J;
   const double pairs = 0.5 * (double)N * (double)(N + 1);
   const double per_pair = 8.0 * (9.0 * J * nb * c->G + J * (double)nb * nb * nb * nb);
-  const double prolog = 8.0 * 9.0 * J * nb * 9.0 * c->nquart;
+  const double prolog = p.psi_u ? 8.0 * 27.0 * J * nb * c->nterm : 8.0 * 9.0 * J * nb * 9.0 * c->nquart;
   st->flops = p.pair ? (double)counts[7] * per_pair + (double)counts[8] * prolog
                      : (double)sel.active_chunks * (pairs * per_pair + (double)N * prolog);
   st->flops += 8.0 * nb * st->vertex_entries;

@@ -295,10 +295,7 @@ __global__ void __launch_bounds__(threads3(NB), NB == 12 ? 1 : 2) rates3_kernel(
         const double dw = __dsub_rn(pr ? __dsub_rn(w, w1) : __dadd_rn(w, w1), sW2[e2]);
         double v = (W.re * W.re + W.im * W.im) * sF[e];
         const double iv8 = sIv8[e];
-        if (__double2hiint(iv8) >= 0) {
-          const double x8 = dw * iv8;
-          v *= pair_exp_neg64(x8 * x8, sExpT);
-        }
+        if (__double2hiint(iv8) >= 0) v *= pair_exp_neg64(dw * iv8, sExpT);
         sVal[i] = v;
       }
       __syncwarp();

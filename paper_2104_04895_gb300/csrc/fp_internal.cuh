@@ -30,6 +30,7 @@ struct RatesArgs {
   int N, nb, natoms, nT, L, G, nquart;
   int grid[3], Lfac[3];
   int J, t1, nchunk, ntile, nq_sel;
+  int nseg;                  // items that share a pair's q'' (pair kernel)
   long long n_items;
   const int* qlist;          // [nq_sel] the q-points the kernel evaluates (work item -> q)
   const unsigned char* mult; // [N*nb] selected modes each evaluated row stands for: 0, 1, or 2 when the row's
@@ -114,6 +115,7 @@ struct Selection {
 // Tile plan of one rates call.
 struct Plan {
   int J, threads, t1, nchunk, ntile, nq_sel, ctas;
+  int nseg = 1;                       // items per pair (pair kernel): its q'' dealt in turn
   long long n_items;
   size_t smem;
   bool pair = false, mirror = false;  // the pair kernel; with a slot per (evaluated point, q')

@@ -292,7 +292,7 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
     const int chunk = (int)(item % a.nchunk);
     const long long rest = item / a.nchunk;
     const int qi = (int)(rest % a.nq_sel);
-    const int tile = (int)(rest / a.nq_sel);
+    const int tile = (int)((rest / a.nq_sel) % a.ntile), seg = (int)(rest / a.nq_sel / a.ntile);
     const int q = a.qlist[qi];
     const int j0b = chunk * J;
     const int g[3] = {q / (a.grid[1] * a.grid[2]), (q / a.grid[2]) % a.grid[1], q % a.grid[2]};
@@ -568,6 +568,7 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
       int g2[3] = {0, 0, 0};
       const int gs[3] = {(g[0] + g1[0]) % a.grid[0], (g[1] + g1[1]) % a.grid[1], (g[2] + g1[2]) % a.grid[2]};
       unsigned it = 0;
+      int turn = seg;  // visits until the segment's next one
       for (int k2 = 0; any && k2 < N; ++k2) {
         if (k2 != 0 && ++g2[2] == a.grid[2]) {
           g2[2] = 0;
@@ -586,6 +587,8 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
         const int k3 = (g3[0] * a.grid[1] + g3[1]) * a.grid[2] + g3[2];
         const int kd = (gd[0] * a.grid[1] + gd[1]) * a.grid[2] + gd[2];
         if (kd < k2) continue;  // {c, d} is visited at its smaller index
+        if (turn-- != 0) continue;
+        turn = a.nseg - 1;
         const bool twice = kd != k2;  // both orders of {c, d} come from this visit
         // ---- tables of k2 and k3
         if ((a.nu_select != 0 || a.split == 1) && tid == 0) s_umask = pair_umklapp_bits(a, g, g1, g2, g3);
@@ -1057,8 +1060,9 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
       niter += it;
       npair += any ? 1 : 0;
       // ---- R(a; b) of the chunk's j0 and R(b; a) of every x, rows summed in a fixed order
-      const size_t slot = a.mirror ? ((size_t)qi * N + k1) * a.nchunk + chunk : 0;
-      const size_t mslot = mir ? ((size_t)role.mirror * N + role.mirror_b) * a.nchunk + chunk : 0;
+      const size_t first = (size_t)seg * a.nq_sel * N * a.nchunk;  // slots of the segment
+      const size_t slot = a.mirror ? first + ((size_t)qi * N + k1) * a.nchunk + chunk : 0;
+      const size_t mslot = mir ? first + ((size_t)role.mirror * N + role.mirror_b) * a.nchunk + chunk : 0;
       const int nout = J + (mir ? NB : 0);
       for (int t = 0; t < nS; ++t) {
         if (has_row) {

@@ -106,8 +106,9 @@ __global__ void pair_reduce_kernel(RatesArgs a, double pref, double* rates) {
   const int chunk = j / a.J, jj = j % a.J;
   double s = 0.0;
   unsigned long long cnt = 0;
-  for (int b = lane; b < a.N; b += 32) {
-    const size_t base = ((size_t)qi * a.N + b) * a.nchunk;
+  for (int i = lane; i < a.N * a.nseg; i += 32) {
+    const int b = i % a.N;
+    const size_t base = ((size_t)(i / a.N) * a.nq_sel * a.N + (size_t)qi * a.N + b) * a.nchunk;
     if (a.nchunk == 1 || pair_role(a, qi, qe, b).run) {
       const size_t v = (base + chunk) * a.nb + jj;
       s += a.partial[v * a.nS + t];
@@ -420,13 +421,31 @@ static int plan_form(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, 
     *err = "cudaDeviceGetAttribute failed";
     return FP_ECUDA;
   }
+  // Small grids do not fill the chip with one item per pair (about half of the (evaluated point, q') run; a block lives
+  // for a prologue of some three to nine q'' and N / 2 q''), so a pair's q'' are dealt to nseg items in turn: up to 1.5
+  // items per resident block while an item keeps eight q'', or any number that leaves one item per SM.  Measured, one
+  // item per pair against the rule: simple cubic 3x3x4 0.322 -> 0.273 ms, 4x4x4 0.974 -> 0.898 (three items 0.935, four
+  // 0.989), diamond 3x3x4 with three temperatures 1.44 -> 1.28, BAs 3x4x3 1.17 -> 1.07; below eight q'' the repeated
+  // prologues cost more (diamond 3x3x3 with three items 0.556 -> 0.626).
+  int nseg = 1;
+  if (mirror) {
+    const double items = 0.5 * ((N + t1 - 1) / t1) * nq_sel * nchunk;
+    auto fits = [&](int n) {
+      const size_t bytes = (size_t)n * mirror_bytes;
+      return n <= N / 2 && bytes <= (size_t(64) << 20) && !(partial_budget && bytes > partial_budget);
+    };
+    while (items > 0.0 && fits(nseg + 1) &&
+           ((nseg * items < 1.5 * nsm * per_sm && N / (2 * (nseg + 1)) >= 8) || (nseg + 1) * items <= nsm))
+      ++nseg;
+  }
   p->J = J;
   p->threads = threads;
   p->t1 = t1;
   p->nchunk = nchunk;
   p->ntile = (N + t1 - 1) / t1;
   p->nq_sel = nq_sel;
-  p->n_items = (long long)p->ntile * nq_sel * nchunk;
+  p->n_items = (long long)p->ntile * nq_sel * nchunk * nseg;
+  p->nseg = nseg;
   p->smem = smem;
   p->pair = pair;
   p->sliced = sliced;
@@ -435,7 +454,7 @@ static int plan_form(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, 
   p->split = split;
   p->operands = sliced;
   p->mirror = mirror;
-  p->values = mirror ? mirror_values : p->n_items * J;
+  p->values = mirror ? mirror_values * nseg : p->n_items * J;
   long long ctas = (long long)nsm * per_sm;
   if (ctas > p->n_items) ctas = p->n_items > 0 ? p->n_items : 1;
   p->ctas = (int)ctas;
@@ -571,6 +590,7 @@ int run_rates(fp_ctx* c, const fp_rates_opts& o, const Selection& sel, const Pla
   a.t1 = p.t1;
   a.nchunk = p.nchunk;
   a.ntile = p.ntile;
+  a.nseg = p.nseg;
   a.nq_sel = p.nq_sel;
   a.n_items = p.n_items;
   a.qlist = sc.qlist;

@@ -176,3 +176,26 @@ def test_parts_in_one_pass(precision, maker, nT):
         assert st_c["accepted"][p] == acc[p]
     assert st["accepted"] == list(total) == st_f["accepted"]
     assert st["candidates"] == 2 * st_f["candidates"] and st_c["candidates"] == st_f["candidates"]
+
+
+@pytest.mark.parametrize("precision", [FP_PREC_FP64, FP_PREC_DOUBLE_FLOAT])
+@pytest.mark.parametrize("maker,nT", [(lambda: synth.simple_cubic((2, 1, 2)), 1), (lambda: synth.simple_cubic((4, 3, 3)), 1),
+                                      (lambda: synth.diamond_si((2, 2, 1)), 3), (lambda: synth.diamond_si((4, 3, 3)), 1)])
+def test_several_items_per_pair(precision, maker, nT):
+    """Grids whose pairs are dealt to several items (up to one per q'', and two of nine q'' each): rates, accepted counts and
+    the per-mode counts of the phase space, which share the items' slots; block_j0 = 1 adds chunks to the slots."""
+    cr = maker()
+    w, e, v = oracle_modes(cr)
+    temps = list(np.linspace(300.0, 900.0, nT))
+    N, nb = cr.nq, cr.nb
+    ref, acc = oracle.rates4(cr, w, e, v, temps=temps)
+    ps, pacc = oracle.rates4(cr, w, e, v, temps=temps, unit_vertex=True)
+    with Context.from_crystal(cr) as ctx:
+        ctx.set_modes(w, e, v)
+        for opts in ({}, dict(block_j0=1), dict(no_time_reversal=1)):
+            out, st = ctx.rates4(temps, cr.scalebroad, precision=precision, **opts)
+            _close_parts(out.reshape(nT, -1), ref)
+            assert st["accepted"] == list(acc)
+            npr, _, wp4 = ctx.phase_space4(temps, cr.scalebroad, precision=precision, **opts)
+            _close(wp4.reshape(nT, -1) * N ** 2, ps)
+            assert npr.sum() == pacc.sum()

@@ -465,11 +465,15 @@ extern "C" int fp_rates3(fp_ctx* c, int nT, const double* T, double scalebroad, 
   int rc = make_selection(c, so, true, &sel, &err);
   if (rc) return fail3(c, rc, "fp_rates3: " + err);
   const int nq = (int)sel.qlist.size();
-  // k1 ranges: enough blocks to fill the SMs about eight times over, so that the last wave costs little
+  // k1 ranges: enough blocks to fill the SMs about eight times over, so that the last wave costs little, of 16 points or
+  // more, and of 4 where those would leave half of the resident blocks empty (measured, 16 against 4: diamond 2x2x2 67 ->
+  // 49 us, 3x3x3 142 -> 64, 4x4x4 157 -> 137, LiCoO2 3x3x3 927 -> 300; but simple cubic 6x6x6 216 -> 277, LiCoO2 5x4x3
+  // 1053 -> 1085)
   int nsm = 0;
   R3_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device));
   int nch = nq > 0 ? (nsm * 16 + nq - 1) / nq : 1;
-  nch = std::max(1, std::min(nch, (N + 15) / 16));
+  const int least = 2LL * nq * ((N + 15) / 16) < (long long)nsm * (nb == 12 ? 1 : 2) ? 4 : 16;
+  nch = std::max(1, std::min(nch, (N + least - 1) / least));
   const int kchunk = (N + nch - 1) / nch;
   nch = (N + kchunk - 1) / kchunk;
   // working memory, kept in the context: T, occupation table, counts, partial sums, rates, selection, Psi

@@ -439,7 +439,10 @@ def main():
                          "frac": achieved_tflops / peak, "traffic": None, "peak_basis": peak_basis,
                          "pipe": "fp32" if main_prec == binding.FP_PREC_MIXED else "fp64",
                          "kernel_ms": kms, "flops_per_launch": st["flops"] + acc_flops,
-                         "flops_vertex": st["flops"], "flops_accumulate": acc_flops},
+                         "flops_vertex": st["flops"], "flops_accumulate": acc_flops,
+                         "note": None if main_prec != binding.FP_PREC_FP64 else
+                         "executed flops of the algorithm over the FP64 pipe's peak; with 6 or 12 branches the two "
+                         "vertex contractions run off that pipe, as exact integer slices on the tensor cores"},
             "other_precision": other,
             "mixed_tensor_cores": tensor,
             "double_float": dfl,

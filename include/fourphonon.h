@@ -38,7 +38,8 @@ extern "C" {
 #define FP_EUNSTABLE (-4)  /* omega^2 < -1e-8 max(omega^2) away from the three Gamma acoustic modes */
 #define FP_ESTATE (-6)     /* call out of order (e.g. rates before modes) */
 
-#define FP_PREC_FP64 0  /* vertex, Gaussian and sums in FP64 (parity path, 1e-10 vs the FP64 definition) */
+#define FP_PREC_FP64 0  /* vertex, Gaussian and sums in FP64, the contractions of six and twelve branches in exact integer
+                           slices of the same accuracy (parity path, 1e-10 vs the FP64 definition) */
 #define FP_PREC_MIXED 1 /* vertex and Gaussian in FP32, window decisions exact, sums in FP64 */
 #define FP_PREC_DOUBLE_FLOAT 2 /* FP64 path whose vertex contraction (Eq. V4 assembly and the two contractions)
                                   runs on the FP32 pipes in double-float: pairs of floats with exact high products
@@ -98,16 +99,20 @@ typedef struct {
 typedef struct {
   double candidates;   /* process terms of the selected modes: (processes) * (selected modes) * N^2 * nb^3 */
   double accepted[3];  /* terms of the selected modes inside the energy window for ++, +-, -- */
-  double flops;        /* vertex assembly + contraction flops executed (8 per complex multiply-add): the
-                          hoisted prologue and assembly per evaluated item and q'-pair, and one nb-term
-                          contraction per vertex entry formed (vertex_entries) */
+  double flops;        /* vertex assembly + contraction flops executed (8 per complex multiply-add, also where
+                          they run as integer slices on the tensor cores): the hoisted prologue and assembly per
+                          evaluated item and q'-pair, and one nb-term contraction per vertex entry formed
+                          (vertex_entries) */
   double ms;           /* device time of the rate kernels (CUDA events on the context stream) */
   int tile[4];         /* block_j0, k1_tile, threads, CTAs launched */
   double candidates_executed;  /* candidates the kernel screened: those of the evaluated rows (time reversal
                                   evaluates one point of each pair {q, -q}) */
-  double vertex_entries;       /* vertex entries W(j0, j1, j2, j3) formed: those with an accepted candidate */
+  double vertex_entries;       /* vertex entries W(j0, j1, j2, j3) formed: every entry of an evaluated row in the
+                                  sliced FP64 and the mixed kernels, one per accepted term in the other kernels
+                                  over pairs, those with an accepted candidate in the kernel over ordered sums */
   double terms_executed;       /* accepted terms the kernel evaluated (Gaussian, Bose factors, |W|^2), all
-                                  processes; accepted[] counts each once per selected mode it stands for */
+                                  processes; accepted[] counts each once per selected mode and order of its
+                                  partners that it stands for */
 } fp_stats;
 
 /* Library version (major * 10000 + minor * 100 + patch). */
@@ -228,8 +233,8 @@ int fp_phase4(fp_ctx* ctx, int nT, const double* T, double scalebroad, int strid
  * The paper prints no formula for P4 and WP4 (it cites them); these are the rate's sum with the vertex, and for
  * P4 also the Bose and frequency factors, set to 1.  Window, Gaussian, small-sigma rule, multiplicities c_p and
  * time reversal (stride 1) as in fp_rates4; opts: precision (FP64 default), window, sigma_min, dq_mode,
- * mode_mask, q range, process_mask and nu_select apply.  Any output may be NULL.  Two kernel passes (unit weights,
- * then Bose weights).  Requires modes (FP_ESTATE otherwise); FP_EINVAL for stride outside [1, N].
+ * mode_mask, q range, process_mask and nu_select apply.  Any output may be NULL.  One kernel pass (unit weights and
+ * the Bose weights of up to seven temperatures share it; mixed precision and eight temperatures take two).  Requires modes (FP_ESTATE otherwise); FP_EINVAL for stride outside [1, N].
  */
 int fp_phase_space4(fp_ctx* ctx, int nT, const double* T, double scalebroad, const fp_rates_opts* opts, int stride,
                     double* numprocess, double* p4, double* wp4);
@@ -237,9 +242,10 @@ int fp_phase_space4(fp_ctx* ctx, int nT, const double* T, double scalebroad, con
 /*
  * Channel-resolved rates: the ++ (recombination), +- (redistribution) and -- (splitting) parts of Eq.
  * 4phgamma, whose sum is fp_rates4's rate.  rates: host, nT x 3 x N x nb, channel index in the order ++, +-,
- * --.  opts->process_mask must be 0.  Each channel is one rate-kernel pass (the vertex is recomputed), so
- * the call costs about three fp_rates4 calls.  stats (nullable) sums the candidates, flops and time of the
- * three passes; accepted[p] is channel p's count.  Errors as fp_rates4.
+ * --.  opts->process_mask must be 0.  With up to two temperatures the three sums share one rate-kernel pass;
+ * with more, in mixed precision and for quartet lists without the transposition symmetry of Eq. TS each channel
+ * is a pass of its own.  stats (nullable) sums the candidates, flops and time of the passes; accepted[p] is
+ * channel p's count.  Errors as fp_rates4.
  */
 int fp_rates4_channels(fp_ctx* ctx, int nT, const double* T, double scalebroad, const fp_rates_opts* opts,
                        double* rates, fp_stats* stats);
@@ -307,7 +313,8 @@ int fp_kappa_rta(fp_ctx* ctx, int nT, const double* T, const double* rates, doub
  * over integers m_a in [-2, 2], with squared lengths within 1e-9 relative counted as equal and such ties won by
  * the lexicographically smallest (m_0, m_1, m_2).  rates: host, nT x 2 x N x nb (normal, then Umklapp); their
  * sum is fp_rates4's rate.  opts->nu_select must be 0; process_mask and the other options apply to both parts.
- * Two rate-kernel passes.  stats (nullable) sums the passes.  Errors as fp_rates4.
+ * One rate-kernel pass up to four temperatures (two beyond, in mixed precision and for quartet lists without the
+ * transposition symmetry of Eq. TS).  stats (nullable) sums the passes.  Errors as fp_rates4.
  */
 int fp_rates4_nu(fp_ctx* ctx, int nT, const double* T, double scalebroad, const fp_rates_opts* opts, double* rates,
                  fp_stats* stats);

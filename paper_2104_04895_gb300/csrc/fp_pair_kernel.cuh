@@ -28,18 +28,20 @@
 // compacted into a list that the warp evaluates 32 at a time (W, Gaussian), and each value returns to the row that
 // owns it: the FP64 pipe, the bound of the FP64 path, runs on full warps however unevenly the terms fall on rows.
 //
-// On the FP64 path with 6 or 12 branches and unit eigenvectors both vertex contractions run on the tensor cores in exact integer slices
-// (SL, fp_slices.cuh): A is built in FP64, its digits contract with those of e3 to T, T's digits with those of e2 to
+// On the FP64 path with 6 or 12 branches and unit eigenvectors both vertex contractions run on the tensor cores in exact
+// integer slices (SL, fp_slices.cuh): A is built in FP64, its digits contract with those of e3 to T, T's digits with those of e2 to
 // every W of the block, which costs the FP64 pipe only the A sums and |W|^2.  A scale per (j0, x), the power of two
 // above the Frobenius norm of its A block, keeps all three in range.
 //
-// Measured (GB300): ordered kernel -> pair kernel -> with slices and the U table of the prologue:
-//   diamond 6^3 FP64            578 -> 223 -> 125 ms      LiCoO2 5x4x3 FP64, 3 T   386 -> 154 -> 82 ms
-//   diamond 7x6x5 double-float  262 -> 88 ms (no slices: 107 ms with them, the FP64 A sums and conversions cost more
-//                               than the FP32 contraction; LiCoO2 4x3x3 24.3 ms either way)
-//   simple cubic 4^3 FP64       2.15 -> 1.49 -> 1.13 ms (nb = 3: no slices)
+// Measured (GB300): ordered kernel -> pair kernel -> with slices and the U table of the prologue -> with U over terms and
+// several items per pair on small grids:
+//   diamond 6^3 FP64            578 -> 223 -> 125 -> 119 ms      LiCoO2 5x4x3 FP64, 3 T   386 -> 154 -> 82 -> 76 ms
+//   diamond 7x6x5 double-float  262 -> 88 -> 87 ms (no slices: 107 ms with them, the FP64 A sums and conversions cost
+//                               more than the FP32 contraction; LiCoO2 4x3x3 24.3 ms either way)
+//   simple cubic 4^3 FP64       2.15 -> 1.49 -> 1.13 -> 0.90 ms (nb = 3: no slices)
 // Without slices the FP64 pipe (about 1.7 lane FMAs per clock and SM) is 91 % busy: per k2 of six branches 31k lane
-// FMAs for T, 20k for W, 8k for A, 12k for the terms.  With them it is the terms, A and the barriers between phases.
+// FMAs for T, 20k for W, 8k for A, 12k for the terms.  With them it is 68 % busy (diamond 4^3), three quarters of that
+// with the terms (20 instructions each), the rest with A; the barriers between the phases cost most of the other 32 %.
 #pragma once
 #include "fp_rates_kernel.cuh"
 #include "fp_slices.cuh"

@@ -1,6 +1,6 @@
 // Host side of the rate path: FP32 prep kernel, fixed-order reduction, tile plan and the launch routine
-// shared by fp_rates4, fp_rates4_device and fp_rates4_noalloc.  The rate kernel itself is in
-// fp_rates_kernel.cuh.
+// shared by fp_rates4, fp_rates4_device and fp_rates4_noalloc.  The rate kernels are in fp_pair_kernel.cuh
+// (FP64 and double-float), fp_dense_kernel.cuh (mixed) and fp_rates_kernel.cuh (the others' fallback).
 #include "fp_dense_kernel.cuh"
 #include "fp_pair_kernel.cuh"
 

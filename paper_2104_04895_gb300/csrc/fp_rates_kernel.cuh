@@ -1,5 +1,8 @@
 // Four-phonon RTA rate kernel template (paper Sec. 2.2 Eqs. tao0, 4phgamma, V4; Sec. 2.4).
 // Instantiated per precision in fp_rates_f64.cu, fp_rates_df.cu and fp_rates_f32.cu; host logic is in fp_rates.cu.
+// It evaluates the ordered sums over (q', q'') as they stand and needs only the symmetry of Phi4 in its legs j and k.  FP64
+// and double-float calls run it where Phi4 lacks the other exchanges (else fp_pair_kernel.cuh), mixed ones with twelve
+// branches, on the tcgen05 option and where fp_dense_kernel.cuh finds no room.
 //
 // One function W serves all three processes.  With k3 = q + k1 + k2 (mod G) and e(-k) = conj e(k),
 //   W(q,j0; k1,j1; k2,j2; k3,j3) = sum_quartets sum_{abgt} Phi4/sqrt(M^4) e_a(q,j0) e_b(k1,j1) e_g(k2,j2)

@@ -36,9 +36,12 @@
 // Measured (GB300): ordered kernel -> pair kernel -> with slices and the U table of the prologue -> with U over terms and
 // several items per pair on small grids:
 //   diamond 6^3 FP64            578 -> 223 -> 125 -> 119 ms      LiCoO2 5x4x3 FP64, 3 T   386 -> 154 -> 82 -> 76 ms
-//   diamond 7x6x5 double-float  262 -> 88 -> 87 ms (no slices: 107 ms with them, the FP64 A sums and conversions cost
-//                               more than the FP32 contraction; LiCoO2 4x3x3 24.3 ms either way)
+//   diamond 7x6x5 double-float  262 -> 88 -> 87 -> 91 ms (no slices: 107 ms with them, the FP64 A sums and conversions
+//                               cost more than the FP32 contraction; LiCoO2 4x3x3 24.3 ms either way)
 //   simple cubic 4^3 FP64       2.15 -> 1.49 -> 1.13 -> 0.90 ms (nb = 3: no slices)
+// The last double-float step evaluates the accepted terms in FP64 (before, in pairs of floats, whose weights underflowed
+// below about 20 K): 87 -> 91 ms with one temperature, 106 -> 103 with three, 126 -> 119 with eight, LiCoO2 4x3x3 17.2 ->
+// 16.8 and 22.3 -> 20.0 with three.
 // Without slices the FP64 pipe (about 1.7 lane FMAs per clock and SM) is 91 % busy: per k2 of six branches 31k lane
 // FMAs for T, 20k for W, 8k for A, 12k for the terms.  With them it is 68 % busy (diamond 4^3), three quarters of that
 // with the terms (20 instructions each), the rest with A; the barriers between the phases cost most of the other 32 %.
@@ -185,13 +188,6 @@ __host__ __device__ inline PairCarve make_pair_carve(int nb, int J, int G, int n
   return c;
 }
 
-template <typename VT>
-__device__ __forceinline__ VT pair_val(double v);
-template <>
-__device__ __forceinline__ double pair_val<double>(double v) { return v; }
-template <>
-__device__ __forceinline__ float2 pair_val<float2>(double v) { return df_make(v); }
-
 // x + y or x - y (the sign flipped in the integer pipe)
 __device__ __forceinline__ double add_signed(double x, double y, bool plus) {
   return __dadd_rn(x, __hiloint2double(__double2hiint(y) ^ (plus ? 0 : 0x80000000), __double2loint(y)));
@@ -217,20 +213,15 @@ __device__ __forceinline__ double pair_exp_neg64(double x, const double* tab) {
 __device__ __noinline__ double pair_two_orders(double ex, double z8, const double* tab) {
   return 0.5 * (ex + pair_exp_neg64(z8, tab));
 }
-__device__ __noinline__ float2 pair_two_orders(float2 ex, float2 z8, const float2* tab) {
-  const float2 m = df_add(ex, df_exp_neg64(df_mul(z8, z8), tab));
-  return make_float2(0.5f * m.x, 0.5f * m.y);
-}
 
-// NB branches, up to MAXT sums per row.  DF: vertex contraction and terms in double-float on the FP32 pipes.  SL: both
-// vertex contractions on the tensor cores in exact slices (fp_slices.cuh; unit eigenvectors, nb = 6 or 12): A in FP64,
+// NB branches, up to MAXT sums per row.  DF: vertex contraction in double-float on the FP32 pipes (the terms in FP64: the
+// weights of c and d fall as exp(-hbar (wc + wd) / k_B T), out of FP32's range at 10 to 20 K).  SL: both vertex contractions on the tensor cores in exact slices (fp_slices.cuh; unit eigenvectors, nb = 6 or 12): A in FP64,
 // T as digits, |W|^2 of every entry in FP64.
 template <int NB, int MAXT, bool DF, bool SL>
 __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pair_kernel(RatesArgs a) {
   static_assert(!(DF && SL), "the double-float contraction has no sliced form");
   constexpr int NB2 = NB * NB, NA = NB / 3;
   using C = Cx<double>;
-  using VT = typename std::conditional<DF, float2, double>::type;  // value of an evaluated entry
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ long long s_item;
   __shared__ unsigned s_umask;
@@ -244,15 +235,12 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
   double* db = reinterpret_cast<double*>(cx + cv.ncx);
   double *sOm0 = db + cv.Om0, *sOm1 = db + cv.Om1, *sOm2 = db + cv.Om2, *sOm3 = db + cv.Om3;
   double *sV2 = db + cv.V2, *sV3 = db + cv.V3, *sWc = db + cv.Wc, *sWd = db + cv.Wd;
-  // values of the path's type: doubles, or double-floats in the same slots
-  double* sX = db + cv.X;
-  VT *sIv8 = reinterpret_cast<VT*>(db + cv.Iv8), *sF = reinterpret_cast<VT*>(db + cv.F);
-  VT *sWB = reinterpret_cast<VT*>(db + cv.WB), *sExpT = reinterpret_cast<VT*>(db + cv.ExpT);
+  double *sX = db + cv.X, *sIv8 = db + cv.Iv8, *sF = db + cv.F, *sWB = db + cv.WB, *sExpT = db + cv.ExpT;
   // sliced: W [j0 x][y][j3] (combine_magic) and the lists take the place of the digits once these are in registers
   double2* sW = reinterpret_cast<double2*>(sT);
   unsigned* sDig = reinterpret_cast<unsigned*>(sT);
   const unsigned* sOp = reinterpret_cast<const unsigned*>(cx + cv.Op);
-  VT* sVal = reinterpret_cast<VT*>(SL ? reinterpret_cast<double*>(sW + (size_t)J * NB * NB2) : db + cv.Val) + (size_t)warp * kPairCap;
+  double* sVal = (SL ? reinterpret_cast<double*>(sW + (size_t)J * NB * NB2) : db + cv.Val) + (size_t)warp * kPairCap;
   double* sRed = reinterpret_cast<double*>(sT);  // the T block, free outside the k2 loop
   float* fb = reinterpret_cast<float*>(db + cv.ndbl);
   float *sH0 = fb + cv.H0, *sH1 = fb + cv.H1, *sH2 = fb + cv.H2, *sH3 = fb + cv.H3;
@@ -280,7 +268,7 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
     return a.split == 0 ? 0 : a.split == 1 ? (int)((um >> kind) & 1u) : kind == 0 ? 1 : kind < 3 ? 0 : 2;
   };
 
-  for (int o = tid; o < kExpTab; o += nthr) sExpT[o] = pair_val<VT>(exp(-(double)o * kExpH));
+  for (int o = tid; o < kExpTab; o += nthr) sExpT[o] = exp(-(double)o * kExpH);
   for (int o = tid; o < NA + 1; o += nthr) sKLs[o] = a.pk_start[o];
   for (int o = tid; o < G; o += nthr) sKLg[o] = a.pk_grp[o];
   for (int o = tid; o < NA * NA; o += nthr) sKLz[o] = a.pk_zero[o];
@@ -478,11 +466,8 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
       const unsigned proc_cand = ((a.cand_mask & 2u) ? 1u : 0u) | ((a.cand_mask & 1u) ? 6u : 0u) |
                                  ((a.cand_mask & 4u) ? 24u : 0u);
       // S1, S4 and S5 of the row; S1 in registers, the others (rarer) in local memory when there are several
-      // temperatures.  Double-float: two-float running sums of S1 (and S4, S5 for one temperature), moved into the
-      // FP64 sums every 64 q'' so that each holds a bounded number of terms.
+      // temperatures
       double S1[MAXT], R45[2 * MAXT];
-      constexpr int kRun = DF ? (MAXT == 1 ? 3 : MAXT) : 1;
-      float sh[kRun], sl[kRun];
       unsigned n1 = 0, n4 = 0, n5 = 0;  // accepted terms of this pair: of both modes, of a only, of b only
 #pragma unroll
       for (int t = 0; t < MAXT; ++t) S1[t] = 0.0;
@@ -491,56 +476,10 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
       } else {
         for (int t = 0; t < 2 * nS; ++t) R45[t] = 0.0;
       }
-#pragma unroll
-      for (int k = 0; k < kRun; ++k) sh[k] = sl[k] = 0.f;
-      auto flush_df = [&]() {
-        if constexpr (DF) {
-#pragma unroll
-          for (int t = 0; t < MAXT; ++t) S1[t] += (double)sh[t] + (double)sl[t];
-          if constexpr (MAXT == 1) {
-            R45[0] += (double)sh[1] + (double)sl[1];
-            R45[1] += (double)sh[2] + (double)sl[2];
-          }
-#pragma unroll
-          for (int k = 0; k < kRun; ++k) sh[k] = sl[k] = 0.f;
-        }
-      };
       // value v of test `kind` at the entry e = (y, j3) into the row's sums, those of its part from slot lo
       unsigned umask = 0;  // Umklapp tests of the current k2
-      auto add = [&](const VT v, const int kind, const int e) {
-        if constexpr (DF) {
-          auto run = [&](int k, float2 term) {
-            float s, er;
-            two_sum(sh[k], term.x, s, er);
-            const float2 nrm = df_fast(s, __fadd_rn(er, __fadd_rn(sl[k], term.y)));
-            sh[k] = nrm.x;
-            sl[k] = nrm.y;
-          };
-          if constexpr (MAXT == 1) {
-            if (kind < 3)
-              run(0, v);
-            else if (kind == 3)
-              run(1, v);
-            else
-              run(2, v);
-          } else {
-            const float2* wb = sWB + (kind < 3 ? kind : 0) * NB2 + e;
-            const int lo = part_of(kind, umask) * nT;
-            if (kind < 3) {
-#pragma unroll
-              for (int t = 0; t < MAXT; ++t) {
-                if (t >= nS) break;
-                if (t >= lo && t < lo + nT) run(t, df_mul(v, wb[3 * (t - lo) * NB2]));
-              }
-            } else {
-#pragma unroll 1
-              for (int t = 0; t < nT; ++t) {
-                const float2 term = df_mul(v, wb[3 * t * NB2]);
-                R45[(kind - 3) * nS + lo + t] += (double)term.x + (double)term.y;
-              }
-            }
-          }
-        } else if constexpr (MAXT == 1) {
+      auto add = [&](const double v, const int kind, const int e) {
+        if constexpr (MAXT == 1) {
           if (kind < 3)
             S1[0] += v;
           else if (kind == 3)
@@ -669,20 +608,20 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
             sigma_f_from_exact(ex, sPM + o, &inv);
             iv = ex[1];
           }
-          sIv8[o] = pair_val<VT>(iv >= 0.0 ? 8.0 * iv : -1.0);
+          sIv8[o] = iv >= 0.0 ? 8.0 * iv : -1.0;
           // 1/2 per order of {c, d} (Eq. tao0; the 1/6 of -- is completed in the epilogue) and the Gaussian's 1/sqrt(pi)
           const double f = iv >= 0.0 ? iv * kInvSqrtPi : 1.0;
           if (tab) {
-            sF[e] = pair_val<VT>((twice ? 1.0 : 0.5) * f * (MAXT == 1 ? sWc[2 * y + 1] * sWd[2 * j3 + 1] : 1.0));
+            sF[e] = (twice ? 1.0 : 0.5) * f * (MAXT == 1 ? sWc[2 * y + 1] * sWd[2 * j3 + 1] : 1.0);
           } else {
-            sF[NB2 + e] = pair_val<VT>(0.5 * f * (MAXT == 1 ? sWc[2 * y] * sWd[2 * j3 + 1] : 1.0));
-            sF[2 * NB2 + e] = pair_val<VT>(0.5 * f * (MAXT == 1 ? sWc[2 * y + 1] * sWd[2 * j3] : 1.0));
+            sF[NB2 + e] = 0.5 * f * (MAXT == 1 ? sWc[2 * y] * sWd[2 * j3 + 1] : 1.0);
+            sF[2 * NB2 + e] = 0.5 * f * (MAXT == 1 ? sWc[2 * y + 1] * sWd[2 * j3] : 1.0);
           }
         }
         if constexpr (MAXT > 1)
           for (int o = tid; o < 3 * nT * NB2; o += nthr) {
             const int t = o / (3 * NB2), k = (o / NB2) % 3, y = (o / NB) % NB, j3 = o % NB;
-            sWB[o] = pair_val<VT>(sWc[2 * (t * NB + y) + (k == 1 ? 0 : 1)] * sWd[2 * (t * NB + j3) + (k == 2 ? 0 : 1)]);
+            sWB[o] = sWc[2 * (t * NB + y) + (k == 1 ? 0 : 1)] * sWd[2 * (t * NB + j3) + (k == 2 ? 0 : 1)];
           }
         if (has_row && !unit) {
           const int ka = rc / 3, ga = rc % 3;
@@ -981,8 +920,8 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
                 const int ejj = row / NB2, ex = (row / NB) % NB, ey = row % NB;
                 const int ab = ejj * NB + ex, e = ey * NB + j3;
                 const bool tab0 = kind == 1 || kind == 2;
-                const VT iv8 = sIv8[(tab0 ? 0 : NB2) + e];
-                VT gv = sF[(tab0 ? kind : 0) * NB2 + e];
+                const double iv8 = sIv8[(tab0 ? 0 : NB2) + e];
+                double gv = sF[(tab0 ? kind : 0) * NB2 + e];
                 // dw in the operation order of the definition (P5 negated): at a resonance of a mode with itself it is
                 // a rounding error, which a small sigma makes visible
                 const double wx = sX[(kind >= 3 ? J * NB : 0) + ab];
@@ -992,52 +931,39 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
                 const double dw = add_signed(add_signed(wx, y1, plus1), y2, plus2);
                 // the other order of {c, d} differs by its rounding, which only a sigma below 1e-3 rad/ps shows
                 const bool orders = twice && !tab0 && !(en & 1024u);
-                VT v;
+                double W2 = 1.0;
                 if constexpr (DF) {
-                  float2 W2 = make_float2(1.f, 0.f);
                   if (!unit) {
                     const float4* tb = reinterpret_cast<const float4*>(sT + (size_t)ab * (NB2 + 1) + j3);
                     const float4* e2 = reinterpret_cast<const float4*>(sE2 + ey * NB);
                     float4 Wd = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
                     for (int c = 0; c < NB; ++c) cdf_mac(Wd, e2[c], tb[c * NB]);
-                    W2 = cdf_abs2_df(cdf_norm(Wd));  // a vanishing W leaves its high parts cancelled
+                    W2 = cdf_abs2(cdf_norm(Wd));  // a vanishing W leaves its high parts cancelled
                   }
-                  if (iv8.x >= 0.f) {
-                    const float2 x8 = df_mul(df_make(dw), iv8);
-                    float2 ex = df_exp_neg64(df_mul(x8, x8), sExpT);
-                    if (iv8.x > 8000.f && orders)
-                      ex = pair_two_orders(ex, df_mul(df_make(add_signed(add_signed(wx, y2, plus1), y1, plus2)), iv8), sExpT);
-                    gv = df_mul(gv, ex);
+                } else if constexpr (SL) {
+                  if (!unit) {
+                    const double2 w = sW[ab * NB2 + e];
+                    const double wr = w.x - slices::kMagic, wi = w.y - slices::kMagic;
+                    W2 = fma(wr, wr, wi * wi);
                   }
-                  v = df_mul(W2, gv);
-                  if (en & 1024u) v = make_float2(0.5f * v.x, 0.5f * v.y);
-                } else {
-                  double W2 = 1.0;
-                  if constexpr (SL) {
-                    if (!unit) {
-                      const double2 w = sW[ab * NB2 + e];
-                      const double wr = w.x - slices::kMagic, wi = w.y - slices::kMagic;
-                      W2 = fma(wr, wr, wi * wi);
-                    }
-                  } else if (!unit) {
-                    const C* tb = sT + (size_t)ab * (NB2 + 1) + j3;
-                    const C* e2 = sE2 + ey * NB;
-                    C Wv = cmk<double>(0, 0);
+                } else if (!unit) {
+                  const C* tb = sT + (size_t)ab * (NB2 + 1) + j3;
+                  const C* e2 = sE2 + ey * NB;
+                  C Wv = cmk<double>(0, 0);
 #pragma unroll
-                    for (int c = 0; c < NB; ++c) cfma(Wv, e2[c], tb[c * NB]);
-                    W2 = Wv.re * Wv.re + Wv.im * Wv.im;
-                  }
-                  if (__double2hiint(iv8) >= 0) {  // not -1 (delta := 1)
-                    const double x8 = dw * iv8;
-                    double ex = pair_exp_neg64(x8, sExpT);
-                    if (__double2hiint(iv8) > 0x40bf4000 && orders)  // 8 / sigma > 8000
-                      ex = pair_two_orders(ex, add_signed(add_signed(wx, y2, plus1), y1, plus2) * iv8, sExpT);
-                    gv *= ex;
-                  }
-                  v = W2 * gv;
-                  if (en & 1024u) v *= 0.5;
+                  for (int c = 0; c < NB; ++c) cfma(Wv, e2[c], tb[c * NB]);
+                  W2 = Wv.re * Wv.re + Wv.im * Wv.im;
                 }
+                if (__double2hiint(iv8) >= 0) {  // not -1 (delta := 1)
+                  const double x8 = dw * iv8;
+                  double ex = pair_exp_neg64(x8, sExpT);
+                  if (__double2hiint(iv8) > 0x40bf4000 && orders)  // 8 / sigma > 8000
+                    ex = pair_two_orders(ex, add_signed(add_signed(wx, y2, plus1), y1, plus2) * iv8, sExpT);
+                  gv *= ex;
+                }
+                double v = W2 * gv;
+                if (en & 1024u) v *= 0.5;
                 sVal[i] = v;
               }
               __syncwarp();
@@ -1055,10 +981,9 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
             }
           }
         }
-        if ((++it & 63u) == 0) flush_df();
+        ++it;
         __syncthreads();
       }
-      flush_df();
       niter += it;
       npair += any ? 1 : 0;
       // ---- R(a; b) of the chunk's j0 and R(b; a) of every x, rows summed in a fixed order

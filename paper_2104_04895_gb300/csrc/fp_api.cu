@@ -193,6 +193,7 @@ void fp_free(fp_ctx* c) {
   dfree(c->d_omega);
   dfree(c->d_evec);
   dfree(c->d_vel);
+  dfree(c->d_wmax);
   dfree(c->d_flag);
   dfree(c->d_scratch);
   dfree(c->d_rates);
@@ -424,6 +425,7 @@ int fp_init(fp_ctx** out, const double lattice[9], int natoms, const double* fra
   INIT_CUDA(dalloc(&c->d_tw, (size_t)c->L));
   INIT_CUDA(fp::launch_twiddles(c, s));
   INIT_CUDA(dalloc(&c->d_flag, 1));
+  INIT_CUDA(dalloc(&c->d_wmax, 1));
   {
     std::vector<int> bzm(3 * (size_t)c->N);
     fp::bz_shifts(c->grid, c->rec, bzm.data());
@@ -450,6 +452,7 @@ int fp_modes(fp_ctx* c, double* omega, double* evec, double* vel) {
   if (rc) return rc;
   cudaStream_t s = c->stream;
   FP_CUDA(c, cudaMemsetAsync(c->d_flag, 0, sizeof(int), s));
+  FP_CUDA(c, cudaMemsetAsync(c->d_wmax, 0, sizeof(double), s));
   FP_CUDA(c, fp::launch_modes(c, s));
   int flag = 0;
   FP_CUDA(c, cudaMemcpyAsync(&flag, c->d_flag, sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -471,6 +474,7 @@ int fp_set_modes(fp_ctx* c, const double* omega, const double* evec, const doubl
   if (!c) return fail(nullptr, FP_EINVAL, "fp_set_modes: NULL context");
   if (!omega || !evec || !vel) return fail(c, FP_EINVAL, "fp_set_modes: NULL table");
   const int nb = c->nb;
+  double wmax = 0.0;
   bool unit = true;  // eigenvectors of norm 1 (a table may scale them; the sliced contraction is built for unit ones)
   for (int q = 0; q < c->N; ++q) {
     const int p = neg_index(c, q);
@@ -482,6 +486,7 @@ int fp_set_modes(fp_ctx* c, const double* omega, const double* evec, const doubl
       }
       unit = unit && std::fabs(norm2 - 1.0) <= 2e-5;
       double w = omega[q * nb + j];
+      wmax = std::max(wmax, w);
       if (!(w >= 0.0) || !std::isfinite(w)) return fail(c, FP_EINVAL, "fp_set_modes: omega must be finite and >= 0");
       if (omega[p * nb + j] != w) return fail(c, FP_EINVAL, "fp_set_modes: omega(-q) != omega(q)");
       for (int d = 0; d < 3; ++d)
@@ -502,6 +507,7 @@ int fp_set_modes(fp_ctx* c, const double* omega, const double* evec, const doubl
   FP_CUDA(c, cudaMemcpyAsync(c->d_omega, omega, nm * sizeof(double), cudaMemcpyHostToDevice, s));
   FP_CUDA(c, cudaMemcpyAsync(c->d_evec, evec, nm * nb * sizeof(double2), cudaMemcpyHostToDevice, s));
   FP_CUDA(c, cudaMemcpyAsync(c->d_vel, vel, nm * 3 * sizeof(double), cudaMemcpyHostToDevice, s));
+  FP_CUDA(c, cudaMemcpyAsync(c->d_wmax, &wmax, sizeof(double), cudaMemcpyHostToDevice, s));
   FP_CUDA(c, cudaStreamSynchronize(s));
   c->have_modes = true;
   c->unit_modes = unit;

@@ -44,6 +44,9 @@ struct RatesArgs {
   const double2* evec;       // [N][nb][nb]
   const double* vel;         // [N][nb][3]
   const double* wt;          // [nT][N*nb][3]: 1/(n w), (1+n)/w, n/w
+  const double* T;           // [nT] temperatures and [1] largest frequency (the pair kernel's scale of the weights)
+  const double* wmax;
+  int unit_weights;          // 1: the weights of the first temperature are 1
   const int* qmeta;          // [nquart][9]: i, j, group, Rj[3], Rl[3]
   const double* qfc;         // [nquart][81], divided by sqrt(Mi Mj Mk Ml)
   const int* gmeta;          // [G][5]: k, l, D = Rk - Rl
@@ -201,6 +204,7 @@ struct fp_ctx {
   double* d_omega = nullptr;
   double2* d_evec = nullptr;
   double* d_vel = nullptr;
+  double* d_wmax = nullptr;  // largest frequency
   int* d_flag = nullptr;
   // per-call working memory (grown on demand) and the output staging buffer of fp_rates4
   unsigned char* d_scratch = nullptr;

@@ -46,6 +46,7 @@ struct ModesArgs {
   double* omega;
   double2* evec;
   double* vel;
+  unsigned long long* wmax;  // bits of the largest frequency (non-negative doubles order like their bits)
   int* flag;
 };
 
@@ -249,6 +250,7 @@ __global__ void __launch_bounds__(32 * kModesWarps) modes_kernel(ModesArgs a) {
     }
     b = e;
   }
+  if (lane == 0) atomicMax(a.wmax, (unsigned long long)__double_as_longlong(wmax));
   for (int b = lane; b < nb; b += 32) {
     a.omega[q * nb + b] = w[b];
     a.omega[partner * nb + b] = w[b];
@@ -311,6 +313,7 @@ cudaError_t launch_modes(fp_ctx* c, cudaStream_t s) {
   a.omega = c->d_omega;
   a.evec = c->d_evec;
   a.vel = c->d_vel;
+  a.wmax = reinterpret_cast<unsigned long long*>(c->d_wmax);
   a.flag = c->d_flag;
   const size_t smem = (size_t)kModesWarps * 3 * c->nb * c->nb * sizeof(double2);  // 27 KB for twelve branches
   modes_kernel<<<(c->N + kModesWarps - 1) / kModesWarps, 32 * kModesWarps, smem, s>>>(a);

@@ -19,6 +19,10 @@
 // The leg weights of a and b leave the inner sum: with S1 = sum over P1, P2, P3 of |W|^2 delta x (c and d weights),
 // S4 and S5 likewise,
 //   R(a; b) = f0(a) [ (1 + nb)/wb S1 + nb/wb S4 ],   R(b; a) = f0(b) [ (1 + na)/wa S1 + na/wa S5 ],   f0 = 1/(n w).
+// With x = hbar w / k_B T the product nc nd inside goes as exp(-(xc + xd)), xc + xd about xa + xb, and f0 as exp(xa): at low
+// temperature the product underflows where the rate, about exp(-xb), does not.  So the c and d weights carry a power of
+// two each, near exp(x/2) of the largest frequency, and f0 carries its inverse square: the products then stay between
+// exp(-x) and exp(x), and every bit is as without it where the plain product is a normal number.
 //
 // Both values go to their own slot of `partial` ([evaluated point][partner b]); pair_reduce_kernel sums the slots of a
 // mode in a fixed order.  No atomics touch the rates.
@@ -225,6 +229,7 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ long long s_item;
   __shared__ unsigned s_umask;
+  __shared__ double s_up[kMaxT], s_down[kMaxT];  // scale of the c and d weights, and its inverse square
   const int J = a.J, G = a.G, nT = a.nT, nS = a.nS, N = a.N;  // nS sums per row: temperatures x parts
   const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, warp = tid >> 5;
   const int rows = J * NB2;
@@ -269,6 +274,13 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
   };
 
   for (int o = tid; o < kExpTab; o += nthr) sExpT[o] = exp(-(double)o * kExpH);
+  for (int t = tid; t < nT; t += nthr) {
+    // at most 2^430: the largest sums, 2^860 times |W|^2 in units of 2^-102, stay below 2^1024
+    const double half = 0.72134752044448170 * kHbar * a.wmax[0] / (kBoltzmann * a.T[t]);  // x / (2 ln 2)
+    const int k = a.unit_weights && t == 0 ? 0 : __double2int_rn(fmin(half, 430.0));
+    s_up[t] = scalbn(1.0, k);
+    s_down[t] = scalbn(1.0, -2 * k);
+  }
   for (int o = tid; o < NA + 1; o += nthr) sKLs[o] = a.pk_start[o];
   for (int o = tid; o < G; o += nthr) sKLg[o] = a.pk_grp[o];
   for (int o = tid; o < NA * NA; o += nthr) sKLz[o] = a.pk_zero[o];
@@ -568,8 +580,8 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
         for (int o = tid; o < 2 * nT * NB; o += nthr) {
           const int t = o / (2 * NB), r = o % (2 * NB);
           const size_t base = 3 * ((size_t)t * NM);
-          sWc[o] = a.wt[base + 3 * ((size_t)k2 * NB + r / 2) + 1 + r % 2];
-          sWd[o] = a.wt[base + 3 * ((size_t)k3 * NB + r / 2) + 1 + r % 2];
+          sWc[o] = a.wt[base + 3 * ((size_t)k2 * NB + r / 2) + 1 + r % 2] * s_up[t];
+          sWd[o] = a.wt[base + 3 * ((size_t)k3 * NB + r / 2) + 1 + r % 2] * s_up[t];
         }
         for (int gi = tid; gi < G; gi += nthr) {
           const int* gm = a.gmeta + 5 * gi;
@@ -1019,7 +1031,7 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
             const double* wo = W + 3 * (direct ? (size_t)k1 * NB + o : (size_t)q * NB + j0b + o);
             sum += wo[1] * s1 + wo[2] * ((1.0 / 3.0) * s2);
           }
-          sum *= W[3 * (direct ? (size_t)q * NB + j0b + m : (size_t)k1 * NB + m)];
+          sum *= W[3 * (direct ? (size_t)q * NB + j0b + m : (size_t)k1 * NB + m)] * s_down[t % nT];
           if (!a.mirror) {
             if (nS == 1) {
               dir += sum;

@@ -603,6 +603,9 @@ int run_rates(fp_ctx* c, const fp_rates_opts& o, const Selection& sel, const Pla
   a.evec = c->d_evec;
   a.vel = c->d_vel;
   a.wt = sc.wt;
+  a.T = sc.T;
+  a.wmax = c->d_wmax;
+  a.unit_weights = x.unit_weights ? 1 : 0;
   a.qmeta = c->d_qmeta;
   a.qfc = c->d_qfc;
   a.gmeta = c->d_gmeta;

@@ -109,6 +109,7 @@ extern "C" int fp_rates4_noalloc(fp_ctx* c, int nT, const double* T, double sb, 
   for (;;) {  // simpler forms of the rate kernel need less scratch
     rc = fp::plan_rates(c, o_probe, nT, sel, 0, &p0, &err, form == fp::kPairMirror ? fp::kPairSliced : form);
     if (rc) return nfail(c, rc, "fp_rates4_noalloc: " + err);
+    p0.psi_u = false;  // a plan with a budget, like the one below, has no table U
     fp::scratch_sizes(c, p0, nT, sz);
     fixed = 0;
     for (int i = 0; i < fp::kScratchParts; ++i)

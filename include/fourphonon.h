@@ -170,7 +170,8 @@ int fp_rates4_device(fp_ctx* ctx, int nT, const double* T, double scalebroad, co
  * Tile autotuner (the paper has no counterpart: it chooses launch tiles of this library's rate kernel).
  * Times every admissible (block_j0, k1_tile, threads) on a sample of q-points with opts->precision and
  * the given temperatures, writes the fastest into opts and remembers it in the context for calls whose
- * tile fields are 0 at that precision and temperature count.  best_ms (nullable) receives its time.
+ * tile fields are 0 at that precision and temperature count (where it fits them).  The untuned default is one of
+ * them and stays unless another is more than 3 % faster.  best_ms (nullable) receives its time.
  */
 int fp_autotune(fp_ctx* ctx, int nT, const double* T, double scalebroad, fp_rates_opts* opts, double* best_ms);
 

@@ -333,8 +333,10 @@ static int plan_form(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, 
   int J = o.block_j0;
   int t1_tuned = 0, th_tuned = 0;
   if (J <= 0 && o.k1_tile <= 0 && o.threads <= 0) {
+    // tuned for the same precision, but perhaps for another form or fewer sums: used where it fits
     const int* tt = c->tuned[o.precision][nT == 1 ? 0 : 1];
-    if (tt[0] > 0) {
+    if (tt[0] > 0 && tt[2] <= (pair ? pair_threads_for(nb) : max_threads_for(nb)) &&
+        smem_bytes(o.precision, nb, tt[0], c->G, c->nquart, nT, nS, tt[2], tc, pair, sliced, dense) <= 227 * 1024) {
       J = tt[0];
       t1_tuned = tt[1];
       th_tuned = tt[2];
@@ -360,9 +362,9 @@ static int plan_form(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, 
   const int rows = J * nb * nb;
   int threads = o.threads > 0 ? o.threads : th_tuned > 0 ? th_tuned : ((rows + 31) / 32) * 32;
   if (threads < 32) threads = 32;
-  const int max_threads = o.block_j0 > 0 || o.threads > 0 || !pair ? max_threads_for(nb) : pair_threads_for(nb);
+  const int max_threads = pair ? pair_threads_for(nb) : max_threads_for(nb);
   if (threads % 32 || threads < rows || threads > max_threads) {
-    *err = "threads must be a multiple of 32, >= block_j0*nb^2 and <= " + std::to_string(max_threads_for(nb));
+    *err = "threads must be a multiple of 32, >= block_j0*nb^2 and <= " + std::to_string(max_threads);
     return FP_EINVAL;
   }
   const int nq_sel = (int)sel.qlist.size();
@@ -468,13 +470,21 @@ static int plan_form(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, 
   return FP_OK;
 }
 
+// The pair kernel identifies vertices whose legs are permuted, so it needs Phi4 to have that symmetry.
+static bool over_pairs(const fp_ctx* c, const fp_rates_opts& o) { return c->leg_symmetric && o.precision != FP_PREC_MIXED; }
+
+int max_tile_threads(const fp_ctx* c, const fp_rates_opts& o) {
+  return over_pairs(c, o) ? pair_threads_for(c->nb) : max_threads_for(c->nb);
+}
+
 int plan_rates(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, size_t partial_budget, Plan* p,
                std::string* err, RateForm form, int split) {
   if (nT * (split == 1 ? 2 : 3) > kMaxT) split = 0;
-  // The pair kernel identifies vertices whose legs are permuted, so it needs Phi4 to have that symmetry; where its
-  // tables do not fit, the ordered kernel runs.  The mixed path keeps the ordered kernel: its FP32 vertex rounds
+  // Where the pair kernel's tables do not fit, the ordered kernel runs; if neither runs, the first one's reason stands, whose
+  // limits are the wider ones.  The mixed path keeps the ordered kernel: its FP32 vertex rounds
   // differently for each order of the legs, and exchanging them moved the rates by up to 2e-8 (its error is 5e-8).
-  if (form != kOrdered && c->leg_symmetric && o.precision != FP_PREC_MIXED) {
+  std::string why;
+  if (form != kOrdered && over_pairs(c, o)) {
     // the FP64 path's contraction in slices: 6 and 12 branches (with 3, K = 6 would leave most of a tile empty)
     if (form != kPair && o.precision == FP_PREC_FP64 && c->unit_modes && c->nb >= 6) {
       const int rc = plan_form(c, o, nT, sel, partial_budget, p, err, true, true, form == kPairMirror, split);
@@ -482,6 +492,7 @@ int plan_rates(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, size_t
     }
     const int rc = plan_form(c, o, nT, sel, partial_budget, p, err, true, false, form == kPairMirror, split);
     if (rc != FP_EINVAL) return rc;
+    why = *err;
   }
   // The mixed path's dense kernel evaluates the ordered sums for three and six branches.  With twelve, 144 rows are one
   // j0 per block and both the columns and the unrolled loop spill: LiCoO2 5x4x4 63.8 ms against 62.6 for the ordered
@@ -491,7 +502,9 @@ int plan_rates(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, size_t
     const int rc = plan_form(c, o, nT, sel, partial_budget, p, err, false, false, false, 0, true);
     if (rc != FP_EINVAL) return rc;
   }
-  return plan_form(c, o, nT, sel, partial_budget, p, err, false, false, false, 0);
+  const int rc = plan_form(c, o, nT, sel, partial_budget, p, err, false, false, false, 0);
+  if (rc == FP_EINVAL && !why.empty()) *err = why;
+  return rc;
 }
 
 void scratch_sizes(const fp_ctx* c, const Plan& p, int nT, size_t s[kScratchParts]) {

@@ -540,25 +540,50 @@ static int validate_opts(fp_ctx* c, int nT, const double* T, double sb, const fp
   return FP_OK;
 }
 
-// run a plan on the context's scratch (grown on demand)
-static int run_planned(fp_ctx* c, const fp_rates_opts& o, const fp::Selection& sel, const fp::Plan& p, int nT,
-                       const double* T, double sb, double* d_out, fp_stats* stats) {
-  size_t sz[fp::kScratchParts], total = 0;
-  fp::scratch_sizes(c, p, nT, sz);
-  for (size_t x : sz) total += x;
-  if (c->scratch_cap < total) {
-    dfree(c->d_scratch);
-    c->scratch_cap = 0;
-    FP_CUDA(c, dalloc(&c->d_scratch, total));
-    c->scratch_cap = total;
-  }
-  const fp::Scratch sc = fp::carve_scratch(c->d_scratch, sz);
-  unsigned long long counts[fp::kCounters] = {0};
+// The forms of a call in the order in which they are tried: one that finds no memory hands over to the next, which needs
+// less (no slot per pair; no table U, which a budget rules out; the ordered sums).
+struct FormTry {
+  fp::RateForm form;
+  size_t budget;
+};
+static const FormTry kFormTries[] = {
+    {fp::kPairMirror, 0}, {fp::kPairSliced, 0}, {fp::kPairSliced, ~size_t(0)}, {fp::kOrdered, 0}};
+
+// Plan a call and run it on the context's scratch (grown on demand).  split > 0 asks for the parts apart in one pass;
+// *did_split says whether the plan does that, and nothing has run where it does not.
+static int plan_and_run(fp_ctx* c, const fp_rates_opts& o, fp::Selection& sel, int nT, const double* T, double sb, double* d_out,
+                        fp_stats* stats, int split = 0, bool* did_split = nullptr) {
   std::string err;
-  const int rc = fp::run_rates(c, o, sel, p, sc, nT, T, sb, d_out, counts, o.no_graph == 0, &err);
-  if (rc) return fail(c, rc, "fp_rates4: " + err);
-  if (stats) fp::fill_stats(c, o, sel, p, counts, stats);
-  return FP_OK;
+  for (const FormTry& f : kFormTries) {
+    fp::Plan p;
+    int rc = fp::plan_rates(c, o, nT, sel, f.budget, &p, &err, f.form, split);
+    if (rc && &f != kFormTries) return fail(c, FP_ENOMEM, "fp_rates4: no memory for the form that takes these tiles");
+    if (rc) return fail(c, rc, "fp_rates4: " + err);
+    if (did_split) *did_split = p.split != 0;
+    if (split && !p.split) return FP_OK;
+    size_t sz[fp::kScratchParts], total = 0;
+    fp::scratch_sizes(c, p, nT, sz);
+    for (size_t x : sz) total += x;
+    if (c->scratch_cap < total) {
+      dfree(c->d_scratch);
+      c->scratch_cap = 0;
+      const cudaError_t e = dalloc(&c->d_scratch, total);
+      if (e == cudaErrorMemoryAllocation && f.form != fp::kOrdered) {
+        cudaGetLastError();  // not sticky: the next form is tried
+        continue;
+      }
+      FP_CUDA(c, e);
+      c->scratch_cap = total;
+    }
+    const fp::Scratch sc = fp::carve_scratch(c->d_scratch, sz);
+    unsigned long long counts[fp::kCounters] = {0};
+    rc = fp::run_rates(c, o, sel, p, sc, nT, T, sb, d_out, counts, o.no_graph == 0, &err);
+    fp::trim_scratch(c);
+    if (rc) return fail(c, rc, "fp_rates4: " + err);
+    if (stats) fp::fill_stats(c, o, sel, p, counts, stats);
+    return FP_OK;
+  }
+  return fail(c, FP_ENOMEM, "fp_rates4: no form fits");  // not reached: the last form returns
 }
 
 static int rates_impl(fp_ctx* c, int nT, const double* T, double sb, const fp_rates_opts* user, double* d_out,
@@ -571,10 +596,7 @@ static int rates_impl(fp_ctx* c, int nT, const double* T, double sb, const fp_ra
   fp::Selection sel;
   rc = fp::make_selection(c, o, true, &sel, &err);
   if (rc) return fail(c, rc, "fp_rates4: " + err);
-  fp::Plan p;
-  rc = fp::plan_rates(c, o, nT, sel, 0, &p, &err);
-  if (rc) return fail(c, rc, "fp_rates4: " + err);
-  return run_planned(c, o, sel, p, nT, T, sb, d_out, stats);
+  return plan_and_run(c, o, sel, nT, T, sb, d_out, stats);
 }
 
 int fp_rates4_device(fp_ctx* c, int nT, const double* T, double scalebroad, const fp_rates_opts* opts,
@@ -711,20 +733,19 @@ int rates_passes(fp_ctx* c, int nT, const double* T, double sb, const fp_rates_o
     so.no_graph = 1;
     std::string err;
     fp::Selection sel;
-    fp::Plan p;
     rc = fp::make_selection(c, sel_o, true, &sel, &err);
-    if (!rc) rc = fp::plan_rates(c, so, nT, sel, 0, &p, &err, fp::kPairMirror, split);
     if (rc) return fail(c, rc, "fp_rates4: " + err);
-    if (p.split) {
-      const size_t all = (size_t)nT * npass * nm;
-      if (c->rates_cap < all) {
-        dfree(c->d_rates);
-        c->rates_cap = 0;
-        FP_CUDA(c, dalloc(&c->d_rates, all));
-        c->rates_cap = all;
-      }
-      rc = run_planned(c, so, sel, p, nT, T, sb, c->d_rates, stats);
-      if (rc) return rc;
+    const size_t all = (size_t)nT * npass * nm;
+    if (c->rates_cap < all) {
+      dfree(c->d_rates);
+      c->rates_cap = 0;
+      FP_CUDA(c, dalloc(&c->d_rates, all));
+      c->rates_cap = all;
+    }
+    bool did_split = false;
+    rc = plan_and_run(c, so, sel, nT, T, sb, c->d_rates, stats, split, &did_split);
+    if (rc) return rc;
+    if (did_split) {
       std::vector<double> part(all);
       FP_CUDA(c, cudaMemcpyAsync(part.data(), c->d_rates, all * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
       FP_CUDA(c, cudaStreamSynchronize(c->stream));
@@ -807,37 +828,43 @@ int phase_pass(fp_ctx* c, const fp_rates_opts& o, int nT, const double* T, doubl
   fp::Selection sel;
   int rc = fp::make_selection(c, o, stride == 1, &sel, err);  // a q' stride is not symmetric under q -> -q
   if (rc) return rc;
-  fp::Plan p;
-  rc = fp::plan_rates(c, o, nT, sel, 0, &p, err, stride == 1 ? fp::kPairMirror : fp::kPairSliced);
-  if (rc) return rc;
-  if (stride > 1) {  // a q' tile of one stride: every item owns exactly one sampled q'
-    p.t1 = stride;
-    p.ntile = (c->N + stride - 1) / stride;
-    p.n_items = (long long)p.ntile * p.nq_sel * p.nchunk;
-    p.values = p.n_items * p.J;
-    if (p.ctas > p.n_items) p.ctas = (int)std::max<long long>(1, p.n_items);
+  for (const FormTry& f : kFormTries) {
+    if (f.budget || (f.form == fp::kPairMirror && stride > 1)) continue;  // a unit vertex needs no table U
+    fp::Plan p;
+    rc = fp::plan_rates(c, o, nT, sel, 0, &p, err, f.form);
+    if (rc) return rc;
+    if (stride > 1) {  // a q' tile of one stride: every item owns exactly one sampled q'
+      p.t1 = stride;
+      p.ntile = (c->N + stride - 1) / stride;
+      p.n_items = (long long)p.ntile * p.nq_sel * p.nchunk;
+      p.values = p.n_items * p.J;
+      if (p.ctas > p.n_items) p.ctas = (int)std::max<long long>(1, p.n_items);
+    }
+    p.psi_u = p.operands = false;  // no vertex
+    size_t sz[fp::kScratchParts], total = 0;
+    fp::scratch_sizes(c, p, nT, sz);
+    for (size_t x : sz) total += x;
+    const size_t cnt_bytes = (size_t)std::max<long long>(1, p.values) * sizeof(unsigned long long);
+    unsigned char* b = nullptr;
+    cudaError_t e = dalloc(&b, total + cnt_bytes);
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      if (f.form != fp::kOrdered) continue;
+      *err = std::string("cudaMalloc: ") + cudaGetErrorString(e);
+      return FP_ENOMEM;
+    }
+    const fp::Scratch sc = fp::carve_scratch(b, sz);
+    fp::RunExtra x;
+    x.unit_stride = stride;
+    x.unit_weights = unit_weights;
+    x.d_item_counts = reinterpret_cast<unsigned long long*>(b + total);
+    x.d_mode_counts = d_counts;
+    unsigned long long counts[fp::kCounters];
+    rc = fp::run_rates(c, o, sel, p, sc, nT, T, sb, d_out, counts, false, err, x);
+    cudaFree(b);
+    return rc;
   }
-  p.psi_u = p.operands = false;  // no vertex
-  size_t sz[fp::kScratchParts], total = 0;
-  fp::scratch_sizes(c, p, nT, sz);
-  for (size_t x : sz) total += x;
-  const size_t cnt_bytes = (size_t)std::max<long long>(1, p.values) * sizeof(unsigned long long);
-  unsigned char* b = nullptr;
-  cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&b), total + cnt_bytes);
-  if (e != cudaSuccess) {
-    *err = std::string("cudaMalloc: ") + cudaGetErrorString(e);
-    return FP_ENOMEM;
-  }
-  const fp::Scratch sc = fp::carve_scratch(b, sz);
-  fp::RunExtra x;
-  x.unit_stride = stride;
-  x.unit_weights = unit_weights;
-  x.d_item_counts = reinterpret_cast<unsigned long long*>(b + total);
-  x.d_mode_counts = d_counts;
-  unsigned long long counts[fp::kCounters];
-  rc = fp::run_rates(c, o, sel, p, sc, nT, T, sb, d_out, counts, false, err, x);
-  cudaFree(b);
-  return rc;
+  return FP_ENOMEM;  // not reached: the last form returns
 }
 
 }  // namespace

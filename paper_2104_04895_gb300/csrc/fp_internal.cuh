@@ -247,6 +247,8 @@ int plan_rates(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, size_t
                std::string* err, RateForm form = kPairMirror, int split = 0);
 // Most threads per block that a tile of these options may ask for.
 int max_tile_threads(const fp_ctx* c, const fp_rates_opts& o);
+// Give the context's working memory back where it exceeds 128 MiB: a call that needs as much takes seconds.
+void trim_scratch(fp_ctx* c);
 // Byte sizes of the Scratch buffers of a plan, in the order of the Scratch fields (each rounded up to 256).
 void scratch_sizes(const fp_ctx* c, const Plan& p, int nT, size_t sizes[kScratchParts]);
 // Scratch pointers laid out from `base` with the sizes of scratch_sizes.

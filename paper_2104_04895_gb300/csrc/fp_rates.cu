@@ -379,9 +379,11 @@ static int plan_form(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, 
   const long long mirror_values = (long long)nq_sel * N * nchunk * nb;
   const size_t mirror_bytes = (size_t)mirror_values * nS * sizeof(double);
   if (mirror && partial_budget && mirror_bytes > partial_budget) mirror = false;
-  if (mirror && mirror_bytes > (size_t(256) << 20) && mirror_bytes > c->scratch_cap) {
+  if (mirror && mirror_bytes > (size_t(256) << 20)) {
+    // at most a sixteenth of the device (18 GB), whatever is free of it: the same call takes the same form and gives the
+    // same bits beside any other program, unless the memory runs out
     size_t mem_free = 0, mem_total = 0;
-    mirror = cudaMemGetInfo(&mem_free, &mem_total) == cudaSuccess && mirror_bytes < mem_free / 2;
+    mirror = cudaMemGetInfo(&mem_free, &mem_total) == cudaSuccess && mirror_bytes <= mem_total / 16;
   }
   if (mirror && o.k1_tile <= 0 && t1_tuned <= 0) t1 = 1;
   // the table U of the Psi prologue, where a call may take the memory for it (1 MB on diamond 3^3, 138 MB on 16^3)
@@ -505,6 +507,13 @@ int plan_rates(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, size_t
   const int rc = plan_form(c, o, nT, sel, partial_budget, p, err, false, false, false, 0);
   if (rc == FP_EINVAL && !why.empty()) *err = why;
   return rc;
+}
+
+void trim_scratch(fp_ctx* c) {
+  if (c->scratch_cap <= (size_t(128) << 20)) return;
+  cudaFree(c->d_scratch);
+  c->d_scratch = nullptr;
+  c->scratch_cap = 0;
 }
 
 void scratch_sizes(const fp_ctx* c, const Plan& p, int nT, size_t s[kScratchParts]) {

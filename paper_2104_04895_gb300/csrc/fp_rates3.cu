@@ -571,6 +571,7 @@ extern "C" int fp_rates3(fp_ctx* c, int nT, const double* T, double scalebroad, 
   R3_CUDA(cudaMemcpyAsync(rates, dr, nT * nm * sizeof(double), cudaMemcpyDeviceToHost, s));
   R3_CUDA(cudaMemcpyAsync(cnt, dc, sizeof(cnt), cudaMemcpyDeviceToHost, s));
   R3_CUDA(cudaStreamSynchronize(s));
+  trim_scratch(c);
   if (stats) {
     std::memset(stats, 0, sizeof(*stats));
     double nsel = 0;

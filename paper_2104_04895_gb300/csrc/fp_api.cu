@@ -103,12 +103,11 @@ int neg_index(const fp_ctx* c, int q) {
 
 // Whether the quartet list obeys the transposition symmetry of Sec. 2.3 (Eq. TS) in the legs that the pair kernel
 // exchanges: (i, a) <-> (j, b), re-based to the new home cell, and (k, c) <-> (l, d).  Quartets listed more than once
-// add up.  The tolerance, 1e-13 of the largest entry, covers the rounding of symmetrised input and keeps the rates
-// within a few 1e-13 of those of the list as given.
+// add up.  The tolerance, 1e-13 of the largest entry of the two quartets compared, covers the rounding of symmetrised input
+// and keeps every vertex, also one that only small quartets make, within a few 1e-13 of that of the list as given.
 bool leg_symmetric(int n, const fp_fc4* fc4) {
   using Key = std::array<int, 13>;
   std::map<Key, std::array<double, 81>> sum;
-  double big = 0.0;
   for (int b = 0; b < n; ++b) {
     const fp_fc4& f = fc4[b];
     const Key key = {f.i, f.j, f.k, f.l, f.Rj[0], f.Rj[1], f.Rj[2], f.Rk[0], f.Rk[1], f.Rk[2], f.Rl[0], f.Rl[1], f.Rl[2]};
@@ -117,12 +116,13 @@ bool leg_symmetric(int n, const fp_fc4* fc4) {
       it = sum.emplace(key, std::array<double, 81>()).first;
       it->second.fill(0.0);
     }
-    for (int x = 0; x < 81; ++x) {
-      it->second[x] += f.fc[x];
-      big = std::max(big, std::fabs(f.fc[x]));
-    }
+    for (int x = 0; x < 81; ++x) it->second[x] += f.fc[x];
   }
-  const double tol = 1e-13 * big;
+  auto largest = [](const std::array<double, 81>& f) {
+    double m = 0.0;
+    for (double v : f) m = std::max(m, std::fabs(v));
+    return m;
+  };
   for (const auto& kv : sum) {
     const Key& q = kv.first;
     Key ij = {q[1], q[0], q[2], q[3], 0, 0, 0, 0, 0, 0, 0, 0, 0}, kl = {q[0], q[1], q[3], q[2], q[4], q[5], q[6], 0, 0, 0, 0, 0, 0};
@@ -134,6 +134,9 @@ bool leg_symmetric(int n, const fp_fc4* fc4) {
       kl[10 + d] = q[7 + d];
     }
     const auto pij = sum.find(ij), pkl = sum.find(kl);
+    const double own = largest(kv.second);
+    const double tij = 1e-13 * (pij == sum.end() ? own : std::max(own, largest(pij->second)));
+    const double tkl = 1e-13 * (pkl == sum.end() ? own : std::max(own, largest(pkl->second)));
     for (int al = 0; al < 3; ++al)
       for (int be = 0; be < 3; ++be)
         for (int ga = 0; ga < 3; ++ga)
@@ -141,7 +144,7 @@ bool leg_symmetric(int n, const fp_fc4* fc4) {
             const double v = kv.second[((al * 3 + be) * 3 + ga) * 3 + th];
             const double vij = pij == sum.end() ? 0.0 : pij->second[((be * 3 + al) * 3 + ga) * 3 + th];
             const double vkl = pkl == sum.end() ? 0.0 : pkl->second[((al * 3 + be) * 3 + th) * 3 + ga];
-            if (!(std::fabs(v - vij) <= tol) || !(std::fabs(v - vkl) <= tol)) return false;
+            if (!(std::fabs(v - vij) <= tij) || !(std::fabs(v - vkl) <= tkl)) return false;
           }
   }
   return true;

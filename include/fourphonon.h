@@ -38,8 +38,10 @@ extern "C" {
 #define FP_EUNSTABLE (-4)  /* omega^2 < -1e-8 max(omega^2) away from the three Gamma acoustic modes */
 #define FP_ESTATE (-6)     /* call out of order (e.g. rates before modes) */
 
-#define FP_PREC_FP64 0  /* vertex, Gaussian and sums in FP64, the contractions of six and twelve branches in exact integer
-                           slices of the same accuracy (parity path, 1e-10 vs the FP64 definition) */
+#define FP_PREC_FP64 0  /* vertex, Gaussian and sums in FP64 (parity path, 1e-10 vs the FP64 definition).  The contractions
+                           of six and twelve branches run in integer slices, exact to 2^-53 of the norm of their block; a
+                           call in which a rate comes from vertices too small beside that norm (more than 5e-13 of the
+                           rate lost) is evaluated again with FP64 contractions, which the stats' ms includes */
 #define FP_PREC_MIXED 1 /* vertex and Gaussian in FP32, window decisions exact, sums in FP64 */
 #define FP_PREC_DOUBLE_FLOAT 2 /* FP64 path whose vertex contraction (Eq. V4 assembly and the two contractions)
                                   runs on the FP32 pipes in double-float: pairs of floats with exact high products

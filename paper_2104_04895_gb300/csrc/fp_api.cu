@@ -557,10 +557,13 @@ static const FormTry kFormTries[] = {
 static int plan_and_run(fp_ctx* c, const fp_rates_opts& o, fp::Selection& sel, int nT, const double* T, double sb, double* d_out,
                         fp_stats* stats, int split = 0, bool* did_split = nullptr) {
   std::string err;
-  for (const FormTry& f : kFormTries) {
+  double spent = 0.0;  // ms of a run that the slices were too coarse for
+  bool slices = true;
+  for (int k = 0; k < 4; ++k) {
+    const FormTry& f = kFormTries[k];
     fp::Plan p;
-    int rc = fp::plan_rates(c, o, nT, sel, f.budget, &p, &err, f.form, split);
-    if (rc && &f != kFormTries) return fail(c, FP_ENOMEM, "fp_rates4: no memory for the form that takes these tiles");
+    int rc = fp::plan_rates(c, o, nT, sel, f.budget, &p, &err, f.form, split, slices);
+    if (rc && k > 0) return fail(c, FP_ENOMEM, "fp_rates4: no memory for the form that takes these tiles");
     if (rc) return fail(c, rc, "fp_rates4: " + err);
     if (did_split) *did_split = p.split != 0;
     if (split && !p.split) return FP_OK;
@@ -583,7 +586,16 @@ static int plan_and_run(fp_ctx* c, const fp_rates_opts& o, fp::Selection& sel, i
     rc = fp::run_rates(c, o, sel, p, sc, nT, T, sb, d_out, counts, o.no_graph == 0, &err);
     fp::trim_scratch(c);
     if (rc) return fail(c, rc, "fp_rates4: " + err);
-    if (stats) fp::fill_stats(c, o, sel, p, counts, stats);
+    fp_stats st;
+    fp::fill_stats(c, o, sel, p, counts, &st);
+    if (counts[fp::kCountWeak]) {
+      spent = st.ms;
+      slices = false;
+      k = -1;
+      continue;
+    }
+    st.ms += spent;
+    if (stats) *stats = st;
     return FP_OK;
   }
   return fail(c, FP_ENOMEM, "fp_rates4: no form fits");  // not reached: the last form returns

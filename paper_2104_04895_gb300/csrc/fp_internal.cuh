@@ -69,9 +69,9 @@ struct RatesArgs {
   double rec[9];
   double* partial;           // [n_items][J][nT]
   unsigned long long* counter;
-  unsigned long long* counts; // [8]: accepted ++, +-, -- (weighted by mult), vertex entries W formed, accepted
+  unsigned long long* counts; // [9]: accepted ++, +-, -- (weighted by mult), vertex entries W formed, accepted
                               // terms evaluated, tensor-core completion waits that ran out of polls, (pair kernel)
-                              // (q, q', q'') iterations and (q, q') pairs evaluated
+                              // (q, q', q'') iterations and (q, q') pairs evaluated, rates too weak for the slices
   int unit_vertex;           // 1: |W|^2 = 1 (weighted phase space), q' on a stride, ordered (q', q'') pairs
   int k1_stride;             // q' stride of the unit-vertex mode
   unsigned cand_mask;        // candidates summed (bit c = ordering * 3 + process), from process_mask
@@ -97,6 +97,8 @@ struct RatesArgs {
   const float* rec32;        // [N][DenseRecord::size] records of the mixed path (fp_dense_kernel.cuh)
   const double2* psi_u;      // [nq_sel][nb][nterm][3][9] table U of the evaluated points (psi_u_kernel), or null
   const unsigned* operands;  // [N][2][Shape::kOperand] sliced eigenvectors in fragment order (fp_slices.cuh)
+  double* weak;              // [nS][N*nb] what the weak vertices of an evaluated mode would add at their block's scale
+                             // (fp_slices.cuh), or null
 };
 
 // Which q-points a rates call evaluates, and for which modes.  Time reversal (e^{-lambda} = conj e^{lambda},
@@ -131,10 +133,11 @@ struct Plan {
 };
 
 // Device working memory of one rates call (owned by the caller of run_rates), in the order of scratch_sizes.
-constexpr int kScratchParts = 19;
+constexpr int kScratchParts = 20;
 constexpr int kScratchPartial = 7;  // index of the per-item partial sums
+constexpr int kCountWeak = 9;
 constexpr int kCounters = 10;       // queue, accepted ++, +-, --, vertex entries, terms evaluated, wait timeouts,
-                                    // iterations, pairs, spare
+                                    // iterations, pairs, rates too weak for the slices
 struct Scratch {
   unsigned long long* counters;  // [kCounters]
   double* T;                     // [kMaxT]
@@ -155,6 +158,7 @@ struct Scratch {
   double2* psi_u;                // [nq_sel][nb][nterm][3][9] (pair kernel, where it fits)
   float* rec32;                  // [N][DenseRecord::size] (dense mixed kernel)
   unsigned* operands;            // [N][2][Shape::kOperand] (sliced pair kernel)
+  double* weak;                  // [nS][N*nb] (sliced pair kernel)
 };
 
 }  // namespace fp
@@ -242,9 +246,10 @@ int make_selection(const fp_ctx* c, const fp_rates_opts& o, bool fold_allowed, S
 // FP_E* code with a message in *err.
 enum RateForm { kOrdered = 0, kPair = 1, kPairSliced = 2, kPairMirror = 3 };
 // `split` keeps the parts of the rates apart (RatesArgs::split) where the pair kernel runs and they fit kMaxT sums;
-// Plan::split says whether it does.
+// Plan::split says whether it does.  `slices` admits the contractions in slices; a run of theirs that leaves
+// counts[kCountWeak] nonzero is to be repeated without.
 int plan_rates(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, size_t partial_budget, Plan* p,
-               std::string* err, RateForm form = kPairMirror, int split = 0);
+               std::string* err, RateForm form = kPairMirror, int split = 0, bool slices = true);
 // Most threads per block that a tile of these options may ask for.
 int max_tile_threads(const fp_ctx* c, const fp_rates_opts& o);
 // Give the context's working memory back where it exceeds 128 MiB: a call that needs as much takes seconds.

@@ -101,45 +101,56 @@ extern "C" int fp_rates4_noalloc(fp_ctx* c, int nT, const double* T, double sb, 
   fp::Selection sel;
   int rc = fp::make_selection(c, o, true, &sel, &err);
   if (rc) return nfail(c, rc, "fp_rates4_noalloc: " + err);
-  fp::Plan p0;
   fp_rates_opts o_probe = o;
   if (o_probe.k1_tile <= 0) o_probe.k1_tile = c->N;  // smallest partials, for the fixed-size part
-  size_t sz[fp::kScratchParts], fixed = 0;
-  fp::RateForm form = fp::kPairMirror;
-  for (;;) {  // simpler forms of the rate kernel need less scratch
-    rc = fp::plan_rates(c, o_probe, nT, sel, 0, &p0, &err, form == fp::kPairMirror ? fp::kPairSliced : form);
+  double spent = 0.0;  // ms of a run that the slices were too coarse for
+  for (const bool slices : {true, false}) {
+    fp::Plan p0;
+    size_t sz[fp::kScratchParts], fixed = 0;
+    fp::RateForm form = fp::kPairMirror;
+    for (;;) {  // simpler forms of the rate kernel need less scratch
+      rc = fp::plan_rates(c, o_probe, nT, sel, 0, &p0, &err, form == fp::kPairMirror ? fp::kPairSliced : form, 0, slices);
+      if (rc) return nfail(c, rc, "fp_rates4_noalloc: " + err);
+      p0.psi_u = false;  // a plan with a budget, like the one below, has no table U
+      fp::scratch_sizes(c, p0, nT, sz);
+      fixed = 0;
+      for (int i = 0; i < fp::kScratchParts; ++i)
+        if (i != fp::kScratchPartial) fixed += sz[i];
+      if (fixed + sz[fp::kScratchPartial] <= kScratchBytes || form == fp::kOrdered) break;
+      form = form == fp::kPairMirror ? fp::kPair : fp::kOrdered;
+    }
+    if (fixed + sz[fp::kScratchPartial] > kScratchBytes)
+      return nfail(c, FP_EINVAL, "fp_rates4_noalloc: this problem needs at least " +
+                                     std::to_string(fixed + sz[fp::kScratchPartial]) +
+                                     " bytes of scratch; the static scratch holds " + std::to_string(kScratchBytes) +
+                                     " bytes (use fp_rates4_device)");
+    fp::Plan p;
+    rc = fp::plan_rates(c, o, nT, sel, kScratchBytes - fixed - 256, &p, &err, form, 0, slices);
     if (rc) return nfail(c, rc, "fp_rates4_noalloc: " + err);
-    p0.psi_u = false;  // a plan with a budget, like the one below, has no table U
-    fp::scratch_sizes(c, p0, nT, sz);
-    fixed = 0;
-    for (int i = 0; i < fp::kScratchParts; ++i)
-      if (i != fp::kScratchPartial) fixed += sz[i];
-    if (fixed + sz[fp::kScratchPartial] <= kScratchBytes || form == fp::kOrdered) break;
-    form = form == fp::kPairMirror ? fp::kPair : fp::kOrdered;
-  }
-  if (fixed + sz[fp::kScratchPartial] > kScratchBytes)
-    return nfail(c, FP_EINVAL, "fp_rates4_noalloc: this problem needs at least " +
-                                   std::to_string(fixed + sz[fp::kScratchPartial]) +
-                                   " bytes of scratch; the static scratch holds " + std::to_string(kScratchBytes) +
-                                   " bytes (use fp_rates4_device)");
-  fp::Plan p;
-  rc = fp::plan_rates(c, o, nT, sel, kScratchBytes - fixed - 256, &p, &err, form);
-  if (rc) return nfail(c, rc, "fp_rates4_noalloc: " + err);
-  fp::scratch_sizes(c, p, nT, sz);
-  size_t total = 0;
-  for (size_t x : sz) total += x;
-  if (total > kScratchBytes)
-    return nfail(c, FP_EINVAL, "fp_rates4_noalloc: this problem needs " + std::to_string(total) +
-                                   " bytes of scratch; the static scratch holds " + std::to_string(kScratchBytes) +
-                                   " bytes (use fp_rates4_device)");
+    fp::scratch_sizes(c, p, nT, sz);
+    size_t total = 0;
+    for (size_t x : sz) total += x;
+    if (total > kScratchBytes)
+      return nfail(c, FP_EINVAL, "fp_rates4_noalloc: this problem needs " + std::to_string(total) +
+                                     " bytes of scratch; the static scratch holds " + std::to_string(kScratchBytes) +
+                                     " bytes (use fp_rates4_device)");
 
-  unsigned char* b = nullptr;
-  NA_CUDA(c, scratch_address(c->device, &b));
-  const fp::Scratch sc = fp::carve_scratch(b, sz);
-  // run_rates clears the counters and the output on every call (the array keeps the last call's contents)
-  unsigned long long counts[fp::kCounters] = {0};
-  rc = fp::run_rates(c, o, sel, p, sc, nT, T, sb, d_out, counts, false, &err);
-  if (rc) return nfail(c, rc, "fp_rates4_noalloc: " + err);
-  if (stats) fp::fill_stats(c, o, sel, p, counts, stats);
-  return FP_OK;
+    unsigned char* b = nullptr;
+    NA_CUDA(c, scratch_address(c->device, &b));
+    const fp::Scratch sc = fp::carve_scratch(b, sz);
+    // run_rates clears the counters and the output on every call (the array keeps the last call's contents)
+    unsigned long long counts[fp::kCounters] = {0};
+    rc = fp::run_rates(c, o, sel, p, sc, nT, T, sb, d_out, counts, false, &err);
+    if (rc) return nfail(c, rc, "fp_rates4_noalloc: " + err);
+    fp_stats st;
+    fp::fill_stats(c, o, sel, p, counts, &st);
+    st.ms += spent;
+    if (counts[fp::kCountWeak]) {
+      spent = st.ms;
+      continue;
+    }
+    if (stats) *stats = st;
+    return FP_OK;
+  }
+  return nfail(c, FP_ECUDA, "fp_rates4_noalloc: no form ran");  // not reached: the second pass returns
 }

@@ -35,7 +35,9 @@
 // On the FP64 path with 6 or 12 branches and unit eigenvectors both vertex contractions run on the tensor cores in exact
 // integer slices (SL, fp_slices.cuh): A is built in FP64, its digits contract with those of e3 to T, T's digits with those of e2 to
 // every W of the block, which costs the FP64 pipe only the A sums and |W|^2.  A scale per (j0, x), the power of two
-// above the Frobenius norm of its A block, keeps all three in range.
+// above the Frobenius norm of its A block, keeps all three in range.  Terms whose W is below 2^-12 of that scale are
+// bounded a second time at the scale itself (sWeak, a.weak), from which the reduction sees the rates that need the FP64
+// contraction (fp_slices.cuh).
 //
 // Measured (GB300): ordered kernel -> pair kernel -> with slices and the U table of the prologue -> with U over terms and
 // several items per pair on small grids:
@@ -150,7 +152,9 @@ __host__ __device__ inline PairCarve make_pair_carve(int nb, int J, int G, int n
   // T blocks (j0, x), padded by one entry; sliced: rows of digits of A and then of T, later |W|^2 and the lists
   c.T = o; o += sliced ? nwarps * 32 * (nb == 6 ? 36 : 76) / 4 : (size_t)J * nb * (nb2 + 1);
   c.Tw2 = o; o += G;
-  c.TwQ = o; o += nquart;
+  // phases of the prologue; sliced: then the weak terms [S1, S4, S5][j0 x][largest of each sum, count]
+  const size_t weak = sliced ? (3 * (size_t)J * nb * (nS + 1) + 3) / 4 : 0;
+  c.TwQ = o; o += weak > (size_t)nquart ? weak : (size_t)nquart;
   c.Op = o; o += sliced ? 2 * 6 * (nb == 6 ? 2 * 32 * 2 : 3 * 32 * 3) / 4 : 0;
   c.ncx = o;
   size_t d = 0;
@@ -218,6 +222,13 @@ __device__ __noinline__ double pair_two_orders(double ex, double z8, const doubl
   return 0.5 * (ex + pair_exp_neg64(z8, tab));
 }
 
+// a weak term (rare: out of line): its number, and per sum the largest factor by its high word (shared memory adds doubles
+// in a loop of compare and swap)
+__device__ __noinline__ void pair_weak(int* wk, int nS, int lo, int nT, double gv, const double* wb, int stride) {
+  atomicAdd(wk + nS, 1);
+  for (int t = 0; t < nT; ++t) atomicMax(wk + lo + t, __double2hiint(wb ? gv * wb[t * stride] : gv));
+}
+
 // NB branches, up to MAXT sums per row.  DF: vertex contraction in double-float on the FP32 pipes (the terms in FP64: the
 // weights of c and d fall as exp(-hbar (wc + wd) / k_B T), out of FP32's range at 10 to 20 K).  SL: both vertex contractions on the tensor cores in exact slices (fp_slices.cuh; unit eigenvectors, nb = 6 or 12): A in FP64,
 // T as digits, |W|^2 of every entry in FP64.
@@ -247,6 +258,7 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
   const unsigned* sOp = reinterpret_cast<const unsigned*>(cx + cv.Op);
   double* sVal = (SL ? reinterpret_cast<double*>(sW + (size_t)J * NB * NB2) : db + cv.Val) + (size_t)warp * kPairCap;
   double* sRed = reinterpret_cast<double*>(sT);  // the T block, free outside the k2 loop
+  int* sWeak = reinterpret_cast<int*>(sTwQ);
   float* fb = reinterpret_cast<float*>(db + cv.ndbl);
   float *sH0 = fb + cv.H0, *sH1 = fb + cv.H1, *sH2 = fb + cv.H2, *sH3 = fb + cv.H3;
   float *sVH2 = fb + cv.VH2, *sVL2 = fb + cv.VL2, *sVH3 = fb + cv.VH3, *sVL3 = fb + cv.VL3;
@@ -446,6 +458,7 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
         // A, T and W (unit eigenvectors)
         double* sB = reinterpret_cast<double*>(sT);
         __syncthreads();
+        for (int o = tid; o < 3 * J * NB * (nS + 1); o += nthr) sWeak[o] = 0;
         if (!unit && any) {
           for (int o = tid; o < J * NB * NB2; o += nthr) {
             const int ab = o / NB2, k = (o / NB) % NB, l = o % NB;
@@ -465,7 +478,7 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
           for (int ab = tid; ab < J * NB; ab += nthr) {
             double f = 0.0;
             for (int o = 0; o < NB2; ++o) f += sB[ab * NB2 + o];
-            sSc[ab] = f > 0.0 ? (f < 1e300 ? ilogb(sqrt(f) * 1.0001) + 1 : 1000) : 0;
+            sSc[ab] = f > 0.0 ? (f < 1e300 ? ilogb(sqrt(f) * 1.0001) + 1 : 1000) : -600;  // -600: W is zero, not weak
           }
         }
       }
@@ -974,8 +987,16 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
                     ex = pair_two_orders(ex, add_signed(add_signed(wx, y2, plus1), y1, plus2) * iv8, sExpT);
                   gv *= ex;
                 }
-                double v = W2 * gv;
-                if (en & 1024u) v *= 0.5;
+                if (en & 1024u) gv *= 0.5;
+                const double v = W2 * gv;
+                if constexpr (SL) {
+                  // |W|^2 is in units of (2^(s - 51))^2
+                  if (__double2hiint(W2) < (1023 + 102 + 2 * slices::kWeakExponent) << 20 && !unit) {
+                    pair_weak(sWeak + ((kind < 3 ? 0 : kind - 2) * J * NB + ab) * (nS + 1), nS,
+                              MAXT == 1 ? 0 : part_of(kind, umask) * nT, MAXT == 1 ? 1 : nT, gv,
+                              MAXT == 1 ? nullptr : sWB + (kind < 3 ? kind : 0) * NB2 + e, 3 * NB2);
+                  }
+                }
                 sVal[i] = v;
               }
               __syncwarp();
@@ -1041,6 +1062,25 @@ __global__ void __launch_bounds__(pair_threads_for(NB), pair_blocks_for(NB)) pai
             }
           } else {
             a.partial[((direct ? slot : mslot) * NB + m) * nS + t] = sum;
+          }
+          if constexpr (SL) {
+            if (!unit) {
+              // bound of the weak terms at their block's scale; the order of these additions decides no bit of a rate
+              double weak = 0.0;
+              for (int o = 0; o < (direct ? NB : J); ++o) {
+                const int ab = (direct ? m : o) * NB + (direct ? o : m);
+                auto bound = [&](int k) {
+                  const int* wk = sWeak + (k * J * NB + ab) * (nS + 1);
+                  return wk[t] ? wk[nS] * __hiloint2double(wk[t] + 1, 0) : 0.0;
+                };
+                const double w1 = bound(0), w2 = bound(direct ? 1 : 2);
+                const double* wo = W + 3 * (direct ? (size_t)k1 * NB + o : (size_t)q * NB + j0b + o);
+                if (w1 > 0.0 || w2 > 0.0) weak += (wo[1] * w1 + wo[2] * ((1.0 / 3.0) * w2)) * scalbn(1.0, 2 * sSc[ab]);
+              }
+              if (weak > 0.0)
+                atomicAdd(a.weak + (size_t)t * NM + (direct ? (size_t)q * NB + j0b + m : (size_t)rq * NB + m),
+                          weak * W[3 * (direct ? (size_t)q * NB + j0b + m : (size_t)k1 * NB + m)] * s_down[t % nT]);
+            }
           }
         }
         __syncthreads();

@@ -62,6 +62,11 @@ __global__ void prep_kernel(RatesArgs a, float* omh, float* oml, float* velh, fl
   }
 }
 
+// Whether the weak vertices of the evaluated mode (q, j) leave its sum s less than FP64's accuracy (fp_slices.cuh)
+__device__ __forceinline__ bool too_weak(const RatesArgs& a, int q, int j, int t, double s) {
+  return a.weak && a.weak[((size_t)t * a.N + q) * a.nb + j] * slices::kWeakLimit > s;
+}
+
 // rates[t][q][j] = pref * sum_tiles partial[(tile, qpos[q], chunk)][jj][t], in a fixed order, for every selected
 // mode of the output range (the others stay zero); under time reversal q and -q read the same partial sums.
 __global__ void reduce_kernel(RatesArgs a, double pref, double* rates) {
@@ -79,6 +84,7 @@ __global__ void reduce_kernel(RatesArgs a, double pref, double* rates) {
     const long long item = ((long long)tile * a.nq_sel + qi) * a.nchunk + chunk;
     s += a.partial[((size_t)item * a.J + jj) * a.nS + t];
   }
+  if (too_weak(a, a.qlist[qi], j, t, s)) atomicAdd(a.counts + kCountWeak - 1, 1ULL);
   rates[((size_t)t * a.N + q) * a.nb + j] = s * pref;
   if (a.mode_counts && t == 0) {
     unsigned long long cnt = 0;
@@ -126,6 +132,7 @@ __global__ void pair_reduce_kernel(RatesArgs a, double pref, double* rates) {
     cnt += __shfl_down_sync(0xffffffffu, cnt, off);
   }
   if (lane) return;
+  if (too_weak(a, qe, j, t, s)) atomicAdd(a.counts + kCountWeak - 1, 1ULL);
   rates[((size_t)t * a.N + q) * a.nb + j] = s * pref;
   if (a.mode_counts && t == 0) a.mode_counts[(size_t)q * a.nb + j] = (double)cnt * a.count_scale;
 }
@@ -480,7 +487,7 @@ int max_tile_threads(const fp_ctx* c, const fp_rates_opts& o) {
 }
 
 int plan_rates(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, size_t partial_budget, Plan* p,
-               std::string* err, RateForm form, int split) {
+               std::string* err, RateForm form, int split, bool slices) {
   if (nT * (split == 1 ? 2 : 3) > kMaxT) split = 0;
   // Where the pair kernel's tables do not fit, the ordered kernel runs; if neither runs, the first one's reason stands, whose
   // limits are the wider ones.  The mixed path keeps the ordered kernel: its FP32 vertex rounds
@@ -488,7 +495,7 @@ int plan_rates(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, size_t
   std::string why;
   if (form != kOrdered && over_pairs(c, o)) {
     // the FP64 path's contraction in slices: 6 and 12 branches (with 3, K = 6 would leave most of a tile empty)
-    if (form != kPair && o.precision == FP_PREC_FP64 && c->unit_modes && c->nb >= 6) {
+    if (slices && form != kPair && o.precision == FP_PREC_FP64 && c->unit_modes && c->nb >= 6) {
       const int rc = plan_form(c, o, nT, sel, partial_budget, p, err, true, true, form == kPairMirror, split);
       if (rc != FP_EINVAL) return rc;
     }
@@ -536,6 +543,7 @@ void scratch_sizes(const fp_ctx* c, const Plan& p, int nT, size_t s[kScratchPart
   s[15] = up256(3 * nm * nT * sizeof(float));
   s[18] = p.dense ? up256((size_t)c->N * make_record(c->nb, c->G, nT).size * sizeof(float)) : 0;
   s[17] = p.psi_u ? up256((size_t)p.nq_sel * c->nb * c->nterm * 27 * sizeof(double2)) : 0;
+  s[19] = p.operands ? up256(nm * p.nS * sizeof(double)) : 0;
   s[16] = p.operands ? up256((size_t)c->N * operand_words(c->nb) * sizeof(unsigned)) : 0;
 }
 
@@ -565,6 +573,7 @@ Scratch carve_scratch(unsigned char* b, const size_t sz[kScratchParts]) {
   sc.operands = reinterpret_cast<unsigned*>(b + off[16]);
   sc.psi_u = reinterpret_cast<double2*>(b + off[17]);
   sc.rec32 = reinterpret_cast<float*>(b + off[18]);
+  sc.weak = reinterpret_cast<double*>(b + off[19]);
   return sc;
 }
 
@@ -646,6 +655,7 @@ int run_rates(fp_ctx* c, const fp_rates_opts& o, const Selection& sel, const Pla
   a.wtf = sc.wtf;
   a.operands = sc.operands;
   a.rec32 = sc.rec32;
+  a.weak = p.operands ? sc.weak : nullptr;
   a.psi_u = p.psi_u ? sc.psi_u : nullptr;
   a.sb = sb;
   a.window = o.window;
@@ -711,6 +721,7 @@ int run_rates(fp_ctx* c, const fp_rates_opts& o, const Selection& sel, const Pla
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     if (p.operands) {
+      if ((e = cudaMemsetAsync(sc.weak, 0, nm * p.nS * sizeof(double), s)) != cudaSuccess) return e;
       if (nb == 6)
         operand_kernel<6><<<4 * 152, 256, 0, s>>>(c->d_evec, N, sc.operands);
       else

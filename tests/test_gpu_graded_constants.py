@@ -2,12 +2,14 @@
 sublattice each: the ++ and -- parts of such a crystal come from vertices 1e-8 times the largest of their block, and have
 to reach the FP64 bar like the others (a contraction in fixed point below one scale per block would lose them); a list
 whose small quartets are not symmetric in their legs has to be evaluated as it is given."""
+import ctypes
+
 import numpy as np
 import pytest
 
 import oracle
 from paper_2104_04895_gb300 import synth
-from paper_2104_04895_gb300.binding import FP_PREC_DOUBLE_FLOAT, FP_PREC_FP64, Context
+from paper_2104_04895_gb300.binding import FP_OK, FP_PREC_DOUBLE_FLOAT, FP_PREC_FP64, Context, fp_stats
 
 from conftest import oracle_modes
 
@@ -61,6 +63,46 @@ def _close(got, ref):
     assert np.max(np.abs(got[~zero] - ref[~zero]) / ref[~zero]) <= RTOL
 
 
+@pytest.mark.parametrize("precision", [FP_PREC_FP64, FP_PREC_DOUBLE_FLOAT])
+@pytest.mark.parametrize("temps", [[300.0], [250.0, 900.0]])
+@pytest.mark.parametrize("maker,light", CASES)
+def test_weak_vertices_keep_their_accuracy(maker, light, temps, precision):
+    cr, _ = _crystal(maker, light)
+    w, e, v = _modes(cr, light, 3)
+    nT = len(temps)
+    refs = [oracle.rates4(cr, w, e, v, temps=temps, processes=(p,)) for p in range(3)]
+    full, acc = oracle.rates4(cr, w, e, v, temps=temps)
+    with Context.from_crystal(cr) as ctx:
+        ctx.set_modes(w, e, v)
+        ch, st = ctx.rates4_channels(temps, cr.scalebroad, precision=precision)
+        assert st["accepted"] == [refs[p][1][p] for p in range(3)]
+        for p in range(3):
+            _close(ch[:, p].reshape(nT, -1), refs[p][0])
+            one, _ = ctx.rates4(temps, cr.scalebroad, precision=precision, process_mask=1 << p)
+            _close(one.reshape(nT, -1), refs[p][0])
+        out, st = ctx.rates4(temps, cr.scalebroad, precision=precision)
+        _close(out.reshape(nT, -1), full)
+        assert st["accepted"] == list(acc)
+
+
+@pytest.mark.parametrize("maker,light", CASES)
+def test_weak_vertices_without_allocation(maker, light):
+    import torch
+    cr, _ = _crystal(maker, light)
+    w, e, v = _modes(cr, light, 5)
+    T = np.array([300.0])
+    ref, acc = oracle.rates4(cr, w, e, v, temps=T, processes=(2,))
+    with Context.from_crystal(cr) as ctx:
+        ctx.set_modes(w, e, v)
+        out = torch.zeros(cr.nq * cr.nb, dtype=torch.float64, device="cuda")
+        o, st = ctx.make_opts(process_mask=4)[0], fp_stats()
+        rc = ctx.L.fp_rates4_noalloc(ctx.h, 1, T.ctypes.data_as(ctypes.POINTER(ctypes.c_double)), cr.scalebroad,
+                                     ctypes.byref(o), ctypes.c_void_p(out.data_ptr()), ctypes.byref(st))
+        assert rc == FP_OK, ctx.L.fp_last_error(ctx.h)
+        _close(out.cpu().numpy().reshape(1, -1), ref)
+        assert list(st.accepted) == list(acc)
+
+
 @pytest.mark.parametrize("maker,light", CASES)
 def test_small_asymmetric_quartets_count(maker, light):
     """The small quartets lose the symmetry under i <-> j by 1e-5 of their size (1e-13 of the largest quartet), keeping
@@ -79,3 +121,16 @@ def test_small_asymmetric_quartets_count(maker, light):
             ref, _ = oracle.rates4(cr, w, e, v, processes=(p,))
             out, _ = ctx.rates4(cr.temps, cr.scalebroad, process_mask=1 << p)
             _close(out.reshape(len(cr.temps), -1), ref)
+
+
+@pytest.mark.parametrize("maker", [lambda: synth.diamond_si((4, 3, 3)), lambda: synth.zincblende_bas((4, 3, 2)),
+                                   lambda: synth.licoo2((3, 2, 2))])
+@pytest.mark.parametrize("temps", [[300.0], [20.0, 100.0, 900.0]])
+def test_ordinary_crystals_keep_the_fast_contraction(maker, temps):
+    """Every entry of an evaluated row is formed there, exactly one per accepted term in the other pair kernels."""
+    cr = maker()
+    w, e, v = oracle_modes(cr)
+    with Context.from_crystal(cr) as ctx:
+        ctx.set_modes(w, e, v)
+        _, st = ctx.rates4(temps, cr.scalebroad)
+        assert st["vertex_entries"] != st["terms_executed"]

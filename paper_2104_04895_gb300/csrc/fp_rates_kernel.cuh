@@ -152,11 +152,12 @@ __device__ __forceinline__ float4 cdf_norm(float4 a) {
   const float rs = __fadd_rn(a.x, a.y), is = __fadd_rn(a.z, a.w);
   return make_float4(rs, __fsub_rn(a.y, __fsub_rn(rs, a.x)), is, __fsub_rn(a.w, __fsub_rn(is, a.z)));
 }
-// |w|^2 in double from a double-float complex: squares with exact high products, two-sum of the two squares
+// |w|^2 in double from a double-float complex: squares with exact high products and
+// those of the low parts (2^-50 of the result, of one sign: without them every rate came out 6e-16 low), two-sum of both
 __device__ __forceinline__ double cdf_abs2(float4 w) {
   const float ph = __fmul_rn(w.x, w.x), qh = __fmul_rn(w.z, w.z);
-  const float pe = __fmaf_rn(2.0f * w.x, w.y, __fmaf_rn(w.x, w.x, -ph));
-  const float qe = __fmaf_rn(2.0f * w.z, w.w, __fmaf_rn(w.z, w.z, -qh));
+  const float pe = __fmaf_rn(2.0f * w.x, w.y, __fmaf_rn(w.y, w.y, __fmaf_rn(w.x, w.x, -ph)));
+  const float qe = __fmaf_rn(2.0f * w.z, w.w, __fmaf_rn(w.w, w.w, __fmaf_rn(w.z, w.z, -qh)));
   const float s = __fadd_rn(ph, qh);
   const float bb = __fsub_rn(s, ph);
   const float t = __fadd_rn(__fsub_rn(ph, __fsub_rn(s, bb)), __fsub_rn(qh, bb));

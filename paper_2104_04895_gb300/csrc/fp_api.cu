@@ -846,7 +846,7 @@ int phase_pass(fp_ctx* c, const fp_rates_opts& o, int nT, const double* T, doubl
   for (const FormTry& f : kFormTries) {
     if (f.budget || (f.form == fp::kPairMirror && stride > 1)) continue;  // a unit vertex needs no table U
     fp::Plan p;
-    rc = fp::plan_rates(c, o, nT, sel, 0, &p, err, f.form);
+    rc = fp::plan_rates(c, o, nT, sel, 0, &p, err, f.form, 0, false);  // nothing to contract in slices
     if (rc) return rc;
     if (stride > 1) {  // a q' tile of one stride: every item owns exactly one sampled q'
       p.t1 = stride;

@@ -156,6 +156,14 @@ def alu_peaks(torch, device_index):
     return fp64, fp32, basis
 
 
+def sliced_flops(binding, prec, st, nb):
+    """Flops of a rate set that run as integer slices on the tensor cores instead of the FP64 pipe: with 6 or 12 branches
+    the FP64 path forms T and W of every entry there, 8 nb flops each (a rate set without slices forms one W per
+    evaluated term)."""
+    sliced = prec == binding.FP_PREC_FP64 and nb in (6, 12) and st["vertex_entries"] != st["terms_executed"]
+    return 16.0 * nb * st["vertex_entries"] if sliced else 0.0
+
+
 def e2e_input_bytes(binding, cr):
     """Bytes a step hands the library from host memory: the buffers passed to fp_init (lattice, positions,
     masses, the packed Phi2 and Phi4 lists), fp_set_fc3 (packed Phi3) and fp_rates4 (temperatures), measured from
@@ -313,7 +321,11 @@ def main():
     # algorithmic flops per launch: the vertex work of this factorization (fp_stats.flops) plus the
     # accumulation of every accepted term at every temperature (Gaussian, Bose weights, |W|^2: 25 flops)
     acc_flops = FLOPS_PER_ACCEPTED_TERM * st["terms_executed"] * nT
-    achieved_tflops = (st["flops"] + acc_flops) / (kms * 1e-3) / 1e12
+    tensor_flops = sliced_flops(binding, main_prec, st, nb)
+    achieved_tflops = (st["flops"] - tensor_flops + acc_flops) / (kms * 1e-3) / 1e12
+    # kernels per step: Bose weights, FP32 tables, rate kernel, reduction; the tables U (kernel over pairs), sliced
+    # eigenvectors and mixed records of the forms that have them
+    launches = 4 + (1 if main_prec != binding.FP_PREC_MIXED else 1 if nb in (3, 6) else 0) + (1 if tensor_flops else 0)
     fp64_peak, fp32_peak, peak_basis = alu_peaks(torch, local)
     peak = fp32_peak if main_prec == binding.FP_PREC_MIXED else fp64_peak
     other = None
@@ -322,7 +334,8 @@ def main():
                                            args.steps, args.warmup, barrier)
         o_ms = max_over_ranks(o_ms, dist if ws > 1 else None, dev)
         o_peak = fp64_peak if other_prec == binding.FP_PREC_FP64 else fp32_peak
-        o_ach = (o_st["flops"] + FLOPS_PER_ACCEPTED_TERM * o_st["terms_executed"] * nT) / (o_kms * 1e-3) / 1e12
+        o_ach = (o_st["flops"] - sliced_flops(binding, other_prec, o_st, nb) +
+                 FLOPS_PER_ACCEPTED_TERM * o_st["terms_executed"] * nT) / (o_kms * 1e-3) / 1e12
         other = {"precision": "fp64" if other_prec == binding.FP_PREC_FP64 else "mixed",
                  "value": cands_step * args.steps / (o_ms * 1e-3), "unit": "process-terms/s",
                  "s_per_rate_set": o_ms / args.steps * 1e-3, "tile": o_st["tile"],
@@ -440,9 +453,9 @@ def main():
                          "pipe": "fp32" if main_prec == binding.FP_PREC_MIXED else "fp64",
                          "kernel_ms": kms, "flops_per_launch": st["flops"] + acc_flops,
                          "flops_vertex": st["flops"], "flops_accumulate": acc_flops,
-                         "note": None if main_prec != binding.FP_PREC_FP64 else
-                         "executed flops of the algorithm over the FP64 pipe's peak; with 6 or 12 branches the two "
-                         "vertex contractions run off that pipe, as exact integer slices on the tensor cores"},
+                         "flops_tensor_slices": tensor_flops,
+                         "note": "achieved and frac count the flops of the named pipe: flops_per_launch without "
+                         "flops_tensor_slices, the contractions that run as integer slices on the tensor cores"},
             "other_precision": other,
             "mixed_tensor_cores": tensor,
             "double_float": dfl,
@@ -451,7 +464,7 @@ def main():
             "cpu_baseline": base,
             "e2e": {"value": e2e_value, "unit": "process-terms/s", "h2d_bytes_per_step": h2d,
                     "d2h_bytes_per_step": d2h, "s_per_rate_set": e2e_s},
-            "gpu_launches": 4 * args.steps,  # per timed step: Bose weights, FP32 tables, rate kernel, reduction
+            "gpu_launches": launches * args.steps,
             "clocks": clk.summary(),
         }
         print(json.dumps(line), flush=True)
@@ -616,16 +629,18 @@ def measure_workload(binding, wl, budget_slice_s=10.0, full_max_s=300.0, oracle_
     An FP64 or mixed rate set estimated (from a one-q probe) to stay under `full_max_s` is timed on the whole grid,
     a double-float one under `df_full_max_s` (default: the same), and the tensor-core option (nb = 6 only) when
     `tensor_cores` is set and the mixed set ran in full.  Otherwise three strided q-slices (q = k mod m, all
-    branches) of about `budget_slice_s` each are timed and scaled to the grid
-    by the candidates the kernel screened (time reversal evaluates (N + self-conjugate points) / 2 points of a full
-    grid); the spread of the three gives the sampling uncertainty.  The rates use the library's own modes
+    branches) of about `budget_slice_s` each are timed and scaled to the grid by the work of their evaluated points (time
+    reversal evaluates (N + self-conjugate points) / 2 points of a full grid): n points are n N ordered pairs (q, q') in
+    the mixed path and n (N - n) pairs in the others, which evaluate a pair of two such points once.  The spread of the
+    three gives the sampling uncertainty.  The rates use the library's own modes
     (fp_modes); with `oracle_check`, the oracle (the CPU-baseline leg of this record) recomputes a ruled mode sample
     (lowest positive frequency and one seeded mode) from the same mode tables, so the error is a strict one; it runs
     only where it finishes within `oracle_max_s` on the host cores."""
     cr = synth.workload(wl)
     N, nb, nT = cr.nq, cr.nb, len(cr.temps)
     cands = 3.0 * N ** 3 * nb ** 4
-    full_exec = 3.0 * N * N * nb ** 3 * nb * (N + _self_conjugate(cr.grid)) / 2.0
+    per_point = 3.0 * N * N * nb ** 3 * nb  # candidates of an evaluated point
+    full_points = (N + _self_conjugate(cr.grid)) / 2.0
     outs = {}
     with binding.Context.from_crystal(cr) as ctx:
         w, e, v = ctx.modes()
@@ -642,15 +657,20 @@ def measure_workload(binding, wl, budget_slice_s=10.0, full_max_s=300.0, oracle_
             probe = np.zeros(N * nb, np.uint8)
             probe[nb:2 * nb] = 1                                   # q = 1, all branches (also warms the kernel)
             _, st = ctx.rates4(cr.temps, cr.scalebroad, precision=prec, mode_mask=probe, no_graph=1)
-            t_rep = st["ms"] * 1e-3 * nb * 3.0 * N * N * nb ** 3 / st["candidates_executed"]
-            est = t_rep * full_exec / (nb * 3.0 * N * N * nb ** 3)
+            ordered = prec == binding.FP_PREC_MIXED
+
+            def to_grid(st):
+                full, n = ((x if ordered else x * (N - x) / N)
+                           for x in (full_points, st["candidates_executed"] / per_point))
+                return st["ms"] * 1e-3 * full / n
+
+            est = to_grid(st)
             limit = df_full_max_s if (name == "double_float" and df_full_max_s is not None) else full_max_s
             if 0.5 * limit < est < 2.0 * limit:
                 # near the limit: one q is not representative (accepted counts vary over the grid); 16 spread q
                 _, st = ctx.rates4(cr.temps, cr.scalebroad, precision=prec,
                                    mode_mask=_slice_mask(cr, max(1, N // 16), 1), no_graph=1)
-                t_rep = st["ms"] * 1e-3 * nb * 3.0 * N * N * nb ** 3 / st["candidates_executed"]
-                est = t_rep * full_exec / (nb * 3.0 * N * N * nb ** 3)
+                est = to_grid(st)
             smask = np.zeros(N * nb, np.uint8)
             smask[sample] = 1
             if est <= limit:
@@ -660,16 +680,17 @@ def measure_workload(binding, wl, budget_slice_s=10.0, full_max_s=300.0, oracle_
                        "accepted": st["accepted"], "candidates_executed": st["candidates_executed"]}
                 outs[name] = out.reshape(nT, -1)[:, sample]
             else:
-                m = max(2, int(np.ceil(N * t_rep / budget_slice_s)))
+                # q = k mod m is about N / m evaluated points
+                m = max(2, int(np.ceil((2.0 if ordered else 4.0) * est / budget_slice_s)))
                 ext = []
                 for k in (0, m // 3, (2 * m) // 3):
                     _, st = ctx.rates4(cr.temps, cr.scalebroad, precision=prec, mode_mask=_slice_mask(cr, m, k),
                                        no_graph=1)
-                    ext.append(st["ms"] * 1e-3 * full_exec / st["candidates_executed"])
+                    ext.append(to_grid(st))
                 secs = float(np.mean(ext))
                 rec = {"s_per_rate_set": secs, "terms_per_s": cands / secs,
                        "timing": f"extrapolated from three strided q-slices (q = k mod {m}, k = 0, {m // 3}, "
-                                 f"{(2 * m) // 3}) by screened candidates",
+                                 f"{(2 * m) // 3}) by the pairs evaluated",
                        "slice_spread": float((max(ext) - min(ext)) / secs)}
                 out, _ = ctx.rates4(cr.temps, cr.scalebroad, precision=prec, mode_mask=smask, no_graph=1)
                 outs[name] = out.reshape(nT, -1)[:, sample]

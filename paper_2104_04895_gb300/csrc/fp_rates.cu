@@ -490,8 +490,8 @@ int plan_rates(fp_ctx* c, const fp_rates_opts& o, int nT, Selection& sel, size_t
                std::string* err, RateForm form, int split, bool slices) {
   if (nT * (split == 1 ? 2 : 3) > kMaxT) split = 0;
   // Where the pair kernel's tables do not fit, the ordered kernel runs; if neither runs, the first one's reason stands, whose
-  // limits are the wider ones.  The mixed path keeps the ordered kernel: its FP32 vertex rounds
-  // differently for each order of the legs, and exchanging them moved the rates by up to 2e-8 (its error is 5e-8).
+  // limits are the wider ones.  The mixed path keeps to ordered sums (below): its FP32 vertex rounds differently for each
+  // order of the legs, and exchanging them moved the rates by 1e-9 to 8e-8 in the 2-norm, as much as its error.
   std::string why;
   if (form != kOrdered && over_pairs(c, o)) {
     // the FP64 path's contraction in slices: 6 and 12 branches (with 3, K = 6 would leave most of a tile empty)

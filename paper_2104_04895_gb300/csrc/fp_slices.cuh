@@ -5,8 +5,9 @@
 // v = sum_i d_i 512^(5-i), d_i in [-256, 255], |d_0| <= 129.  Each digit is exact in FP16; the product of two digit
 // matrices over K <= 24 and the sum of the up to six products with i + j = s are integers below 2^23, so
 // mma.sync (FP16 operands, FP32 accumulators) forms them exactly: D_s = sum_{i+j=s} A_i B_j.  The levels s = 0..6 are
-// added up in 64-bit integers, sum_s D_s 512^(10-s) / 2^52; the dropped levels are below 2^-6 of the last place.  The
-// result is the product to 2^-53 of the scale, the rounding that FP64 has for its largest elements.
+// added up in 64-bit integers, sum_s D_s 512^(10-s) / 2^52.  The dropped levels are at most 0.09 of the last place with six
+// branches and 0.19 with twelve (every digit at the end of its range), 0.005 and 0.007 rms.  The result is the product to
+// about 2^-53 of the scale, the rounding that FP64 has for its largest elements.
 //
 // A complex product over nb components is a real one over K = 2 nb: row elements (re, im) at K = 2 l, 2 l + 1, and
 // two columns (re, im) per output.  FP64 runs at 2 lane FMAs per clock and SM on this chip, mma.sync at about 950

@@ -402,7 +402,7 @@ __global__ void __launch_bounds__(256) back_kernel(BackArgs a) {
     if (tid < 32) a.gw4[32 * b + tid] = column_sum(a.H3 + 32 * b + tid, kH, a.M, a.dy) + 0.f;
     return;
   }
-  // loss = mean r^2: strided partial sums in FP64, added in thread order; gb4 by the last warp
+  // loss = mean r^2: strided partial sums in FP64, added in thread order; gb4 by the first lane of the second warp
   double s = 0.0;
   for (int i = tid; i < a.M; i += 256) {
     const float r = a.y[i] - a.t[i];

@@ -1,7 +1,7 @@
 // Mixed-precision four-phonon rate kernel: the sums of fp_rates_kernel.cuh (ordered q', k1 <= k2, six candidates per
 // entry, the FP32 form) with every FP32 vertex and weight product formed by the same operations in the same order.  Only dw
 // (one sum of tabulated pairs instead of a chain of three, the last bits of the float that enters the Gaussian) and the
-// order of the compensated sums differ: rates move by at most 1e-12 and 1e-13 in the 2-norm (six crystals and grids up to
+// order of the compensated sums differ: rates move by at most 2e-12, 1e-13 in the 2-norm (six crystals and grids up to
 // 8x8x8, one and eight temperatures).
 //
 // The path is bound by instruction issue; this layout spends fewer instructions per entry (j0, x, y, j3):

@@ -41,10 +41,10 @@
 //
 // Measured (GB300): ordered kernel -> pair kernel -> with slices and the U table of the prologue -> with U over terms and
 // several items per pair on small grids:
-//   diamond 6^3 FP64            578 -> 223 -> 125 -> 119 ms      LiCoO2 5x4x3 FP64, 3 T   386 -> 154 -> 82 -> 76 ms
+//   diamond 6^3 FP64            578 -> 223 -> 125 -> 120 ms      LiCoO2 5x4x3 FP64, 3 T   386 -> 154 -> 82 -> 77 ms
 //   diamond 7x6x5 double-float  262 -> 88 -> 87 -> 91 ms (no slices: 107 ms with them, the FP64 A sums and conversions
 //                               cost more than the FP32 contraction; LiCoO2 4x3x3 24.3 ms either way)
-//   simple cubic 4^3 FP64       2.15 -> 1.49 -> 1.13 -> 0.90 ms (nb = 3: no slices)
+//   simple cubic 4^3 FP64       2.15 -> 1.49 -> 1.13 -> 0.91 ms (nb = 3: no slices)
 // The last double-float step evaluates the accepted terms in FP64 (before, in pairs of floats, whose weights underflowed
 // below about 20 K): 87 -> 91 ms with one temperature, 106 -> 103 with three, 126 -> 119 with eight, LiCoO2 4x3x3 17.2 ->
 // 16.8 and 22.3 -> 20.0 with three.
